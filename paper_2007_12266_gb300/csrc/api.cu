@@ -103,7 +103,7 @@ void free_image(lbpm_ctx* c) {
 
 size_t state_bytes(const lbpm_ctx* c, int q) {
     const size_t e = c->params.precision == LBPM_FP16 ? 2 : 4;
-    return e * static_cast<size_t>(q) * static_cast<size_t>(c->N);
+    return e * static_cast<size_t>(q) * static_cast<size_t>(pitch_of(c->N));
 }
 
 lbpm_status alloc_state(lbpm_ctx* c) {
@@ -111,14 +111,15 @@ lbpm_status alloc_state(lbpm_ctx* c) {
     c->d_f = dalloc(c, state_bytes(c, 19));
     c->d_a = dalloc(c, state_bytes(c, 7));
     c->d_b = dalloc(c, state_bytes(c, 7));
-    c->d_nsum = static_cast<float*>(dalloc(c, sizeof(float) * c->N));
-    c->d_acc = static_cast<unsigned long long*>(dalloc(c, sizeof(unsigned long long) * 2 * c->N));
+    const size_t P = static_cast<size_t>(pitch_of(c->N));
+    c->d_nsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
+    c->d_acc = static_cast<unsigned long long*>(dalloc(c, sizeof(unsigned long long) * 2 * P));
     bool ok = c->d_f && c->d_a && c->d_b && c->d_nsum && c->d_acc;
     if (c->params.precision == LBPM_FP16) {
         // the second phase grid starts as a copy of the first (solids, walls
         // and their periodic mirrors are static and the same in both)
-        c->d_drho = static_cast<float*>(dalloc(c, sizeof(float) * c->N));
-        c->d_rsum = static_cast<float*>(dalloc(c, sizeof(float) * c->N));
+        c->d_drho = static_cast<float*>(dalloc(c, sizeof(float) * P));
+        c->d_rsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
         c->d_phi_alt = static_cast<float*>(dalloc(c, sizeof(float) * c->Vp));
         ok = ok && c->d_drho && c->d_rsum && c->d_phi_alt;
         if (ok && cudaMemcpyAsync(c->d_phi_alt, c->d_phi, sizeof(float) * c->Vp, cudaMemcpyDeviceToDevice,
@@ -164,7 +165,7 @@ lbpm_status build_boundaries(lbpm_ctx* c) {
         }
     }
     if (e == cudaSuccess && !c->d_wall6) {
-        c->d_wall6 = static_cast<unsigned char*>(dalloc(c, c->N));
+        c->d_wall6 = static_cast<unsigned char*>(dalloc(c, pitch_of(c->N)));
         if (!c->d_wall6) e = cudaErrorMemoryAllocation;
     }
     if (e == cudaSuccess) e = launch_wall_mask(c, c->stream);
@@ -339,7 +340,7 @@ bool sum_form_capable(const lbpm_ctx* c) {
 }
 
 cudaError_t clear_sums(const lbpm_ctx* c, int par, cudaStream_t s) {
-    return cudaMemsetAsync(c->d_acc + static_cast<size_t>(par) * static_cast<size_t>(c->N), 0,
+    return cudaMemsetAsync(c->d_acc + static_cast<size_t>(par) * static_cast<size_t>(pitch_of(c->N)), 0,
                            sizeof(unsigned long long) * static_cast<size_t>(c->N), s);
 }
 
@@ -546,7 +547,7 @@ lbpm_status lbpm_load_image(lbpm_ctx* c, const uint16_t* labels, int nx, int ny,
         dfree(c, scan);
         return fail(c, LBPM_E_INVALID, "the image has no pore voxel (label 0)");
     }
-    c->d_site_vox = static_cast<int*>(dalloc(c, sizeof(int) * c->N));
+    c->d_site_vox = static_cast<int*>(dalloc(c, sizeof(int) * pitch_of(c->N)));
     c->d_vsite = static_cast<int*>(dalloc(c, sizeof(int) * c->Vp));
     c->d_phi = static_cast<float*>(dalloc(c, sizeof(float) * c->Vp));
     if (!c->d_site_vox || !c->d_vsite || !c->d_phi) {

@@ -19,6 +19,7 @@ namespace lbm {
 // periodic axis mirrors the opposite face; on a non-periodic axis it is wall.
 struct DomainView {
     int n_sites;        // N: pore sites
+    int pitch;          // P: row length of the per-site arrays, N rounded up (see kPitch)
     int n_halo;         // H: halo voxels that mirror a pore site
     int px, pxpy;       // padded-grid strides in y and z: xi_q is at offset cx + cy px + cz pxpy
     const int* site_vox;   // [N] padded voxel of each site
@@ -36,15 +37,15 @@ struct DomainView {
                            //     next phase pass reads (collision -> phase pass, see StoreF16)
     float* drho;           // [N] rho - 1 of each site at the last even step, fp16 store: the
                            //     reference of the stored momentum deviations
-    void* f;               // [19][N] momentum distributions (AA in place)
-    void* a;               // [7][N]  component A
-    void* b;               // [7][N]  component B
+    void* f;               // [19][P] momentum distributions (AA in place)
+    void* a;               // [7][P]  component A
+    void* b;               // [7][P]  component B
     unsigned long long* acc[2];  // [N] sum form: packed fixed-point (Na, Nb) of each site at the step of
                                  //     parity p, accumulated by the previous collision (see pack_sums)
     float tau_a, tau_b, alpha, beta;
     float fx, fy, fz;
-    float fterm[9];        // 3 t_q xi_q . F of the odd directions q = 2k + 1 (forcing term per pair), in
-                           // the collision's working units (times 2^14 with fp16 storage)
+    float fs[3];           // F / s_m when tau_a == tau_b, in the collision's working units (times 2^14
+                           // with fp16 storage)
     float s_nu, s_m;       // rates when tau_a == tau_b
     int uniform_tau;
 };
@@ -53,6 +54,14 @@ struct DomainView {
 __host__ __device__ __forceinline__ int stencil_off(const DomainView& d, int q) {
     return stencil_offset(q, d.px, d.pxpy);
 }
+
+// Per-site arrays are allocated for N rounded up to a multiple of kPitch
+// entries, which is also the distance between the rows of f, a and b: every row
+// then starts on a 128-byte (fp32; 64-byte, fp16) boundary, so that a warp's
+// accesses to a row at an even step touch no extra sector, and two neighbouring
+// sites can be accessed at once.
+constexpr long long kPitch = 32;
+inline long long pitch_of(long long n) { return (n + kPitch - 1) / kPitch * kPitch; }
 
 struct Allocation {
     void* ptr;

@@ -172,10 +172,10 @@ __global__ void __launch_bounds__(kBlock) k_init(DomainView d, const float* phi0
         d.drho[n] = 0.0f;
         wall = __ldg(d.wall6 + n);
     }
-    const size_t N = d.n_sites;
+    const size_t P = d.pitch;
     static_for<0, Q19>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        S::template st_f<q>(d.f, q * N + n, t19(q));
+        S::template st_f<q>(d.f, q * P + n, t19(q));
         if constexpr (q < Q7) {
             float av = w7(q) * na, bv = w7(q) * nb;
             if constexpr (S::kRef) {
@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(kBlock) k_init(DomainView d, const float* phi0
                 av -= w7(q) * 0.5f * (1.0f + pw);
                 bv -= w7(q) * 0.5f * (1.0f - pw);
             }
-            S::template st_c<q>(d.a, q * N + n, av);
-            S::template st_c<q>(d.b, q * N + n, bv);
+            S::template st_c<q>(d.a, q * P + n, av);
+            S::template st_c<q>(d.b, q * P + n, bv);
         }
     });
 }
@@ -196,6 +196,7 @@ inline unsigned blocks_for(long long n) { return static_cast<unsigned>((n + kBlo
 DomainView make_view(const lbpm_ctx* c) {
     DomainView d{};
     d.n_sites = static_cast<int>(c->N);
+    d.pitch = static_cast<int>(pitch_of(c->N));
     d.n_halo = static_cast<int>(c->H);
     d.px = static_cast<int>(c->px);
     d.pxpy = static_cast<int>(c->px * c->py);
@@ -213,7 +214,7 @@ DomainView make_view(const lbpm_ctx* c) {
     d.a = c->d_a;
     d.b = c->d_b;
     d.acc[0] = c->d_acc;
-    d.acc[1] = c->d_acc ? c->d_acc + c->N : nullptr;
+    d.acc[1] = c->d_acc ? c->d_acc + d.pitch : nullptr;
     const lbpm_params& p = c->params;
     d.tau_a = static_cast<float>(p.tau_a);
     d.tau_b = static_cast<float>(p.tau_b);
@@ -222,15 +223,12 @@ DomainView make_view(const lbpm_ctx* c) {
     d.fx = static_cast<float>(p.force[0]);
     d.fy = static_cast<float>(p.force[1]);
     d.fz = static_cast<float>(p.force[2]);
-    const float K = p.precision == LBPM_FP16 ? StoreF16::kK : StoreF32::kK;
-    for (int k = 0; k < 9; ++k) {
-        const int q = 2 * k + 1;
-        d.fterm[k] = K * (3.0f * t19(q) * (cx(q) * d.fx + cy(q) * d.fy + cz(q) * d.fz));
-    }
     d.uniform_tau = p.tau_a == p.tau_b;
     const float s_nu = 1.0f / static_cast<float>(p.tau_a);
     d.s_nu = s_nu;
     d.s_m = 8.0f * (2.0f - s_nu) / (8.0f - s_nu);
+    const float K = p.precision == LBPM_FP16 ? StoreF16::kK : StoreF32::kK;
+    for (int a = 0; a < 3; ++a) d.fs[a] = static_cast<float>(static_cast<double>(K) * p.force[a] / static_cast<double>(d.s_m));
     return d;
 }
 

@@ -2,7 +2,7 @@
 // single-domain launchers and the batched launcher.
 //
 // State layout (structure of arrays, population-major, in place):
-//   F[q*N + n], A[q*N + n], B[q*N + n]
+//   F[q*P + n], A[q*P + n], B[q*P + n]      (P: N rounded up, DomainView::pitch)
 // AA streaming: at an even step site n reads its own slots F[q][n] and writes
 // the post-collision value of direction q to F[opp(q)][n]. At an odd step it
 // reads direction q from F[opp(q)][m] where m is the upstream neighbour
@@ -17,6 +17,12 @@
 
 namespace lbm {
 
+// explicitly rounded fp32 operations (never contracted)
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
 // ---------------------------------------------------------------------------
 // storage of the distributions
 // ---------------------------------------------------------------------------
@@ -26,14 +32,11 @@ namespace lbm {
 struct StoreF32 {
     using T = float;
     static constexpr bool kRef = false;   // component values stored as they are
-    // Hot-path forms: p points at the slot itself and values are in the
-    // collision's working units, deviations times kK (here 1).
+    // Hot-path forms: p points at the slot itself; the stored number as it
+    // is (see collide_thread).
     static constexpr float kK = 1.0f;
-    template <int Q>
-    static __device__ __forceinline__ float ld_fs(const T* p) { return *p - t19(Q); }
-    template <int Q>
-    static __device__ __forceinline__ void st_fs(T* p, float dev) { *p = t19(Q) + dev; }
-    static __device__ __forceinline__ void st_cs(T* p, float v) { *p = v; }
+    static __device__ __forceinline__ float ld_s(const T* p) { return *p; }
+    static __device__ __forceinline__ void st_s(T* p, float v) { *p = v; }
     template <int Q>
     static __device__ __forceinline__ float ld_fdev(const void* p, size_t i) {
         return static_cast<const float*>(p)[i] - t19(Q);
@@ -101,11 +104,8 @@ struct StoreF16 {
     // the deviations), so the stored number is used as it is and the scale
     // costs no multiplication per value.
     static constexpr float kK = kScale;
-    template <int Q>
-    static __device__ __forceinline__ float ld_fs(const T* p) { return __half2float(*p); }
-    template <int Q>
-    static __device__ __forceinline__ void st_fs(T* p, float v) { *p = __float2half_rn(v); }
-    static __device__ __forceinline__ void st_cs(T* p, float v) { *p = __float2half_rn(v); }
+    static __device__ __forceinline__ float ld_s(const T* p) { return __half2float(*p); }
+    static __device__ __forceinline__ void st_s(T* p, float v) { *p = __float2half_rn(v); }
     template <int Q>
     static __device__ __forceinline__ float ld_fdev(const void* p, size_t i) {
         return __half2float(static_cast<const __half*>(p)[i]) * kInv;
@@ -211,13 +211,13 @@ __device__ __forceinline__ int ldg_keep(const int* p, unsigned long long pol) {
 // ---------------------------------------------------------------------------
 template <int PAR, int Q>
 __device__ __forceinline__ size_t read_slot(const DomainView& d, int n, const int* nb) {
-    const size_t N = static_cast<size_t>(d.n_sites);
+    const size_t P = static_cast<size_t>(d.pitch);
     if constexpr (Q == 0 || PAR == 0) {
-        return static_cast<size_t>(Q) * N + n;
+        return static_cast<size_t>(Q) * P + n;
     } else {
         // upstream site x - xi_Q = x + xi_opp(Q), or -1 (bounce-back)
         const int up = nb[opp(Q)];
-        return up >= 0 ? static_cast<size_t>(opp(Q)) * N + up : static_cast<size_t>(Q) * N + n;
+        return up >= 0 ? static_cast<size_t>(opp(Q)) * P + up : static_cast<size_t>(Q) * P + n;
     }
 }
 
@@ -417,325 +417,76 @@ __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, in
 // opp(q) at n itself when that voxel is solid. With fp16 storage both also
 // use the same density reference (that neighbour's density of the last even
 // step, which odd steps do not change). SlotCache keeps the slot (relative to
-// row q, a signed 32-bit offset) and the reference of each direction between
-// the gather and the scatter, in shared memory laid out [q - 1][thread] so
-// that a warp's accesses fall in distinct banks.
+// row q, a signed 32-bit offset) of each direction and the references' part
+// of each opposite pair between the gather and the scatter, in shared memory
+// laid out [row][site of the block] so that a warp's accesses fall in
+// distinct banks.
 struct SlotCache {
     int* slot;      // entry of direction 1 of this thread; direction q at slot[(q - 1) * stride]
                     // (even steps of the sum form: the face neighbour's site id, -1 if solid)
-    float* ref;     // same layout (fp16 storage only)
+    float* ref;     // pair p (directions 2p + 1, 2p + 2) at ref[p * stride] (fp16 storage only)
     int stride;     // threads per block
 };
 
-// Incoming distributions of site n (voxel v), as deviations d_q = f_q - t_q
-// from the rest state (exact in fp32 near rest), so that density and
-// momentum are sums of small numbers and the relaxation acts on small
-// quantities; in working units, i.e. times S::kK. Odd steps also fill the
-// slot cache.
-template <int PAR, class S>
-__device__ __forceinline__ void load_f(const DomainView& d, int n, int v, float (&f)[Q19], SlotCache sc) {
-    const int Ni = d.n_sites;
-    const size_t N = static_cast<size_t>(Ni);
-    const typename S::T* const F = static_cast<const typename S::T*>(d.f);
-    constexpr float K = S::kK;
+// Collision, recoloring and streaming of site n. The arithmetic is written in
+// explicitly rounded operations (no contraction is left to the compiler), so a
+// site's result is the same bit for bit in every kernel this is compiled into.
+//
+// What bounds it: the loads in flight. The kernel is latency-bound at 36
+// resident warps per SM, so the arithmetic is arranged for few instructions
+// (sums and differences over opposite pairs shared by the moments, the
+// equilibrium and the relaxation; the interfacial terms in closed form per
+// direction): 617 (even) and 816 (odd) instructions per site against 726 and
+// 890 in the form that evaluated each direction's terms by itself, 161.2
+// against 165.7 us per step on 3.69 M sites of a 256^3 pack (fp32), 11.3
+// against 11.9 us on 255 k sites. Two sites per thread on fma.rn.f32x2 took 463
+// instructions per site but ran slower (171-177 us): twice the registers left
+// fewer warps to cover the latency.
+template <int PAR, class S, int CF>
+__device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotCache sc) {
+    using T = typename S::T;
+    constexpr float K = S::kK;                      // working units: deviations times K
+    constexpr float iK = 1.0f / K;
+    const size_t P = static_cast<size_t>(d.pitch);
+    T* const F = static_cast<T*>(d.f);
+    const unsigned long long pol = l2_keep();
+    const int v = CF != 0 ? ldg_keep(d.site_vox + n, pol) : __ldg(d.site_vox + n);
+
+    // incoming momentum populations, the stored numbers s_q as they are:
+    // fp32: f_q; fp16: f_q - t_q rho_ref, in units of 1 / K
+    float f[Q19];
+    float ref_own = 0.0f;                                     // fp16: K times the reference density of the own slots
+    float ref_sum[9];                                    // fp16, odd steps: K t (ref_q + ref_o) of each pair
     if constexpr (PAR == 0) {
-        // even step: own slots, row q; fp16 references are all this site's
-        float r = 0.0f;
-        if constexpr (S::kRef) r = d.drho[n];
+        if constexpr (S::kRef) ref_own = d.drho[n];
         static_for<0, Q19>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
-            f[q] = S::template ld_fs<q>(F + q * N + n);
-            if constexpr (S::kRef) f[q] = fmaf(t19(q) * K, r, f[q]);
+            f[q] = S::ld_s(F + q * P + n);
         });
     } else {
-        f[0] = S::template ld_fs<0>(F + n);
-        if constexpr (S::kRef) f[0] = fmaf(t19(0) * K, d.drho[n], f[0]);
-        static_for<1, Q19>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;   // direction of the downstream slot
-            constexpr int o = opp(q);                // direction read from it
-            const int m = __ldg(d.vsite + v + stencil_off(d, q));
-            const int s = m >= 0 ? m : n + (o - q) * Ni;
-            sc.slot[(q - 1) * sc.stride] = s;
-            f[o] = S::template ld_fs<o>(F + q * N + s);
+        f[0] = S::ld_s(F + n);
+        if constexpr (S::kRef) ref_own = d.drho[n];
+        static_for<0, 9>([&](auto pc) {
+            constexpr int p = decltype(pc)::value;
+            float r[2];
+            static_for<0, 2>([&](auto hc) {
+                constexpr int h = decltype(hc)::value;
+                constexpr int q = 2 * p + 1 + h;     // direction of the downstream slot
+                constexpr int o = opp(q);            // direction read from it
+                const int m = __ldg(d.vsite + v + stencil_off(d, q));
+                const int s = m >= 0 ? m : n + (o - q) * d.pitch;
+                sc.slot[(q - 1) * sc.stride] = s;
+                f[o] = S::ld_s(F + q * P + s);
+                if constexpr (S::kRef) r[h] = d.drho[m >= 0 ? m : n];
+            });
             if constexpr (S::kRef) {
-                const float r = d.drho[m >= 0 ? m : n];
-                sc.ref[(q - 1) * sc.stride] = r;
-                f[o] = fmaf(t19(o) * K, r, f[o]);
+                // reference of the slot of direction o minus that of direction q, o = q + 1
+                constexpr float tk = t19(2 * p + 1) * K;
+                ref_sum[p] = mul(tk, add(r[0], r[1]));
+                sc.ref[p * sc.stride] = mul(tk, sub(r[1], r[0]));
             }
         });
     }
-}
-
-
-// colour gradient C = sum_q g_q xi_q phi(x + xi_q); phi_at(q) gives the
-// neighbour's phase (solids hold phi_s)
-template <class PhiAt>
-__device__ __forceinline__ void color_gradient(PhiAt&& phi_at, float& Cx, float& Cy, float& Cz) {
-    Cx = 0.0f;
-    Cy = 0.0f;
-    Cz = 0.0f;
-    static_for<1, Q19>([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        constexpr float g = grad_w(q);
-        const float p = phi_at(qc);
-        if constexpr (cx(q) != 0) Cx = fmaf(g * cx(q), p, Cx);
-        if constexpr (cy(q) != 0) Cy = fmaf(g * cy(q), p, Cy);
-        if constexpr (cz(q) != 0) Cz = fmaf(g * cz(q), p, Cz);
-    });
-}
-
-// macroscopic moments: drho = rho - 1 and j from the deviations
-struct Moments {
-    float drho, jx, jy, jz;
-};
-__device__ __forceinline__ Moments moments(const float (&f)[Q19]) {
-    Moments m{0.0f, 0.0f, 0.0f, 0.0f};
-    static_for<0, Q19>([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        m.drho += f[q];
-        if constexpr (cx(q) > 0) m.jx += f[q];
-        if constexpr (cx(q) < 0) m.jx -= f[q];
-        if constexpr (cy(q) > 0) m.jy += f[q];
-        if constexpr (cy(q) < 0) m.jy -= f[q];
-        if constexpr (cz(q) > 0) m.jz += f[q];
-        if constexpr (cz(q) < 0) m.jz -= f[q];
-    });
-    return m;
-}
-
-// Collision, recoloring and streaming of site n, given its incoming
-// deviations f and their moments, its phase phi_c, Na, Nb and the colour
-// gradient.
-// Nt: Na + Nb from the phase pass (Na = Nt (1 + phi_c)/2, Nb = Nt (1 - phi_c)/2).
-// a_own, b_own (CF == 2): the site's component sums in fixed point.
-template <int PAR, class S, int CF = 0>
-__device__ __forceinline__ void collide_site(const DomainView& d, int n, const float (&f)[Q19], Moments mo,
-                                             float phi_c, float Nt, int a_own, int b_own, float Cx, float Cy,
-                                             float Cz, SlotCache sc) {
-    using T = typename S::T;
-    const size_t N = static_cast<size_t>(d.n_sites);
-    T* const F = static_cast<T*>(d.f);
-    // f, drho and j are in working units (times K); the equilibrium's
-    // quadratic terms take one factor 1/K, the interfacial terms and the
-    // forcing (d.fterm is stored in working units) one factor K
-    constexpr float K = S::kK;
-    constexpr float iK = 1.0f / K;
-    const float drho = mo.drho, jx = mo.jx, jy = mo.jy, jz = mo.jz;
-
-    const float C2 = Cx * Cx + Cy * Cy + Cz * Cz;
-    float nx = 0.0f, ny = 0.0f, nz = 0.0f, Cmag = 0.0f;
-    if (C2 > 0.0f) {
-        const float inv = rsqrtf(C2);
-        Cmag = C2 * inv;
-        nx = Cx * inv;
-        ny = Cy * inv;
-        nz = Cz * inv;
-    }
-
-    // relaxation rates from the viscosity (tau mixed linearly in phi)
-    float s_nu = d.s_nu, s_m = d.s_m;
-    if (!d.uniform_tau) {
-        const float tau = d.tau_b + (d.tau_a - d.tau_b) * 0.5f * (1.0f + phi_c);
-        s_nu = 1.0f / tau;
-        s_m = 8.0f * (2.0f - s_nu) / (8.0f - s_nu);
-    }
-
-    // MRT collision, evaluated in its equivalent two-relaxation-time form.
-    // With S from the viscosity, every non-conserved even moment (m1, m2,
-    // m9..m15) relaxes with s_nu and every non-conserved odd moment (m4, m6,
-    // m8, m16..m18) with s_m; the conserved ones equal their equilibria. So
-    //   f* = f - s_nu (f+ - feq+) - s_m (f- - feq-) + 3 t_q xi_q . F
-    // with f+- the even/odd parts over opposite pairs and feq the velocity-
-    // space equilibrium whose moments are m^eq:
-    //   feq+ = t_q (rho + 4.5 (xi.j)^2 - 1.5 j.j) + M^-1 dm_alpha
-    //   feq- = 3 t_q xi.j
-    // where dm_alpha holds the interfacial-tension terms of m1, m9, m11,
-    // m13, m14, m15 (rho0 = 1). Everything below is relative to the rest
-    // state t_q (rho = 1), i.e. in deviations.
-    const float jj = jx * jx + jy * jy + jz * jz;
-    const float ac = (d.alpha * K) * Cmag;
-    const float hac = 0.5f * ac;
-    float dma[Q19];
-    dma[1] = -ac;
-    dma[9] = hac * (2.0f * nx * nx - ny * ny - nz * nz);
-    dma[11] = hac * (ny * ny - nz * nz);
-    dma[13] = hac * nx * ny;
-    dma[14] = hac * ny * nz;
-    dma[15] = hac * nx * nz;
-    const float drho_iso = fmaf(-1.5f * iK, jj, drho);
-
-    // recoloring weights Nb/N and Na/N are (1 - phi)/2 and (1 + phi)/2
-    const float bxa = d.beta * 0.5f * (1.0f - phi_c);
-    const float bxb = d.beta * 0.5f * (1.0f + phi_c);
-
-    // destination of direction q (q >= 1): row opp(q) at n (even step) or
-    // the cached slot of row q (odd step)
-    auto dst = [&](auto qc, auto* base) {
-        constexpr int q = decltype(qc)::value;
-        if constexpr (PAR == 0) return base + opp(q) * N + n;
-        else return base + q * N + sc.slot[(q - 1) * sc.stride];
-    };
-
-    // The increments of the moving populations sum to minus the rest
-    // increment in exact arithmetic; taking the rest increment as that sum
-    // keeps fp32 mass exact up to unbiased rounding.
-    float dsum = 0.0f;
-    static_for<0, 9>([&](auto pc) {
-        constexpr int q = 2 * decltype(pc)::value + 1;   // q odd, opp(q) = q + 1
-        constexpr int o = q + 1;
-        constexpr float t = t19(q);
-        float cu = 0.0f;
-        if constexpr (cx(q) != 0) cu += cx(q) * jx;
-        if constexpr (cy(q) != 0) cu += cy(q) * jy;
-        if constexpr (cz(q) != 0) cu += cz(q) * jz;
-        float eqp = t * fmaf((4.5f * iK) * cu, cu, drho_iso);
-        static_for<1, 16>([&](auto kc) {
-            constexpr int k = decltype(kc)::value;
-            if constexpr (k == 1 || k == 9 || k == 11 || k == 13 || k == 14 || k == 15) {
-                if constexpr (mrow(k, q) != 0) eqp = fmaf(minv(q, k), dma[k], eqp);
-            }
-        });
-        const float eqm = 3.0f * t * cu;
-        const float fp = 0.5f * (f[q] + f[o]);
-        const float fm = 0.5f * (f[q] - f[o]);
-        const float dp = -s_nu * (fp - eqp);
-        const float dmi = fmaf(-s_m, fm - eqm, d.fterm[q >> 1]);
-        const float inc_q = dp + dmi, inc_o = dp - dmi;
-        dsum += inc_q + inc_o;
-        float vq = f[q] + inc_q, vo = f[o] + inc_o;
-        if constexpr (S::kRef) {
-            // even step: relative to this site's rest state t_q rho; odd step:
-            // relative to the destination's density of the last even step
-            if constexpr (PAR == 0) {
-                vq = fmaf(-t, drho, vq);
-                vo = fmaf(-t, drho, vo);
-            } else {
-                vq = fmaf(-t * K, sc.ref[(q - 1) * sc.stride], vq);
-                vo = fmaf(-t * K, sc.ref[(o - 1) * sc.stride], vo);
-            }
-        }
-        S::template st_fs<q>(dst(std::integral_constant<int, q>{}, F), vq);
-        S::template st_fs<o>(dst(std::integral_constant<int, o>{}, F), vo);
-    });
-    if constexpr (S::kRef) {
-        if constexpr (PAR == 0) {
-            S::template st_fs<0>(F + n, fmaf(-t19(0), drho, f[0] - dsum));
-            d.drho[n] = drho * iK;
-        } else {
-            S::template st_fs<0>(F + n, fmaf(-t19(0) * K, d.drho[n], f[0] - dsum));
-        }
-    } else {
-        S::template st_fs<0>(F + n, f[0] - dsum);
-    }
-
-    // recolored component distributions (Eqs. LBE-mass-a/b), streamed on the
-    // fly; the rest populations take the remainder of Na and Nb so that the
-    // fp32 weights (whose sum is not exactly 1) create no mass. With fp16
-    // storage the stored quantity is the deviation from w_q (1 +- phi_c)/2: the
-    // deviation from w_q Na (w_q Nb), which the formula gives directly as
-    // w_q Na (4.5 u.xi + beta Nb/N n.xi), plus w_q times
-    //   Na - (1 + phi_c)/2 = (N - 1)(1 + phi_c)/2   (likewise for Nb).
-    // (working units: Na, Nb times K, j divided by K back to u)
-    const float NaK = (0.5f * K) * Nt * (1.0f + phi_c), NbK = (0.5f * K) * Nt * (1.0f - phi_c);
-    if constexpr (CF != 0) {
-        // Sum form: A*_q = w_q Na [1 + 4.5 u.xi_q + beta (Nb/N) n.xi_q] (likewise B*_q)
-        // in fixed point, added into the sums of the site that receives it; the
-        // rest value takes the remainder of the site's own Na (Nb), so the seven
-        // values add up to it exactly.
-        constexpr float kFix = kSumOne / K;   // working units -> fixed point
-        int ra = a_own, rb = b_own;
-        if constexpr (CF == 1) {
-            ra = __float2int_rn(NaK * kFix);
-            rb = __float2int_rn(NbK * kFix);
-        }
-        unsigned long long* const acc = d.acc[PAR ^ 1];
-        const unsigned long long pol = l2_keep();
-        static_for<1, Q7>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;
-            float ux = 0.0f, nn = 0.0f;
-            if constexpr (cx(q) != 0) { ux = cx(q) * jx; nn = cx(q) * nx; }
-            if constexpr (cy(q) != 0) { ux = cy(q) * jy; nn = cy(q) * ny; }
-            if constexpr (cz(q) != 0) { ux = cz(q) * jz; nn = cz(q) * nz; }
-            const float base = fmaf(4.5f * iK, ux, 1.0f);
-            const int ia = __float2int_rn(w7(q) * NaK * (base + bxa * nn) * kFix);
-            const int ib = __float2int_rn(w7(q) * NbK * (base - bxb * nn) * kFix);
-            ra -= ia;
-            rb -= ib;
-            // receiver: x + xi_q if it is a pore site, else x itself (bounce-back)
-            int m;
-            if constexpr (PAR == 0) {
-                m = sc.slot[(q - 1) * sc.stride];
-            } else {
-                const int sl = sc.slot[(q - 1) * sc.stride];
-                m = static_cast<unsigned>(sl) < static_cast<unsigned>(d.n_sites) ? sl : -1;
-            }
-            if (m >= 0) {
-                red_add(acc + m, pack_sums(ia, ib), pol);
-            } else {
-                ra += ia;
-                rb += ib;
-            }
-        });
-        red_add(acc + n, pack_sums(ra, rb), pol);
-        // this step's sums of the site are consumed (the phase pass before this
-        // collision was their last other reader): they receive the step after next
-        st_keep(d.acc[PAR] + n, 0ull, pol);
-        return;
-    }
-    T* const A = static_cast<T*>(d.a);
-    T* const B = static_cast<T*>(d.b);
-    // fp16 only: K (N - 1)(1 +- phi_c)/2, the offsets of the references
-    const float hN = (0.5f * K) * (Nt - 1.0f);
-    const float eA = hN * (1.0f + phi_c), eB = hN * (1.0f - phi_c);
-    float asum = 0.0f, bsum = 0.0f;
-    static_for<1, Q7>([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        float ux = 0.0f, nn = 0.0f;
-        if constexpr (cx(q) != 0) { ux = cx(q) * jx; nn = cx(q) * nx; }
-        if constexpr (cy(q) != 0) { ux = cy(q) * jy; nn = cy(q) * ny; }
-        if constexpr (cz(q) != 0) { ux = cz(q) * jz; nn = cz(q) * nz; }
-        float av, bv;
-        if constexpr (S::kRef) {
-            const float du = (4.5f * iK) * ux;
-            av = w7(q) * NaK * (du + bxa * nn);
-            bv = w7(q) * NbK * (du - bxb * nn);
-            asum += av;
-            bsum += bv;
-            av = fmaf(w7(q), eA, av);
-            bv = fmaf(w7(q), eB, bv);
-        } else {
-            const float base = fmaf(4.5f * iK, ux, 1.0f);
-            av = w7(q) * NaK * (base + bxa * nn);
-            bv = w7(q) * NbK * (base - bxb * nn);
-            asum += av;
-            bsum += bv;
-        }
-        S::st_cs(dst(qc, A), av);
-        S::st_cs(dst(qc, B), bv);
-    });
-    if constexpr (S::kRef) {
-        // The phase pass adds (1 + S)/2 to the seven values a site reads, S
-        // holding w_q phi_c for this site's value of direction q; the seven
-        // stored values above sum to Wsum (Na - (1 + phi_c)/2) with Wsum the
-        // fp32 weights' sum 1 + 2^-26. The rest value takes the difference,
-        // K (1 - Wsum)(Na - 1/2), so that its readers rebuild exactly Na (and
-        // Nb) and the fp32 weights create no mass.
-        constexpr double kWsum = static_cast<double>(w7(0)) + 6.0 * static_cast<double>(w7(1));
-        constexpr float kWerr = static_cast<float>(1.0 - kWsum);
-        S::st_cs(A + n, fmaf(kWerr, fmaf(-0.5f, K, NaK), fmaf(w7(0), eA, -asum)));
-        S::st_cs(B + n, fmaf(kWerr, fmaf(-0.5f, K, NbK), fmaf(w7(0), eB, -bsum)));
-    } else {
-        S::st_cs(A + n, NaK - asum);
-        S::st_cs(B + n, NbK - bsum);
-    }
-}
-
-// One site per thread, direct loads.
-template <int PAR, class S, int CF = 0>
-__device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotCache sc) {
-    const int v = CF != 0 ? ldg_keep(d.site_vox + n, l2_keep()) : __ldg(d.site_vox + n);
-    float f[Q19];
-    load_f<PAR, S>(d, n, v, f, sc);
     if constexpr (CF != 0 && PAR == 0) {
         // sum form, even step: the face neighbours that receive the component values
         static_for<1, Q7>([&](auto qc) {
@@ -745,8 +496,8 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     }
     // sum form from the sums: the site's own Na, Nb (complete before the
     // previous phase pass, like f)
-    int a_own = 0, b_own = 0;
-    if constexpr (CF == 2) unpack_sums(ld_keep(d.acc[PAR] + n, l2_keep()), a_own, b_own);
+    unsigned long long own = 0;
+    if constexpr (CF == 2) own = ld_keep(d.acc[PAR] + n, pol);
 
     // Everything above (site and neighbour ids, f and the sums from the
     // previous collision) is safe to read before the phase pass of this step
@@ -755,16 +506,24 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     allow_next_grid();
     wait_prior_grid();
 
-    const float* pv = d.phi[PAR] + v;
-    float phi_c, Nt;
+    // colour gradient C = sum_q g_q xi_q phi(x + xi_q) (solids hold phi_s),
+    // g = 1 on faces and 1/2 on edges, from the differences over opposite
+    // neighbours; twice C is what is used below (n does not depend on the scale)
+    const float* const pv = d.phi[PAR] + v;
+    float dphi[9];
+    static_for<0, 9>([&](auto pc) {
+        constexpr int p = decltype(pc)::value;
+        dphi[p] = sub(pv[stencil_off(d, 2 * p + 1)], pv[stencil_off(d, 2 * p + 2)]);
+    });
+    const float phi_c = *pv;
+    float Nt;
     if constexpr (CF == 2) {
-        sums_phase(a_own, b_own, Nt, phi_c);
+        int a, b;
+        unpack_sums(own, a, b);
+        Nt = mul(add(static_cast<float>(a), static_cast<float>(b)), kSumInv);
     } else {
-        phi_c = *pv;
         Nt = d.nsum[n];
     }
-    float Cx, Cy, Cz;
-    color_gradient([&](auto qc) { return pv[stencil_off(d, decltype(qc)::value)]; }, Cx, Cy, Cz);
     if constexpr (S::kRef && CF == 0) {
         // references of the values the next phase pass reads at this site: the
         // phase of x - xi_q, which this step writes, or this site's own on a
@@ -777,7 +536,269 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
         });
         d.rsum[n] = fmaf(w7(1), Sf, w7(0) * phi_c);
     }
-    collide_site<PAR, S, CF>(d, n, f, moments(f), phi_c, Nt, a_own, b_own, Cx, Cy, Cz, sc);
+
+    // pair sums of deviations S = (f_q - t) + (f_o - t) and differences
+    // D = f_q - f_o (both exact or once rounded: f_q - 2t is exact for f near
+    // t)
+    const float mt[2] = {-2.0f * t19(1), -2.0f * t19(7)};
+    float two_ref[2];
+    if constexpr (S::kRef && PAR == 0) {
+        two_ref[0] = mul(2.0f * t19(1) * K, ref_own);
+        two_ref[1] = mul(2.0f * t19(7) * K, ref_own);
+    }
+    auto pair_sum = [&](auto pc) {
+        constexpr int p = decltype(pc)::value;
+        constexpr int q = 2 * p + 1, o = q + 1, c = p < 3 ? 0 : 1;
+        if constexpr (!S::kRef) return add(add(f[q], mt[c]), f[o]);
+        else if constexpr (PAR == 0) return add(add(f[q], f[o]), two_ref[c]);
+        else return add(add(f[q], f[o]), ref_sum[p]);
+    };
+    // fp16, odd steps: difference of the references, for D and the results
+    auto pair_ref = [&](auto pc) { return sc.ref[decltype(pc)::value * sc.stride]; };
+    auto pair_diff = [&](auto pc) {
+        constexpr int q = 2 * decltype(pc)::value + 1;
+        if constexpr (S::kRef && PAR == 1) return add(sub(f[q], f[q + 1]), pair_ref(pc));
+        else return sub(f[q], f[q + 1]);
+    };
+    // drho = rho - 1 and j, in working units
+    float drho, jx, jy, jz;
+    {
+        if constexpr (!S::kRef) drho = add(f[0], -t19(0));
+        else drho = fma(t19(0) * K, ref_own, f[0]);
+        float s = pair_sum(std::integral_constant<int, 0>{});
+        static_for<1, 9>([&](auto pc) { s = add(s, pair_sum(pc)); });
+        drho = add(drho, s);
+        float D[9];
+        static_for<0, 9>([&](auto pc) { D[decltype(pc)::value] = pair_diff(pc); });
+        // pairs: x, y, z; (++), (+-) of xy, xz, yz
+        jx = add(add(add(D[3], D[4]), add(D[5], D[6])), D[0]);
+        jy = add(add(sub(D[3], D[4]), add(D[7], D[8])), D[1]);
+        jz = add(add(sub(D[5], D[6]), sub(D[7], D[8])), D[2]);
+    }
+    // From here on the compiler knows nothing about the populations: it derives
+    // S and D again below instead of keeping all of them in registers.
+    static_for<1, Q19>([&](auto qc) { asm volatile("" : "+f"(f[decltype(qc)::value])); });
+
+    // 2 C, its inverse length (0 where C vanishes) and the normal n
+    const float Cx = add(add(dphi[0], dphi[0]), add(add(dphi[3], dphi[4]), add(dphi[5], dphi[6])));
+    const float Cy = add(add(dphi[1], dphi[1]), add(sub(dphi[3], dphi[4]), add(dphi[7], dphi[8])));
+    const float Cz = add(add(dphi[2], dphi[2]), add(sub(dphi[5], dphi[6]), sub(dphi[7], dphi[8])));
+    const float C2 = fma(Cx, Cx, fma(Cy, Cy, mul(Cz, Cz)));
+    const float inv = C2 > 0.0f ? rsqrtf(C2) : 0.0f;
+
+    // relaxation rates from the viscosity (tau mixed linearly in phi): half of
+    // s_nu, -s_m / 2, s_m / 12, and the force (times K) over s_m
+    float h_nu, h_m, b_m, gx, gy, gz;
+    if (d.uniform_tau) {
+        h_nu = 0.5f * d.s_nu;
+        h_m = -0.5f * d.s_m;
+        b_m = d.s_m * (1.0f / 12.0f);
+        gx = d.fs[0];
+        gy = d.fs[1];
+        gz = d.fs[2];
+    } else {
+        const float tau = fma(mul(d.tau_a - d.tau_b, 0.5f), add(1.0f, phi_c), d.tau_b);
+        const float s_nu = __fdiv_rn(1.0f, tau);
+        const float s_m = __fdiv_rn(mul(8.0f, sub(2.0f, s_nu)), sub(8.0f, s_nu));
+        h_nu = mul(0.5f, s_nu);
+        h_m = mul(-0.5f, s_m);
+        b_m = mul(s_m, 1.0f / 12.0f);
+        const float g = mul(K, __fdiv_rn(1.0f, s_m));
+        gx = mul(g, d.fx);
+        gy = mul(g, d.fy);
+        gz = mul(g, d.fz);
+    }
+
+    // MRT collision, evaluated in its equivalent two-relaxation-time form.
+    // With S from the viscosity, every non-conserved even moment (m1, m2,
+    // m9..m15) relaxes with s_nu and every non-conserved odd moment (m4, m6,
+    // m8, m16..m18) with s_m; the conserved ones equal their equilibria. So
+    //   f* = f - s_nu (f+ - feq+) - s_m (f- - feq-) + 3 t_q xi_q . F
+    // with f+- the even/odd parts over opposite pairs and feq the velocity-
+    // space equilibrium whose moments are m^eq:
+    //   feq+ = t_q (rho + 4.5 (xi.j)^2 - 1.5 j.j) + M^-1 dm_alpha
+    //   feq- = 3 t_q xi.j
+    // where dm_alpha holds the interfacial-tension terms of m1, m9, m11,
+    // m13, m14, m15 (rho0 = 1). With E_ij = alpha |C| n_i n_j (whose trace is
+    // alpha |C|) the rows of M^-1 combine to
+    //   faces  (11/2394 - 1/36) alpha|C| + E_ii / 12
+    //   edges  (-8/2394 - 1/18) alpha|C| + (E_ii + E_jj) / 12 +- E_ij / 8
+    // and with q_i = j_i^2 / 4, G_i = q_i + E_ii / 6, H_ij = j_i j_j / 2 + E_ij / 4
+    //   faces  2 feq+ = bF + q_i + G_i
+    //   edges  2 feq+ = bE + G_i + G_j +- H_ij
+    // bF, bE holding rho - 1 - 1.5 j.j and the alpha |C| parts. The relaxation
+    // is h_nu (2 feq+ - S) on both populations of a pair and
+    // +-(-s_m/2 D + s_m/12 {2, 1} xi.(j + F/s_m)) on each, F/s_m bringing in
+    // the force. Everything is relative to the rest state (rho = 1), in
+    // working units: q_i and j_i j_j / 2 take one factor 1/K (as 2^-7 on each
+    // j with fp16 storage), alpha one factor K (ga below: alpha K / (12 |2C|)).
+    constexpr float kHalf = S::kRef ? 0.5f / 128.0f : 0.5f;   // 0.5 / sqrt(K)
+    const float px = mul(kHalf, jx), py = mul(kHalf, jy), pz = mul(kHalf, jz);
+    const float ga = mul(d.alpha * (K / 12.0f), inv);
+    const float ax = mul(ga, Cx), ay = mul(ga, Cy), az = mul(ga, Cz);
+    const float qx = mul(px, px), qy = mul(py, py), qz = mul(pz, pz);
+    const float Gx = fma(ax, Cx, qx), Gy = fma(ay, Cy, qy), Gz = fma(az, Cz, qz);
+    const float ac = mul(ga, C2);                                // alpha |C| K / 6
+    const float i9 = mul(1.0f / 9.0f, fma(-6.0f, add(add(qx, qy), qz), drho));
+    constexpr float kF = static_cast<float>(12.0 * (11.0 / 2394.0 - 1.0 / 36.0));
+    constexpr float kE = static_cast<float>(12.0 * (-8.0 / 2394.0 - 1.0 / 18.0));
+    const float bF = fma(kF, ac, i9);
+    const float bE = fma(kE, ac, mul(0.5f, i9));
+    const float Hxy = fma(add(px, px), py, mul(mul(1.5f, ax), Cy));
+    const float Hxz = fma(add(px, px), pz, mul(mul(1.5f, ax), Cz));
+    const float Hyz = fma(add(py, py), pz, mul(mul(1.5f, ay), Cz));
+    const float Ux = mul(b_m, add(jx, gx)), Uy = mul(b_m, add(jy, gy)), Uz = mul(b_m, add(jz, gz));
+
+    // destination of direction q (q >= 1): row opp(q) at n (even step) or the
+    // cached slot of row q (odd step)
+    auto store = [&](auto qc, T* base, float x) {
+        constexpr int q = decltype(qc)::value;
+        if constexpr (PAR == 0) S::st_s(base + opp(q) * P + n, x);
+        else S::st_s(base + q * P + sc.slot[(q - 1) * sc.stride], x);
+    };
+
+    // fp16, even steps: the results are relative to this site's new density
+    // instead of the old reference
+    float moved[2] = {0.0f, 0.0f}, rref = 0.0f;
+    if constexpr (S::kRef && PAR == 0) {
+        rref = sub(mul(K, ref_own), drho);
+        moved[0] = mul(t19(1), rref);
+        moved[1] = mul(t19(7), rref);
+    }
+    // The even increments of the moving populations sum to minus the rest
+    // increment in exact arithmetic; taking the rest increment as that sum
+    // keeps fp32 mass exact up to unbiased rounding.
+    float esum;
+    static_for<0, 9>([&](auto pc) {
+        constexpr int p = decltype(pc)::value;
+        constexpr int q = 2 * p + 1, o = q + 1, c = p < 3 ? 0 : 1;
+        float e, u;
+        if constexpr (p == 0) { e = add(bF, add(qx, Gx)); u = add(Ux, Ux); }
+        if constexpr (p == 1) { e = add(bF, add(qy, Gy)); u = add(Uy, Uy); }
+        if constexpr (p == 2) { e = add(bF, add(qz, Gz)); u = add(Uz, Uz); }
+        if constexpr (p == 3) { e = add(add(bE, add(Gx, Gy)), Hxy); u = add(Ux, Uy); }
+        if constexpr (p == 4) { e = sub(add(bE, add(Gx, Gy)), Hxy); u = sub(Ux, Uy); }
+        if constexpr (p == 5) { e = add(add(bE, add(Gx, Gz)), Hxz); u = add(Ux, Uz); }
+        if constexpr (p == 6) { e = sub(add(bE, add(Gx, Gz)), Hxz); u = sub(Ux, Uz); }
+        if constexpr (p == 7) { e = add(add(bE, add(Gy, Gz)), Hyz); u = add(Uy, Uz); }
+        if constexpr (p == 8) { e = sub(add(bE, add(Gy, Gz)), Hyz); u = sub(Uy, Uz); }
+        e = sub(e, pair_sum(pc));
+        if constexpr (p == 0) esum = e;
+        else esum = add(esum, e);
+        float even, odd = fma(h_m, pair_diff(pc), u);
+        if constexpr (S::kRef && PAR == 0) even = fma(h_nu, e, moved[c]);
+        else even = mul(h_nu, e);
+        if constexpr (S::kRef && PAR == 1) odd = add(odd, pair_ref(pc));
+        store(std::integral_constant<int, q>{}, F, add(f[q], add(even, odd)));
+        store(std::integral_constant<int, o>{}, F, add(f[o], sub(even, odd)));
+    });
+    {
+        const float m2 = mul(-2.0f, h_nu);
+        float r0 = fma(m2, esum, f[0]);
+        if constexpr (S::kRef && PAR == 0) {
+            r0 = fma(t19(0), rref, r0);
+            d.drho[n] = mul(iK, drho);
+        }
+        S::st_s(F + n, r0);
+    }
+
+    // recolored component distributions (Eqs. LBE-mass-a/b), streamed on the
+    // fly; the rest populations take the remainder of Na and Nb so that the
+    // fp32 weights (whose sum is not exactly 1) create no mass. Over a pair of
+    // opposite directions the values are P +- P (4.5 u_i + beta Nb/N n_i) with
+    // P = w_q Na (likewise B, with the normal's sign turned); the recoloring
+    // weights Nb/N and Na/N are (1 - phi)/2 and (1 + phi)/2.
+    const float nx = mul(Cx, inv), ny = mul(Cy, inv), nz = mul(Cz, inv);
+    const float c45 = 4.5f * iK, one = 1.0f;
+    const float wx = mul(c45, jx), wy = mul(c45, jy), wz = mul(c45, jz);
+    const float pa1 = add(one, phi_c), pb1 = sub(one, phi_c);   // 1 + phi, 1 - phi
+    const float bxa = mul(0.5f * d.beta, pb1), bxb = mul(-0.5f * d.beta, pa1);
+    const float rA[3] = {fma(bxa, nx, wx), fma(bxa, ny, wy), fma(bxa, nz, wz)};
+    const float rB[3] = {fma(bxb, nx, wx), fma(bxb, ny, wy), fma(bxb, nz, wz)};
+    if constexpr (CF != 0) {
+        // Sum form: the values in fixed point, added into the sums of the site
+        // that receives them; what stays (the rest value, and the values of
+        // bounce-back links) is the remainder of the site's own Na (Nb), so all
+        // seven add up to it exactly.
+        if constexpr (CF == 1) {
+            const float half = mul(0.5f * kSumOne, Nt);
+            own = pack_sums(__float2int_rn(mul(half, pa1)), __float2int_rn(mul(half, pb1)));
+        }
+        unsigned long long* const acc = d.acc[PAR ^ 1];
+        const float wN = mul(w7(1) * 0.5f * kSumOne, Nt);
+        const float PA = mul(wN, pa1), PB = mul(wN, pb1);
+        static_for<0, 3>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            const float dA = mul(PA, rA[i]), dB = mul(PB, rB[i]);
+            static_for<0, 2>([&](auto hc) {
+                constexpr int q = 2 * i + 1 + decltype(hc)::value;
+                const unsigned long long x = pack_sums(__float2int_rn(q & 1 ? add(PA, dA) : sub(PA, dA)),
+                                                       __float2int_rn(q & 1 ? add(PB, dB) : sub(PB, dB)));
+                // receiver: x + xi_q if it is a pore site, else x itself (bounce-back)
+                const int m = sc.slot[(q - 1) * sc.stride];
+                if (static_cast<unsigned>(m) < static_cast<unsigned>(d.n_sites)) {
+                    own -= x;
+                    red_add(acc + m, x, pol);
+                }
+            });
+        });
+        red_add(acc + n, own, pol);
+        // this step's sums of the site are consumed (the phase pass before this
+        // collision was their last other reader): they receive the step after next
+        st_keep(d.acc[PAR] + n, 0ull, pol);
+    } else {
+        // Populations. With fp16 storage the stored quantity is the deviation
+        // from w_q (1 +- phi_c)/2: the deviation from w_q Na (w_q Nb), which is
+        // +- P (4.5 u_i + ...), plus w_q times Na - (1 + phi_c)/2 = (N - 1)(1 + phi_c)/2
+        // (likewise for Nb); the working units' K on both.
+        T* const A = static_cast<T*>(d.a);
+        T* const B = static_cast<T*>(d.b);
+        const float NK = mul(0.5f * K, Nt);
+        const float Na = mul(NK, pa1), Nb = mul(NK, pb1);
+        const float PA = mul(w7(1), Na), PB = mul(w7(1), Nb);
+        float cA = PA, cB = PB, eA = 0.0f, eB = 0.0f;
+        if constexpr (S::kRef) {
+            const float hN = mul(0.5f * K, add(Nt, -1.0f));
+            eA = mul(hN, pa1);
+            eB = mul(hN, pb1);
+            cA = mul(w7(1), eA);
+            cB = mul(w7(1), eB);
+        }
+        float asum = 0.0f, bsum = 0.0f;
+        static_for<0, 3>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            const float dA = mul(PA, rA[i]), dB = mul(PB, rB[i]);
+            const float a1 = add(cA, dA), a2 = sub(cA, dA), b1 = add(cB, dB), b2 = sub(cB, dB);
+            store(std::integral_constant<int, 2 * i + 1>{}, A, a1);
+            store(std::integral_constant<int, 2 * i + 2>{}, A, a2);
+            store(std::integral_constant<int, 2 * i + 1>{}, B, b1);
+            store(std::integral_constant<int, 2 * i + 2>{}, B, b2);
+            if constexpr (!S::kRef) {
+                if constexpr (i == 0) {
+                    asum = add(a1, a2);
+                    bsum = add(b1, b2);
+                } else {
+                    asum = add(asum, add(a1, a2));
+                    bsum = add(bsum, add(b1, b2));
+                }
+            }
+        });
+        if constexpr (S::kRef) {
+            // The phase pass adds (1 + S)/2 to the seven values a site reads, S
+            // holding w_q phi_c for this site's value of direction q; the seven
+            // stored values above sum to Wsum (Na - (1 + phi_c)/2) with Wsum the
+            // fp32 weights' sum 1 + 2^-26. The rest value takes the difference,
+            // K (1 - Wsum)(Na - 1/2), so that its readers rebuild exactly Na (and
+            // Nb) and the fp32 weights create no mass.
+            constexpr double kWsum = static_cast<double>(w7(0)) + 6.0 * static_cast<double>(w7(1));
+            constexpr float kWerr = static_cast<float>(1.0 - kWsum);
+            S::st_s(A + n, fma(kWerr, add(-0.5f * K, Na), mul(w7(0), eA)));
+            S::st_s(B + n, fma(kWerr, add(-0.5f * K, Nb), mul(w7(0), eB)));
+        } else {
+            S::st_s(A + n, sub(Na, asum));
+            S::st_s(B + n, sub(Nb, bsum));
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
