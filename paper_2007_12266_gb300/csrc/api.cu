@@ -65,12 +65,13 @@ void free_state(lbpm_ctx* c) {
     dfree(c, c->d_b);
     dfree(c, c->d_nsum);
     dfree(c, c->d_drho);
+    dfree(c, c->d_phi);
     dfree(c, c->d_phi_alt);
     dfree(c, c->d_rsum);
     dfree(c, c->d_acc);
     c->d_acc = nullptr;
     c->d_drho = nullptr;
-    c->d_phi_alt = nullptr;
+    c->d_phi = c->d_phi_alt = nullptr;
     c->d_rsum = nullptr;
     c->d_f = c->d_a = c->d_b = nullptr;
     c->d_nsum = nullptr;
@@ -82,11 +83,13 @@ void free_image(lbpm_ctx* c) {
     dfree(c, c->d_labels);
     dfree(c, c->d_site_vox);
     dfree(c, c->d_vsite);
-    dfree(c, c->d_phi);
-    dfree(c, c->d_halo_dst);
-    dfree(c, c->d_halo_site);
-    dfree(c, c->d_wall6);
-    c->d_wall6 = nullptr;
+    dfree(c, c->d_phis);
+    dfree(c, c->d_link_a);
+    dfree(c, c->d_link_b);
+    dfree(c, c->d_wall_c);
+    c->d_link_a = nullptr;
+    c->d_link_b = nullptr;
+    c->d_wall_c = nullptr;
     dfree(c, c->d_slab_site);
     dfree(c, c->d_slab_side);
     dfree(c, c->d_face_part);
@@ -94,10 +97,10 @@ void free_image(lbpm_ctx* c) {
     c->d_face_part = nullptr;
     c->d_face_rho = nullptr;
     c->d_labels = nullptr;
-    c->d_site_vox = c->d_vsite = c->d_halo_dst = c->d_halo_site = c->d_slab_site = nullptr;
-    c->d_phi = nullptr;
+    c->d_site_vox = c->d_vsite = c->d_slab_site = nullptr;
+    c->d_phis = nullptr;
     c->d_slab_side = nullptr;
-    c->N = c->H = c->n_slab = 0;
+    c->N = c->n_slab = 0;
     c->have_image = false;
 }
 
@@ -114,16 +117,16 @@ lbpm_status alloc_state(lbpm_ctx* c) {
     const size_t P = static_cast<size_t>(pitch_of(c->N));
     c->d_nsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
     c->d_acc = static_cast<unsigned long long*>(dalloc(c, sizeof(unsigned long long) * 2 * P));
-    bool ok = c->d_f && c->d_a && c->d_b && c->d_nsum && c->d_acc;
+    c->d_phi = static_cast<float*>(dalloc(c, sizeof(float) * P));
+    bool ok = c->d_f && c->d_a && c->d_b && c->d_nsum && c->d_acc && c->d_phi;
     if (c->params.precision == LBPM_FP16) {
-        // the second phase grid starts as a copy of the first (solids, walls
-        // and their periodic mirrors are static and the same in both)
         c->d_drho = static_cast<float*>(dalloc(c, sizeof(float) * P));
         c->d_rsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
-        c->d_phi_alt = static_cast<float*>(dalloc(c, sizeof(float) * c->Vp));
+        c->d_phi_alt = static_cast<float*>(dalloc(c, sizeof(float) * P));
         ok = ok && c->d_drho && c->d_rsum && c->d_phi_alt;
-        if (ok && cudaMemcpyAsync(c->d_phi_alt, c->d_phi, sizeof(float) * c->Vp, cudaMemcpyDeviceToDevice,
-                                  c->stream) != cudaSuccess)
+        // a state restored without an initialisation takes its references from these
+        if (ok && (cudaMemsetAsync(c->d_phi, 0, sizeof(float) * P, c->stream) != cudaSuccess ||
+                   cudaMemsetAsync(c->d_phi_alt, 0, sizeof(float) * P, c->stream) != cudaSuccess))
             ok = false;
     }
     if (!ok) {
@@ -133,46 +136,25 @@ lbpm_status alloc_state(lbpm_ctx* c) {
     return LBPM_OK;
 }
 
-// halo list (periodic mirrors of pore voxels) and reservoir site list
+// what depends on the periodic axes and the boundaries: the grids' halo, each
+// site's neighbour record and the solids' part of its colour gradient, and the
+// reservoir site list
 lbpm_status build_boundaries(lbpm_ctx* c) {
     drop_graphs(c);
-    dfree(c, c->d_halo_dst);
-    dfree(c, c->d_halo_site);
-    c->d_halo_dst = c->d_halo_site = nullptr;
-    c->H = 0;
     LBPM_CK(c, launch_fill_halo(c, c->stream));
+    const size_t P = static_cast<size_t>(pitch_of(c->N));
+    if (!c->d_link_a) c->d_link_a = static_cast<int4*>(dalloc(c, sizeof(int4) * P));
+    if (!c->d_link_b) c->d_link_b = static_cast<int2*>(dalloc(c, sizeof(int2) * P));
+    if (!c->d_wall_c) c->d_wall_c = static_cast<float*>(dalloc(c, sizeof(float) * 3 * P));
+    if (!c->d_link_a || !c->d_link_b || !c->d_wall_c)
+        return fail(c, LBPM_E_OOM, "device allocation of the neighbour records failed");
+    LBPM_CK(c, launch_links(c, c->stream));
+    LBPM_CK(c, launch_wall_gradient(c, c->stream));
+    LBPM_CK(c, cudaStreamSynchronize(c->stream));
     int* flags;
     int* scan;
-    LBPM_ALLOC(c, flags, int, c->Vp);
-    scan = static_cast<int*>(dalloc(c, sizeof(int) * c->Vp));
-    if (!scan) {
-        dfree(c, flags);
-        return fail(c, LBPM_E_OOM, "device allocation of the halo scan failed");
-    }
-    cudaError_t e = launch_halo_flags(c, flags, c->stream);
-    if (e == cudaSuccess) e = exclusive_scan(c, flags, scan, c->Vp);
     int tail[2] = {0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&tail[0], scan + c->Vp - 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&tail[1], flags + c->Vp - 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e == cudaSuccess) {
-        c->H = static_cast<long long>(tail[0]) + tail[1];
-        if (c->H > 0) {
-            c->d_halo_dst = static_cast<int*>(dalloc(c, sizeof(int) * c->H));
-            c->d_halo_site = static_cast<int*>(dalloc(c, sizeof(int) * c->H));
-            if (!c->d_halo_dst || !c->d_halo_site) e = cudaErrorMemoryAllocation;
-            else e = launch_halo_scatter(c, flags, scan, c->stream);
-        }
-    }
-    if (e == cudaSuccess && !c->d_wall6) {
-        c->d_wall6 = static_cast<unsigned char*>(dalloc(c, pitch_of(c->N)));
-        if (!c->d_wall6) e = cudaErrorMemoryAllocation;
-    }
-    if (e == cudaSuccess) e = launch_wall_mask(c, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    dfree(c, flags);
-    dfree(c, scan);
-    if (e != cudaSuccess) return fail_cuda(c, "halo construction", e);
+    cudaError_t e = cudaSuccess;
 
     // reservoir slabs / boundary faces
     dfree(c, c->d_slab_site);
@@ -549,8 +531,8 @@ lbpm_status lbpm_load_image(lbpm_ctx* c, const uint16_t* labels, int nx, int ny,
     }
     c->d_site_vox = static_cast<int*>(dalloc(c, sizeof(int) * pitch_of(c->N)));
     c->d_vsite = static_cast<int*>(dalloc(c, sizeof(int) * c->Vp));
-    c->d_phi = static_cast<float*>(dalloc(c, sizeof(float) * c->Vp));
-    if (!c->d_site_vox || !c->d_vsite || !c->d_phi) {
+    c->d_phis = static_cast<float*>(dalloc(c, sizeof(float) * c->Vp));
+    if (!c->d_site_vox || !c->d_vsite || !c->d_phis) {
         dfree(c, flags);
         dfree(c, scan);
         return fail(c, LBPM_E_OOM, "device allocation of the index failed");
@@ -580,10 +562,11 @@ lbpm_status lbpm_set_affinity_table(lbpm_ctx* c, const float* table, int n_label
     cudaError_t e = cudaMemcpyAsync(d_t, table, sizeof(float) * n_labels, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = launch_affinity_table(c, d_t, n_labels, c->stream);
     if (e == cudaSuccess) e = launch_fill_halo(c, c->stream);
+    if (e == cudaSuccess) e = launch_wall_gradient(c, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d_t);
     if (e != cudaSuccess) return fail_cuda(c, "affinity table", e);
-    c->launches += 2;
+    c->launches += 3;
     return LBPM_OK;
 }
 
@@ -597,10 +580,11 @@ lbpm_status lbpm_set_affinity_map(lbpm_ctx* c, const float* map) {
     cudaError_t e = cudaMemcpyAsync(d_m, map, sizeof(float) * c->V, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = launch_affinity_map(c, d_m, c->stream);
     if (e == cudaSuccess) e = launch_fill_halo(c, c->stream);
+    if (e == cudaSuccess) e = launch_wall_gradient(c, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d_m);
     if (e != cudaSuccess) return fail_cuda(c, "affinity map", e);
-    c->launches += 2;
+    c->launches += 3;
     return LBPM_OK;
 }
 
@@ -620,7 +604,7 @@ lbpm_status lbpm_init_fluids(lbpm_ctx* c, const float* phi0) {
     c->step = 0;
     c->have_fluids = true;
     c->unstable = false;
-    c->launches += c->params.precision == LBPM_FP16 ? 5 : 2;
+    c->launches += c->params.precision == LBPM_FP16 ? 4 : 2;
     return LBPM_OK;
 }
 

@@ -74,10 +74,10 @@ __global__ void __launch_bounds__(BT) k_batch_phase_sum(const __grid_constant__ 
 }
 
 // CF: component form of the collision (see collide_site).
-// 36 resident warps per SM where the block size allows (56 registers at 128
-// threads), as for the single-domain collision.
+// 32 resident warps per SM where the block size allows (64 registers), as for
+// the single-domain collision.
 template <int PAR, class S, int CF, int BT>
-__global__ void __launch_bounds__(BT, 1152 / BT) k_batch_collide(const __grid_constant__ BatchLaunch p) {
+__global__ void __launch_bounds__(BT, 1024 / BT) k_batch_collide(const __grid_constant__ BatchLaunch p) {
     constexpr int kSlots = PAR == 1 ? (Q19 - 1) * BT : (CF != 0 ? (Q7 - 1) * BT : 1);
     constexpr int kRefs = PAR == 1 && S::kRef ? (Q19 - 1) * BT : 1;
     __shared__ int slot[kSlots];

@@ -41,7 +41,7 @@ struct lbpm_batch {
     // one block per tile). The default is the fastest shape measured on GB300
     // for mixed job sizes in both storages: one block per tile (the hardware
     // block scheduler balances uneven tiles better than a static round-robin
-    // over persistent blocks) of 192 threads (six blocks, 36 warps per SM at 56
+    // over persistent blocks) of 192 threads (five blocks, 30 warps per SM at 64
     // registers for the collision).
     int bt = 192;
     int bps[2] = {-1, -1};
@@ -136,7 +136,7 @@ lbpm_status rebuild(lbpm_batch* b) {
         const lbpm_ctx* c = b->jobs[j];
         views[j] = make_view(c);
         parity[j] = static_cast<int>(c->step & 1);
-        const long long counts[2] = {c->N + c->H, c->N};
+        const long long counts[2] = {c->N, c->N};
         for (int k = 0; k < 2; ++k) {
             if (j % kBatchLaunchJobs == 0) {
                 b->launch[k].emplace_back();
@@ -199,7 +199,7 @@ lbpm_status rebuild(lbpm_batch* b) {
         for (int j = 0; j < J; ++j) {
             const lbpm_ctx* c = b->jobs[j];
             const long long n_slab = c->params.reservoir_z == 1 ? c->n_slab : 0;
-            const long long counts[3] = {c->N + c->H, c->N, n_slab};
+            const long long counts[3] = {c->N, c->N, n_slab};
             const long long per_tile[3] = {static_cast<long long>(b->bt) * fused_phase_per(b->bt), b->bt, b->bt};
             for (int k = 0; k < 3; ++k)
                 F.tiles[k][j + 1] = F.tiles[k][j] + static_cast<int>((counts[k] + per_tile[k] - 1) / per_tile[k]);
@@ -434,7 +434,6 @@ lbpm_status lbpm_batch_add(lbpm_batch* b, lbpm_ctx* job) {
         return bfail(b, LBPM_E_INVALID, "job is already in the batch");
     if (b->precision >= 0 && job->params.precision != b->precision)
         return bfail(b, LBPM_E_INVALID, "all jobs of a batch share the storage precision");
-    if (job->N + job->H >= (1LL << 31)) return bfail(b, LBPM_E_INVALID, "job too large");
     // the job's pending work (on its own stream) must be done before the batch uses it
     if (cudaStreamSynchronize(job->stream) != cudaSuccess) return bfail(b, LBPM_E_CUDA, "job stream failed");
     b->precision = job->params.precision;

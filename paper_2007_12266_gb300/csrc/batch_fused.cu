@@ -114,7 +114,7 @@ struct FusedKind {
 
 // NS timesteps of the given kind, the first at parity PAR0.
 template <class S, int BT, int KIND, int PAR0, int NS>
-__global__ void __launch_bounds__(BT, 1152 / BT) k_batch_fused(const __grid_constant__ FusedLaunch p) {
+__global__ void __launch_bounds__(BT, 1024 / BT) k_batch_fused(const __grid_constant__ FusedLaunch p) {
     using K = FusedKind<KIND>;
     __shared__ int slot[(Q19 - 1) * BT];
     __shared__ float ref[S::kRef ? (Q19 - 1) * BT : 1];

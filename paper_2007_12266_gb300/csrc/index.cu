@@ -4,13 +4,15 @@
 // order by an exclusive prefix sum over the pore flags, which makes the site
 // numbering identical to a sequential scan of the image. Two padded grids
 // (one halo voxel per face) then resolve neighbours without branches:
-// vsite[pv] is the site id of padded voxel pv (-1: solid or wall) and
-// phi[pv] holds the phase field, with phi_s (Sec. 3.2, Eq. phi_s) at solids and
-// 0 outside non-periodic faces. Halo voxels of periodic axes copy the voxel
-// they wrap to; those that mirror pores are listed so the phase pass can
-// refresh them every step.
+// vsite[pv] is the site id of padded voxel pv (negative: solid, where it is the
+// complement of the voxel's rank, or wall, -1) and phis[pv] holds phi_s
+// (Sec. 3.2, Eq. phi_s) at solids and 0 elsewhere. Halo voxels of periodic axes
+// copy the voxel they wrap to. The steps themselves read what is derived from
+// these grids per site: the neighbour ids (SiteLinks) and the solids' part of
+// the colour gradient.
 #include "internal.h"
 #include "lattice.cuh"
+#include "links.cuh"
 
 namespace lbm {
 
@@ -100,18 +102,18 @@ __global__ void k_flag_pore(const uint16_t* labels, long long V, int* flags) {
 }
 
 __global__ void k_scatter_sites(const uint16_t* labels, const int* scan, long long V, int nx, int ny,
-                                int px, int py, int* site_vox, int* vsite, float* phi) {
+                                int px, int py, int* site_vox, int* vsite, float* phis) {
     const long long v = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
     if (v >= V) return;
     const long long pv = padded_of(v, nx, ny, px, py);
+    const int s = scan[v];
     if (labels[v] == 0) {
-        const int s = scan[v];
         site_vox[s] = static_cast<int>(pv);
         vsite[pv] = s;
     } else {
-        vsite[pv] = -1;
+        vsite[pv] = ~s;
     }
-    phi[pv] = 0.0f;
+    phis[pv] = 0.0f;
 }
 
 // Resolve a padded voxel: returns 0 for interior voxels, 1 for a halo voxel
@@ -146,60 +148,36 @@ Geo geo_of(const lbpm_ctx* c) {
                c->params.periodic[2], c->Vp};
 }
 
-// phi2: the second phase grid (fp16 storage), or nullptr
-__global__ void k_fill_halo(Geo g, int* vsite, float* phi, float* phi2) {
+__global__ void k_fill_halo(Geo g, int* vsite, float* phis) {
     const long long pv = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
     if (pv >= g.Vp) return;
     long long src = 0;
     const int k = halo_kind(pv, g.nx, g.ny, g.nz, g.px, g.py, g.perx, g.pery, g.perz, &src);
     if (k == 1) {
         vsite[pv] = vsite[src];
-        phi[pv] = phi[src];
-        if (phi2) phi2[pv] = phi2[src];
+        phis[pv] = phis[src];
     } else if (k == 2) {
         vsite[pv] = -1;
-        phi[pv] = 0.0f;
-        if (phi2) phi2[pv] = 0.0f;
+        phis[pv] = 0.0f;
     }
 }
 
-__global__ void k_halo_flags(Geo g, const int* vsite, int* flags) {
-    const long long pv = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
-    if (pv >= g.Vp) return;
-    long long src = 0;
-    const int k = halo_kind(pv, g.nx, g.ny, g.nz, g.px, g.py, g.perx, g.pery, g.perz, &src);
-    flags[pv] = (k == 1 && vsite[pv] >= 0) ? 1 : 0;
-}
-
-__global__ void k_halo_scatter(long long Vp, const int* flags, const int* scan, const int* vsite,
-                               int* halo_dst, int* halo_site) {
-    const long long pv = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
-    if (pv >= Vp || !flags[pv]) return;
-    const int e = scan[pv];
-    halo_dst[e] = static_cast<int>(pv);
-    halo_site[e] = vsite[pv];
-}
-
 __global__ void k_affinity_table(const uint16_t* labels, long long V, int nx, int ny, int px, int py,
-                                 const float* table, int n_labels, float* phi, float* phi2) {
+                                 const float* table, int n_labels, float* phis) {
     const long long v = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
     if (v >= V) return;
     const int lab = labels[v];
     if (lab == 0) return;
     const float a = lab < n_labels ? table[lab] : 0.0f;
-    const long long pv = padded_of(v, nx, ny, px, py);
-    phi[pv] = a;
-    if (phi2) phi2[pv] = a;
+    phis[padded_of(v, nx, ny, px, py)] = a;
 }
 
 __global__ void k_affinity_map(const uint16_t* labels, long long V, int nx, int ny, int px, int py,
-                               const float* map, float* phi, float* phi2) {
+                               const float* map, float* phis) {
     const long long v = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
     if (v >= V) return;
     if (labels[v] == 0) return;
-    const long long pv = padded_of(v, nx, ny, px, py);
-    phi[pv] = map[v];
-    if (phi2) phi2[pv] = map[v];
+    phis[padded_of(v, nx, ny, px, py)] = map[v];
 }
 
 // 1: inlet (the first `depth` z layers), 2: outlet (the last ones), 0: neither
@@ -235,22 +213,62 @@ __global__ void k_export_index(const int* site_vox, const int* vsite, long long 
         site2vox[n] = (X - 1) + static_cast<long long>(nx) * ((Y - 1) + static_cast<long long>(ny) * (Z - 1));
     }
     if (nbr) {
-        for (int q = 1; q < Q19; ++q) nbr[static_cast<long long>(q - 1) * N + n] = vsite[pv + stencil_off(d, q)];
+        for (int q = 1; q < Q19; ++q) nbr[static_cast<long long>(q - 1) * N + n] = max(vsite[pv + stencil_off(d, q)], -1);
     }
 }
 
-// Which face links of each site bounce back: bit q - 1 for x + xi_q solid or
-// wall (q = 1..6). Read by the fp16 collision to pick the site whose phase is
-// the reference of each stored component value.
-__global__ void k_wall_mask(const int* site_vox, const int* vsite, long long N, int px, int pxpy,
-                            unsigned char* wall6) {
+__device__ __forceinline__ int rank_of(int id) { return id >= 0 ? id : ~id; }
+__device__ __forceinline__ int pack16(int lo, int hi) {
+    return static_cast<int>((static_cast<unsigned>(lo) & 0xffffu) | (static_cast<unsigned>(hi) << 16));
+}
+
+// The neighbour record of each site (SiteLinks). Every id that the record gives
+// is compared with the dense grid's; a site with any difference is marked
+// irregular.
+__global__ void k_links(const int* site_vox, const int* vsite, long long N, int px, int pxpy, int4* link_a,
+                        int2* link_b) {
     const long long n = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
     if (n >= N) return;
     const int pv = site_vox[n];
-    unsigned m = 0;
-    for (int q = 1; q < Q7; ++q)
-        if (vsite[pv + stencil_offset(q, px, pxpy)] < 0) m |= 1u << (q - 1);
-    wall6[n] = static_cast<unsigned char>(m);
+    int nb[Q19];
+    unsigned bits = 0;
+    static_for<1, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        nb[q] = vsite[pv + stencil_offset(q, px, pxpy)];
+        if (nb[q] >= 0) bits |= 1u << (q - 1);
+    });
+    const int id = static_cast<int>(n);
+    const int zp = rank_of(nb[5]), zm = rank_of(nb[6]);
+    int4 a = make_int4(pack16(rank_of(nb[3]) - id, rank_of(nb[4]) - id), zp, zm, static_cast<int>(bits));
+    const int2 b = make_int2(pack16(rank_of(nb[15]) - zp, rank_of(nb[18]) - zp),
+                             pack16(rank_of(nb[17]) - zm, rank_of(nb[16]) - zm));
+    const SiteLinks l{a, b};
+    bool ok = true;
+    static_for<1, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        if (nb[q] >= 0 && link_id<q>(id, l) != nb[q]) ok = false;
+    });
+    if (!ok) a.w |= kIrregular;
+    link_a[n] = a;
+    link_b[n] = b;
+}
+
+// The solids' part of twice the colour gradient at each site (face weight 1,
+// edge weight 1/2): static between changes of the wetting map.
+__global__ void k_wall_gradient(const int* site_vox, const float* phis, long long N, long long P, int px, int pxpy,
+                                float* wall_c) {
+    const long long n = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
+    if (n >= N) return;
+    const int pv = site_vox[n];
+    float c[3] = {0.0f, 0.0f, 0.0f};
+    static_for<1, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        const float p = 2.0f * grad_w(q) * phis[pv + stencil_offset(q, px, pxpy)];
+        if constexpr (cx(q) != 0) c[0] += cx(q) * p;
+        if constexpr (cy(q) != 0) c[1] += cy(q) * p;
+        if constexpr (cz(q) != 0) c[2] += cz(q) * p;
+    });
+    for (int i = 0; i < 3; ++i) wall_c[i * P + n] = c[i];
 }
 
 }  // namespace
@@ -289,35 +307,24 @@ cudaError_t exclusive_scan(lbpm_ctx* c, const int* in, int* out, long long n) {
 
 cudaError_t launch_scatter_sites(const lbpm_ctx* c, const int* scan, cudaStream_t s) {
     k_scatter_sites<<<blocks_for(c->V), kBlock, 0, s>>>(c->d_labels, scan, c->V, c->nx, c->ny, c->px,
-                                                        c->py, c->d_site_vox, c->d_vsite, c->d_phi);
+                                                        c->py, c->d_site_vox, c->d_vsite, c->d_phis);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fill_halo(const lbpm_ctx* c, cudaStream_t s) {
-    k_fill_halo<<<blocks_for(c->Vp), kBlock, 0, s>>>(geo_of(c), c->d_vsite, c->d_phi, c->d_phi_alt);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_halo_flags(const lbpm_ctx* c, int* flags, cudaStream_t s) {
-    k_halo_flags<<<blocks_for(c->Vp), kBlock, 0, s>>>(geo_of(c), c->d_vsite, flags);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_halo_scatter(const lbpm_ctx* c, const int* flags, const int* scan, cudaStream_t s) {
-    k_halo_scatter<<<blocks_for(c->Vp), kBlock, 0, s>>>(c->Vp, flags, scan, c->d_vsite, c->d_halo_dst,
-                                                       c->d_halo_site);
+    k_fill_halo<<<blocks_for(c->Vp), kBlock, 0, s>>>(geo_of(c), c->d_vsite, c->d_phis);
     return cudaGetLastError();
 }
 
 cudaError_t launch_affinity_table(const lbpm_ctx* c, const float* table, int n_labels, cudaStream_t s) {
     k_affinity_table<<<blocks_for(c->V), kBlock, 0, s>>>(c->d_labels, c->V, c->nx, c->ny, c->px, c->py,
-                                                         table, n_labels, c->d_phi, c->d_phi_alt);
+                                                         table, n_labels, c->d_phis);
     return cudaGetLastError();
 }
 
 cudaError_t launch_affinity_map(const lbpm_ctx* c, const float* map, cudaStream_t s) {
     k_affinity_map<<<blocks_for(c->V), kBlock, 0, s>>>(c->d_labels, c->V, c->nx, c->ny, c->px, c->py,
-                                                       map, c->d_phi, c->d_phi_alt);
+                                                       map, c->d_phis);
     return cudaGetLastError();
 }
 
@@ -343,10 +350,17 @@ cudaError_t launch_export_index(const lbpm_ctx* c, long long* site2vox, int* nbr
     return cudaGetLastError();
 }
 
-cudaError_t launch_wall_mask(const lbpm_ctx* c, cudaStream_t s) {
+cudaError_t launch_links(const lbpm_ctx* c, cudaStream_t s) {
     if (c->N == 0) return cudaSuccess;
-    k_wall_mask<<<blocks_for(c->N), kBlock, 0, s>>>(c->d_site_vox, c->d_vsite, c->N, c->px,
-                                                    c->px * c->py, c->d_wall6);
+    k_links<<<blocks_for(c->N), kBlock, 0, s>>>(c->d_site_vox, c->d_vsite, c->N, c->px, c->px * c->py, c->d_link_a,
+                                                c->d_link_b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_wall_gradient(const lbpm_ctx* c, cudaStream_t s) {
+    if (c->N == 0) return cudaSuccess;
+    k_wall_gradient<<<blocks_for(c->N), kBlock, 0, s>>>(c->d_site_vox, c->d_phis, c->N, pitch_of(c->N), c->px,
+                                                        c->px * c->py, c->d_wall_c);
     return cudaGetLastError();
 }
 

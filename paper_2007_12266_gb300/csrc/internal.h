@@ -13,6 +13,25 @@
 
 namespace lbm {
 
+// Where a site's neighbours are. Sites are numbered in x-fastest order, so in
+// the x-row through x + (0, dy, dz) the site at the row's middle voxel has the
+// rank r of that voxel (the number of pore voxels before it, defined at solids
+// too), the one at dx = +1 has r + 1 (r if the middle voxel is solid) and the
+// one at dx = -1 has r - 1: eight ranks and one bit per direction give all 18
+// neighbour ids. The ranks of the rows next to a known one are stored as 16-bit
+// differences, so a site's record is 24 bytes, read with two coalesced vector
+// loads.
+struct SiteLinks {
+    int4 a;             // x: ranks of rows (+y, -y) minus the site's own id (low, high 16 bits);
+                        // y, z: ranks of rows +z, -z; w: bit q - 1 set when x + xi_q is a pore
+                        // site (q = 1..18), kIrregular when the record does not hold for the site
+    int2 b;             // ranks of rows (+z +y, +z -y) minus that of +z; (-z +y, -z -y) minus that of -z
+};
+// Sites next to a periodic x face (where the next voxel of the row is at its
+// other end), and those whose differences exceed 16 bits: their neighbours are
+// looked up in the dense grid of site ids.
+constexpr int kIrregular = static_cast<int>(0x80000000u);
+
 // Everything a step kernel needs, passed by value as a kernel parameter.
 // Grids are "padded": (nx+2)(ny+2)(nz+2) voxels, one halo layer per face, so
 // neighbour voxel = v + off[q] never leaves the allocation. The halo of a
@@ -20,18 +39,16 @@ namespace lbm {
 struct DomainView {
     int n_sites;        // N: pore sites
     int pitch;          // P: row length of the per-site arrays, N rounded up (see kPitch)
-    int n_halo;         // H: halo voxels that mirror a pore site
     int px, pxpy;       // padded-grid strides in y and z: xi_q is at offset cx + cy px + cz pxpy
     const int* site_vox;   // [N] padded voxel of each site
-    const int* vsite;      // [Vp] site id, -1 for solid / wall
-    float* phi[2];         // [Vp] phase field by step parity: the phase pass of a step of parity P
+    const int* vsite;      // [Vp] site id; negative for solid (the complement of its rank) and wall (-1)
+    const int4* link_a;    // [N] SiteLinks::a
+    const int2* link_b;    // [N] SiteLinks::b
+    const float* wall_c;   // [3][P] the solids' part of twice the colour gradient, sum_q 2 g_q xi_q phi_s
+    float* phi[2];         // [N] phase of each site by step parity: the phase pass of a step of parity P
                            //     writes phi[P] and the collision reads it; with fp16 storage the
                            //     previous step's phi[P ^ 1] is the reference of the stored
-                           //     components (with fp32 storage both point to one grid).
-                           //     Solids hold phi_s, walls 0.
-    const int* halo_dst;   // [H] padded halo voxel
-    const int* halo_site;  // [H] site it mirrors
-    const unsigned char* wall6;  // [N] bit q - 1 set when x + xi_q (q = 1..6) is solid or wall
+                           //     components (with fp32 storage both point to one array)
     float* nsum;           // [N] Na + Nb of the current step (phase pass -> collision)
     float* rsum;           // [N] fp16 store: sum_q w_q phi_w(q) of the component references that the
                            //     next phase pass reads (collision -> phase pass, see StoreF16)
@@ -83,16 +100,17 @@ struct lbpm_ctx {
     int nx = 0, ny = 0, nz = 0;
     int px = 0, py = 0, pz = 0;
     long long V = 0, Vp = 0;
-    long long N = 0, H = 0;
+    long long N = 0;
     bool have_image = false, have_fluids = false, unstable = false;
     uint16_t* d_labels = nullptr;   // [V]
     int* d_site_vox = nullptr;      // [N]
     int* d_vsite = nullptr;         // [Vp]
-    float* d_phi = nullptr;         // [Vp]
-    float* d_phi_alt = nullptr;     // [Vp] fp16 storage: the phase grid of odd steps
-    int* d_halo_dst = nullptr;      // [H]
-    int* d_halo_site = nullptr;     // [H]
-    unsigned char* d_wall6 = nullptr;  // [N] face links that bounce back
+    float* d_phis = nullptr;        // [Vp] phi_s of solid voxels, 0 at pores and walls
+    int4* d_link_a = nullptr;       // [N] SiteLinks
+    int2* d_link_b = nullptr;       // [N]
+    float* d_wall_c = nullptr;      // [3][N] the solids' part of the colour gradient
+    float* d_phi = nullptr;         // [N] phase of each site
+    float* d_phi_alt = nullptr;     // [N] fp16 storage: the phase at odd steps
     float* d_nsum = nullptr;        // [N]
     float* d_rsum = nullptr;        // [N] fp16 storage
     double* d_face_part = nullptr;          // flux inlet: per-block sums (2 * kFaceBlocks)
@@ -137,14 +155,13 @@ cudaError_t launch_flag_pore(const uint16_t* labels, long long V, int* flags, cu
 cudaError_t exclusive_scan(lbpm_ctx* c, const int* in, int* out, long long n);
 cudaError_t launch_scatter_sites(const lbpm_ctx* c, const int* scan, cudaStream_t s);
 cudaError_t launch_fill_halo(const lbpm_ctx* c, cudaStream_t s);
-cudaError_t launch_halo_flags(const lbpm_ctx* c, int* flags, cudaStream_t s);
-cudaError_t launch_halo_scatter(const lbpm_ctx* c, const int* flags, const int* scan, cudaStream_t s);
 cudaError_t launch_affinity_table(const lbpm_ctx* c, const float* table, int n_labels, cudaStream_t s);
 cudaError_t launch_affinity_map(const lbpm_ctx* c, const float* map, cudaStream_t s);
 cudaError_t launch_slab_flags(const lbpm_ctx* c, int* flags, cudaStream_t s);
 cudaError_t launch_slab_scatter(const lbpm_ctx* c, const int* flags, const int* scan, cudaStream_t s);
 cudaError_t launch_export_index(const lbpm_ctx* c, long long* site2vox, int* nbr, cudaStream_t s);
-cudaError_t launch_wall_mask(const lbpm_ctx* c, cudaStream_t s);
+cudaError_t launch_links(const lbpm_ctx* c, cudaStream_t s);
+cudaError_t launch_wall_gradient(const lbpm_ctx* c, cudaStream_t s);
 
 // Look up (once per device, with that device current) the device address of
 // the static staging array of lbpm_read_field_noalloc; called by lbpm_create.
@@ -180,8 +197,8 @@ cudaError_t launch_morph(const lbpm_ctx* c, int parity, float delta, int R, int 
 constexpr int NSUM = 27;  // per-site sums reduced by the measure kernel
 void fill_measures(const lbpm_ctx* c, const double* S, lbpm_measures* out);
 
-// One tile of a batched launch: `first` is the first thread index (site, or
-// site/halo entry for the phase pass) of job `job` that the block handles.
+// One tile of a batched launch: `first` is the first site of job `job` that the
+// block handles.
 struct BatchTile {
     int job;
     int first;

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kBlock) k_box(DomainView d, int which, int3 lo
 // fp16 store: the reference density of imported momentum populations is the
 // sum of the imported values at each site (any reference works as long as the
 // reader uses the same one); imported component values are stored relative to
-// the references the next step reads them with (the previous phase grid).
+// the references the next step reads them with (the previous phases).
 __global__ void __launch_bounds__(kBlock) k_import_ref(DomainView d, const float* in) {
     const int n = blockIdx.x * kBlock + threadIdx.x;
     if (n >= d.n_sites) return;
@@ -139,15 +139,15 @@ template <int PAR, class S>
 __global__ void __launch_bounds__(kBlock) k_import(DomainView d, int which, const float* in) {
     const int n = blockIdx.x * kBlock + threadIdx.x;
     if (n >= d.n_sites) return;
-    const int v = d.site_vox[n];
     int nb[Q19];
     if constexpr (PAR == 1) {
+        const int v = d.site_vox[n];
         static_for<1, Q19>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
             nb[q] = __ldg(d.vsite + v + stencil_off(d, q));
         });
     }
-    const unsigned wall = S::kRef ? __ldg(d.wall6 + n) : 0u;
+    if constexpr (S::kRef && PAR == 0) face_neighbours(d, n, nb);
     const size_t N = d.n_sites;
     static_for<0, Q19>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kBlock) k_import(DomainView d, int which, cons
             if (which != LBPM_DIST_F) {
                 float val = in[q * N + n];
                 if constexpr (S::kRef) {
-                    const float pw = writer_phase<PAR, q>(d, v, wall);
+                    const float pw = writer_phase<PAR, q>(d, n, nb);
                     val -= w7(q) * 0.5f * (which == LBPM_DIST_A ? 1.0f + pw : 1.0f - pw);
                 }
                 if (which == LBPM_DIST_A) S::template st_c<q>(d.a, i, val);

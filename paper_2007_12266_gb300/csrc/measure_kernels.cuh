@@ -12,20 +12,21 @@ namespace lbm {
 template <int PAR, class S>
 __device__ __forceinline__ void load_site(const DomainView& d, int n, float (&f)[Q19], float (&a)[Q7],
                                           float (&b)[Q7]) {
-    const int v = d.site_vox[n];
     int nb[Q19];
     if constexpr (PAR == 1) {
+        const int v = d.site_vox[n];
         static_for<1, Q19>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
             nb[q] = __ldg(d.vsite + v + stencil_off(d, q));
         });
     }
+    if constexpr (need_face_nb<PAR, S>() && PAR == 0) face_neighbours(d, n, nb);
     static_for<0, Q19>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
         f[q] = S::template ld_f<q>(d.f, read_slot<PAR, q>(d, n, nb));
         if constexpr (S::kRef) f[q] = fmaf(t19(q), d.drho[f_ref_read<PAR, q>(n, nb)], f[q]);
     });
-    load_components<PAR, S>(d, n, v, nb, a, b);
+    load_components<PAR, S>(d, n, nb, a, b);
 }
 
 // Per-thread accumulator of per-site fp32 quantities: compensated fp32

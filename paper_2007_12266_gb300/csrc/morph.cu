@@ -131,13 +131,13 @@ __global__ void __launch_bounds__(kMorphBlock) k_morph_apply(DomainView d, Morph
                     });
                 }
                 const float na = 0.5f * N * (1.0f + phin), nbb = 0.5f * N * (1.0f - phin);
-                const unsigned wall = S::kRef ? __ldg(d.wall6 + n) : 0u;
+                if constexpr (S::kRef && PAR == 0) face_neighbours(d, n, nb);
                 static_for<0, Q7>([&](auto qc) {
                     constexpr int q = decltype(qc)::value;
                     float av = w7(q) * na, bv = w7(q) * nbb;
                     if constexpr (S::kRef) {
                         // the reference the next step reads it with
-                        const float pw = writer_phase<PAR, q>(d, v, wall);
+                        const float pw = writer_phase<PAR, q>(d, n, nb);
                         av -= w7(q) * 0.5f * (1.0f + pw);
                         bv -= w7(q) * 0.5f * (1.0f - pw);
                     }

@@ -41,14 +41,14 @@ __global__ void __launch_bounds__(kBlock) k_phase_sum(DomainView d) {
     phase_sum_thread<PAR, WRITE_N, kPhaseSumPer>(d, blockIdx.x * kBlock * kPhaseSumPer + threadIdx.x, kBlock);
 }
 
-// Launch shape of the collision: 56 registers and 36 resident warps per SM
-// (six blocks of 192 threads in FP32, nine of 128 in FP16) measured 4-5 %
-// faster on the 256^3 workload than 64 registers and 32 warps (four blocks of
-// 256), which leaves fewer warps to cover the memory latency.
+// Launch shape of the collision: 64 registers and 32 resident warps per SM.
+// Blocks of 256 in FP32 and 128 in FP16 measured 146 and 135 us per step on the
+// 256^3 workload; 56 registers and 36 warps (192 and 128 threads) spill and took
+// 152-155 and 153 us.
 template <class S>
 struct CollideShape {
-    static constexpr int kThreads = S::kRef ? 128 : 192;
-    static constexpr int kBlocksPerSm = S::kRef ? 9 : 6;
+    static constexpr int kThreads = S::kRef ? 128 : 256;
+    static constexpr int kBlocksPerSm = 1024 / kThreads;
 };
 
 // CF: component form of the collision (see collide_site)
@@ -137,13 +137,13 @@ __device__ __forceinline__ float phi0_of_site(const DomainView& d, int n, const 
     return fminf(1.0f, fmaxf(-1.0f, p));
 }
 
-// The phase grid that step 0 reads as the previous step's: phi0 (fp16
+// The phases that step 0 reads as the previous step's: phi0 (fp16
 // storage: the references of the initial component values).
 __global__ void __launch_bounds__(kBlock) k_init_phase(DomainView d, const float* phi0, int nx, int ny, int px,
                                                        int pxpy) {
     const int n = blockIdx.x * kBlock + threadIdx.x;
     if (n >= d.n_sites) return;
-    d.phi[1][d.site_vox[n]] = phi0_of_site(d, n, phi0, nx, ny, px, pxpy);
+    d.phi[1][n] = phi0_of_site(d, n, phi0, nx, ny, px, pxpy);
 }
 
 // fp16 storage: the references' phase sum of every site for a step of parity
@@ -152,13 +152,13 @@ template <int PAR>
 __global__ void __launch_bounds__(kBlock) k_ref_sum(DomainView d) {
     const int n = blockIdx.x * kBlock + threadIdx.x;
     if (n >= d.n_sites) return;
-    d.rsum[n] = reference_phase_sum<PAR>(d, n, d.site_vox[n]);
+    d.rsum[n] = reference_phase_sum<PAR>(d, n);
 }
 
 // Initial state consistent with phi0 (rho = 1, u = 0), written in the even
 // (natural) layout: Na = (1 + phi0)/2, Nb = (1 - phi0)/2. With fp16 storage the
 // density reference is rho = 1 and the component references come from the
-// phase grid that k_init_phase wrote (periodic mirrors included).
+// phases that k_init_phase wrote.
 template <class S>
 __global__ void __launch_bounds__(kBlock) k_init(DomainView d, const float* phi0, int nx, int ny,
                                                  int px, int pxpy) {
@@ -166,11 +166,10 @@ __global__ void __launch_bounds__(kBlock) k_init(DomainView d, const float* phi0
     if (n >= d.n_sites) return;
     const float p = phi0_of_site(d, n, phi0, nx, ny, px, pxpy);
     const float na = 0.5f * (1.0f + p), nb = 0.5f * (1.0f - p);
-    const int v = d.site_vox[n];
-    unsigned wall = 0;
+    int face[Q7];
     if constexpr (S::kRef) {
         d.drho[n] = 0.0f;
-        wall = __ldg(d.wall6 + n);
+        face_neighbours(d, n, face);
     }
     const size_t P = d.pitch;
     static_for<0, Q19>([&](auto qc) {
@@ -179,7 +178,7 @@ __global__ void __launch_bounds__(kBlock) k_init(DomainView d, const float* phi0
         if constexpr (q < Q7) {
             float av = w7(q) * na, bv = w7(q) * nb;
             if constexpr (S::kRef) {
-                const float pw = writer_phase<0, q>(d, v, wall);
+                const float pw = writer_phase<0, q>(d, n, face);
                 av -= w7(q) * 0.5f * (1.0f + pw);
                 bv -= w7(q) * 0.5f * (1.0f - pw);
             }
@@ -197,16 +196,15 @@ DomainView make_view(const lbpm_ctx* c) {
     DomainView d{};
     d.n_sites = static_cast<int>(c->N);
     d.pitch = static_cast<int>(pitch_of(c->N));
-    d.n_halo = static_cast<int>(c->H);
     d.px = static_cast<int>(c->px);
     d.pxpy = static_cast<int>(c->px * c->py);
     d.site_vox = c->d_site_vox;
     d.vsite = c->d_vsite;
     d.phi[0] = c->d_phi;
     d.phi[1] = c->d_phi_alt ? c->d_phi_alt : c->d_phi;
-    d.halo_dst = c->d_halo_dst;
-    d.halo_site = c->d_halo_site;
-    d.wall6 = c->d_wall6;
+    d.link_a = c->d_link_a;
+    d.link_b = c->d_link_b;
+    d.wall_c = c->d_wall_c;
     d.nsum = c->d_nsum;
     d.drho = c->d_drho;
     d.rsum = c->d_rsum;
@@ -239,7 +237,6 @@ cudaError_t launch_init_fluids(const lbpm_ctx* c, const float* phi0, cudaStream_
     if (h) {
         k_init_phase<<<blocks_for(c->N), kBlock, 0, s>>>(d, phi0, c->nx, c->ny, c->px, c->px * c->py);
         cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) e = launch_fill_halo(c, s);   // periodic mirrors of the initial phase
         if (e != cudaSuccess) return e;
         k_init<StoreF16><<<blocks_for(c->N), kBlock, 0, s>>>(d, phi0, c->nx, c->ny, c->px, c->px * c->py);
         k_ref_sum<0><<<blocks_for(c->N), kBlock, 0, s>>>(d);
@@ -258,7 +255,7 @@ cudaError_t launch_ref_sum(const lbpm_ctx* c, int parity, cudaStream_t s) {
 
 cudaError_t launch_phase(const lbpm_ctx* c, int parity, cudaStream_t s) {
     DomainView d = make_view(c);
-    const unsigned g = blocks_for(c->N + c->H);
+    const unsigned g = blocks_for(c->N);
     if (g == 0) return cudaSuccess;
     const bool h = c->params.precision == LBPM_FP16;
     if (parity == 0) return h ? launch_pdl(k_phase<0, StoreF16>, g, s, d) : launch_pdl(k_phase<0, StoreF32>, g, s, d);
@@ -284,7 +281,7 @@ cudaError_t launch_collide(const lbpm_ctx* c, int parity, cudaStream_t s) {
 
 cudaError_t launch_phase_sum(const lbpm_ctx* c, int parity, bool write_nsum, cudaStream_t s) {
     DomainView d = make_view(c);
-    const unsigned g = blocks_for((c->N + c->H + kPhaseSumPer - 1) / kPhaseSumPer);
+    const unsigned g = blocks_for((c->N + kPhaseSumPer - 1) / kPhaseSumPer);
     if (g == 0) return cudaSuccess;
     if (parity == 0) return write_nsum ? launch_pdl(k_phase_sum<0, true>, g, s, d) : launch_pdl(k_phase_sum<0, false>, g, s, d);
     return write_nsum ? launch_pdl(k_phase_sum<1, true>, g, s, d) : launch_pdl(k_phase_sum<1, false>, g, s, d);

@@ -14,6 +14,7 @@
 
 #include "internal.h"
 #include "lattice.cuh"
+#include "links.cuh"
 
 namespace lbm {
 
@@ -72,10 +73,9 @@ struct StoreF32 {
 // one coalesced load); drho is written only at even steps.
 // Components: A_q - w_q (1 + phi_w)/2 and B_q - w_q (1 - phi_w)/2, with phi_w
 // the phase of the site w that wrote the value, at that step. The writer uses
-// its own phase; the reader finds phi_w in the previous step's phase grid
-// (DomainView::phi is double-buffered by step parity) at the upstream voxel
-// x - xi_q, or at its own voxel when that link bounced back (DomainView::wall6),
-// so no neighbour id is looked up for it. The phase pass needs only the sum
+// its own phase; the reader finds phi_w in the previous step's phases
+// (DomainView::phi is double-buffered by step parity) at the upstream site
+// x - xi_q, or at its own when that link bounced back. The phase pass needs only the sum
 // of the references over the seven directions, Na = sum_q s_q + (1 + S)/2
 // with S = sum_q w_q phi_w(q) (likewise Nb with -S; the writers' rest values
 // absorb the fp32 weights' excess over 1); the collision, which holds those
@@ -244,35 +244,27 @@ __device__ __forceinline__ int f_ref_read(int n, const int* nb) {
     else return writer_of<Q>(n, nb);
 }
 
-// Phase of the site that wrote the component value read as direction Q by the
-// site at voxel v at a step of parity PAR (fp16 storage, see StoreF16): from
-// the previous step's phase grid, at the upstream voxel x - xi_Q, or at v when
-// x - xi_Q is solid (bit opp(Q) - 1 of the site's wall mask).
+// Phase of the site that wrote the component value read as direction Q by site
+// n at a step of parity PAR (fp16 storage, see StoreF16): from the previous
+// step's phases, at the upstream site x - xi_Q, or at n when x - xi_Q is solid
+// (nb: the face neighbours' ids, negative where there is none).
 template <int PAR, int Q>
-__device__ __forceinline__ float writer_phase(const DomainView& d, int v, unsigned wall) {
-    const float* prev = d.phi[PAR ^ 1];
-    if constexpr (Q == 0) {
-        return prev[v];
-    } else {
-        constexpr int o = opp(Q);
-        return prev[((wall >> (o - 1)) & 1u) ? v : v + stencil_off(d, o)];
-    }
+__device__ __forceinline__ float writer_phase(const DomainView& d, int n, const int* nb) {
+    return d.phi[PAR ^ 1][writer_of<Q>(n, nb)];
 }
 
-// A_q, B_q of site n (voxel v) at a step of parity PAR (nb[1..6]: face
-// neighbours at odd steps).
+// A_q, B_q of site n at a step of parity PAR (nb[1..6]: face neighbours, needed
+// where need_face_nb() says so).
 template <int PAR, class S>
-__device__ __forceinline__ void load_components(const DomainView& d, int n, int v, const int* nb, float (&a)[Q7],
+__device__ __forceinline__ void load_components(const DomainView& d, int n, const int* nb, float (&a)[Q7],
                                                 float (&b)[Q7]) {
-    unsigned wall = 0;
-    if constexpr (S::kRef) wall = __ldg(d.wall6 + n);
     static_for<0, Q7>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
         const size_t i = read_slot<PAR, q>(d, n, nb);
         a[q] = S::template ld_c<q>(d.a, i);
         b[q] = S::template ld_c<q>(d.b, i);
         if constexpr (S::kRef) {
-            const float pw = writer_phase<PAR, q>(d, v, wall);
+            const float pw = writer_phase<PAR, q>(d, n, nb);
             a[q] = fmaf(w7(q) * 0.5f, 1.0f + pw, a[q]);
             b[q] = fmaf(w7(q) * 0.5f, 1.0f - pw, b[q]);
         }
@@ -280,55 +272,43 @@ __device__ __forceinline__ void load_components(const DomainView& d, int n, int 
 }
 
 // fp16 storage: S = sum_q w_q phi_w(q) over the seven component values that
-// site n (voxel v) reads at a step of parity PAR (see writer_phase).
+// site n reads at a step of parity PAR (see writer_phase).
 template <int PAR>
-__device__ __forceinline__ float reference_phase_sum(const DomainView& d, int n, int v) {
-    const unsigned wall = __ldg(d.wall6 + n);
+__device__ __forceinline__ float reference_phase_sum(const DomainView& d, int n) {
+    int nb[Q7];
+    face_neighbours(d, n, nb);
     float S = 0.0f;
     static_for<0, Q7>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        S = fmaf(w7(q), writer_phase<PAR, q>(d, v, wall), S);
+        S = fmaf(w7(q), writer_phase<PAR, q>(d, n, nb), S);
     });
     return S;
 }
 
-// Whether the face-neighbour ids are needed to read the components.
-template <int PAR>
-constexpr bool need_face_nb() { return PAR == 1; }
+// Whether the face-neighbour ids are needed to read or write the components:
+// for their slots at odd steps, for their references with fp16 storage.
+template <int PAR, class S>
+constexpr bool need_face_nb() { return PAR == 1 || S::kRef; }
 
 // ---------------------------------------------------------------------------
-// phase pass: Na, Nb -> phi (dense grid) and N (per site)          Sec. 3.1
+// phase pass: Na, Nb -> phi and N of each site                      Sec. 3.1
 // ---------------------------------------------------------------------------
-// Phase pass of one site (or one periodic halo voxel mirroring a site).
-// Ordering with the neighbouring kernels under programmatic launch: only the
-// static index (site_vox, vsite) is read before wait_prior_grid(); A and B
-// (written by the previous collision) are read, and phi / nsum (read by the
-// previous collision) are written, only after it. Dependents are released
+// Phase pass of one site. Ordering with the neighbouring kernels under
+// programmatic launch: only the static index is read before wait_prior_grid();
+// A and B (written by the previous collision) are read, and phi / nsum (read by
+// the previous collision) are written, only after it. Dependents are released
 // after the wait, so the next collision never starts before the previous
 // one has completed.
 template <int PAR, class S>
-__device__ __forceinline__ void phase_thread(const DomainView& d, int t) {
-    int n = -1, dst = -1;
-    if (t < d.n_sites) {
-        n = t;
-    } else if (t < d.n_sites + d.n_halo) {
-        n = __ldg(d.halo_site + (t - d.n_sites));
-        dst = __ldg(d.halo_dst + (t - d.n_sites));
-    }
-    int v = 0;
-    int nb[7];
-    if (n >= 0) {
-        v = __ldg(d.site_vox + n);
-        if constexpr (need_face_nb<PAR>()) {
-            static_for<1, 7>([&](auto qc) {
-                constexpr int q = decltype(qc)::value;
-                nb[q] = __ldg(d.vsite + v + stencil_off(d, q));
-            });
-        }
+__device__ __forceinline__ void phase_thread(const DomainView& d, int n) {
+    const bool ok = n < d.n_sites;
+    int nb[Q7];
+    if constexpr (PAR == 1) {
+        if (ok) face_neighbours(d, n, nb);
     }
     wait_prior_grid();
     allow_next_grid();
-    if (n < 0) return;
+    if (!ok) return;
     float Na = 0.0f, Nb = 0.0f;
     if constexpr (S::kRef) {
         // stored deviations plus the references' sum, (1 +- rsum)/2 (the
@@ -344,7 +324,7 @@ __device__ __forceinline__ void phase_thread(const DomainView& d, int t) {
         Nb = fmaf(0.5f, 1.0f - Sr, Nb);
     } else {
         float a[Q7], b[Q7];
-        load_components<PAR, S>(d, n, v, nb, a, b);
+        load_components<PAR, S>(d, n, nb, a, b);
         static_for<0, Q7>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
             Na += a[q];
@@ -352,56 +332,35 @@ __device__ __forceinline__ void phase_thread(const DomainView& d, int t) {
         });
     }
     const float Nt = Na + Nb;
-    const float phi = Nt > 0.0f ? (Na - Nb) / Nt : 0.0f;
-    if (dst < 0) {
-        d.phi[PAR][v] = phi;
-        d.nsum[n] = Nt;
-    } else {
-        d.phi[PAR][dst] = phi;    // halo voxel of a periodic face
-    }
+    d.phi[PAR][n] = Nt > 0.0f ? (Na - Nb) / Nt : 0.0f;
+    d.nsum[n] = Nt;
 }
 
 // Phase pass of the sum form: phi (and, for a population-form collision
-// next, N) from the site's component sums, for PER entries per thread
-// (entries t0 + k * stride: sites, then periodic halo voxels). Ordering as in
-// phase_thread: the sums were completed by the collision before the previous
-// phase pass.
+// next, N) from the site's component sums, for PER sites per thread (t0 + k *
+// stride). Ordering as in phase_thread: the sums were completed by the
+// collision before the previous phase pass.
 template <int PAR, bool WRITE_N, int PER>
 __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, int stride) {
     const unsigned long long pol = l2_keep();
-    int n[PER], dst[PER], v[PER];
-    #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int t = t0 + k * stride;
-        n[k] = -1;
-        dst[k] = -1;
-        v[k] = 0;
-        if (t < d.n_sites) {
-            n[k] = t;
-            v[k] = ldg_keep(d.site_vox + t, pol);
-        } else if (t < d.n_sites + d.n_halo) {
-            n[k] = __ldg(d.halo_site + (t - d.n_sites));
-            dst[k] = __ldg(d.halo_dst + (t - d.n_sites));
-        }
-    }
     wait_prior_grid();
     allow_next_grid();
     unsigned long long s[PER];
     #pragma unroll
-    for (int k = 0; k < PER; ++k) s[k] = n[k] >= 0 ? ld_keep(d.acc[PAR] + n[k], pol) : 0ull;
+    for (int k = 0; k < PER; ++k) {
+        const int n = t0 + k * stride;
+        s[k] = n < d.n_sites ? ld_keep(d.acc[PAR] + n, pol) : 0ull;
+    }
     #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        if (n[k] < 0) continue;
+        const int n = t0 + k * stride;
+        if (n >= d.n_sites) continue;
         int a, b;
         unpack_sums(s[k], a, b);
         float Nt, phi;
         sums_phase(a, b, Nt, phi);
-        if (dst[k] < 0) {
-            d.phi[PAR][v[k]] = phi;
-            if constexpr (WRITE_N) d.nsum[n[k]] = Nt;
-        } else {
-            d.phi[PAR][dst[k]] = phi;    // halo voxel of a periodic face
-        }
+        d.phi[PAR][n] = phi;
+        if constexpr (WRITE_N) d.nsum[n] = Nt;
     }
 }
 
@@ -416,106 +375,138 @@ __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, in
 // to, the same slot: row q at the downstream neighbour x + xi_q, or row
 // opp(q) at n itself when that voxel is solid. With fp16 storage both also
 // use the same density reference (that neighbour's density of the last even
-// step, which odd steps do not change). SlotCache keeps the slot (relative to
-// row q, a signed 32-bit offset) of each direction and the references' part
-// of each opposite pair between the gather and the scatter, in shared memory
-// laid out [row][site of the block] so that a warp's accesses fall in
-// distinct banks.
+// step, which odd steps do not change); SlotCache keeps it between the gather
+// and the scatter, in shared memory laid out [row][thread] so that a warp's
+// accesses fall in distinct banks.
+// The neighbours' ids come from the site's record (DENSE = false: every lane's
+// record is regular), formed again from its eight ranks wherever one is used,
+// or from the dense grid of ids (DENSE = true), each looked up once and kept in
+// the slot cache.
 struct SlotCache {
-    int* slot;      // entry of direction 1 of this thread; direction q at slot[(q - 1) * stride]
-                    // (even steps of the sum form: the face neighbour's site id, -1 if solid)
-    float* ref;     // pair p (directions 2p + 1, 2p + 2) at ref[p * stride] (fp16 storage only)
+    int* slot;      // DENSE: entry of direction 1 of this thread, direction q at slot[(q - 1) * stride]:
+                    // the slot relative to row q (odd steps), the face neighbour's site id (even steps
+                    // of the sum form)
+    float* ref;     // the density reference of direction q's slot at ref[(q - 1) * stride] (fp16, odd steps)
     int stride;     // threads per block
+};
+
+// What a site reads before anything is known about its neighbours.
+template <class S>
+struct SiteState {
+    SiteLinks l;
+    float f[Q19];                   // even steps: the populations in the own slots (stored numbers); odd: f[0]
+    float ref = 0.0f;               // fp16: the own slots' reference density (deviation)
+    unsigned long long own = 0;     // sum form from the sums: own Na, Nb
+    float cw[3];                    // the solids' part of twice the colour gradient
 };
 
 // Collision, recoloring and streaming of site n. The arithmetic is written in
 // explicitly rounded operations (no contraction is left to the compiler), so a
 // site's result is the same bit for bit in every kernel this is compiled into.
 //
-// What bounds it: the loads in flight. The kernel is latency-bound at 36
-// resident warps per SM, so the arithmetic is arranged for few instructions
-// (sums and differences over opposite pairs shared by the moments, the
-// equilibrium and the relaxation; the interfacial terms in closed form per
-// direction): 617 (even) and 816 (odd) instructions per site against 726 and
-// 890 in the form that evaluated each direction's terms by itself, 161.2
-// against 165.7 us per step on 3.69 M sites of a 256^3 pack (fp32), 11.3
-// against 11.9 us on 255 k sites. Two sites per thread on fma.rn.f32x2 took 463
-// instructions per site but ran slower (171-177 us): twice the registers left
-// fewer warps to cover the latency.
-template <int PAR, class S, int CF>
-__device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotCache sc) {
+// What bounds it: DRAM at even steps with fp32 storage (6.1 TB/s, 92 % of a
+// plain copy, on 3.69 M sites of a 256^3 pack), elsewhere the latency of the
+// loads, with 32 warps per SM resident, and the instructions (605 and 854 per
+// site at even and odd steps in fp32, 667 and 1093 in fp16). So neighbours come
+// from a 24-byte record per site and the phase is kept per site: against
+// gathering 18 phases and 18 (odd) or 6 site ids from dense voxel grids, where
+// the 32 sites of a warp span about 150 voxels, a warp touches half the cache
+// lines (L1 data-pipe wavefronts per warp 289 -> 175 odd, 171 -> 122 even), and
+// the phase pass needs no site -> voxel map and no scattered stores: 161 -> 146 us
+// per step in fp32, 154 -> 135 in fp16, 7.7 -> 6.3 on 79 k sites. Two sites per
+// thread on fma.rn.f32x2 took 463 instructions per site in an earlier form but
+// ran slower: twice the registers left fewer warps to cover the latency.
+template <int PAR, class S, int CF, bool DENSE>
+__device__ __forceinline__ void collide_site(const DomainView& d, int n, const SiteState<S>& in, SlotCache sc) {
+    SiteLinks l = in.l;
     using T = typename S::T;
     constexpr float K = S::kK;                      // working units: deviations times K
     constexpr float iK = 1.0f / K;
-    const size_t P = static_cast<size_t>(d.pitch);
+    int pitch = d.pitch;
     T* const F = static_cast<T*>(d.f);
     const unsigned long long pol = l2_keep();
-    const int v = CF != 0 ? ldg_keep(d.site_vox + n, pol) : __ldg(d.site_vox + n);
+    const int v = DENSE ? __ldg(d.site_vox + n) : 0;
+    // id of x + xi_q where has(q)
+    auto has = [&](auto qc) { return link_has<decltype(qc)::value>(l); };
+    auto id = [&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        if constexpr (!DENSE) return link_id<q>(n, l);
+        else if constexpr (PAR == 1 || (CF != 0 && q < Q7)) return sc.slot[(q - 1) * sc.stride];
+        else return __ldg(d.vsite + v + stencil_off(d, q));
+    };
+    // slot that direction q is written to (and opp(q) read from) at odd steps, relative to row q
+    auto slot = [&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        if constexpr (DENSE) return sc.slot[(q - 1) * sc.stride];
+        else return has(qc) ? id(qc) : n + (opp(q) - q) * pitch;
+    };
+    // the record and the pitch from here on are values the compiler knows nothing
+    // about: ids, slots and row addresses formed before are formed again instead
+    // of being kept in registers (in the batched kernels, whose views are not
+    // compile-time uniform, keeping them spilled 140-290 bytes per thread and took
+    // 270 / 284 us per step of a 12-job set in fp32 / fp16 against 246 / 229)
+    auto forget_ids = [&] {
+        if constexpr (!DENSE) asm volatile("" : "+r"(l.a.x), "+r"(l.a.y), "+r"(l.a.z), "+r"(l.b.x), "+r"(l.b.y));
+        asm volatile("" : "+r"(l.a.w), "+r"(n), "+r"(pitch));
+    };
 
-    // incoming momentum populations, the stored numbers s_q as they are:
-    // fp32: f_q; fp16: f_q - t_q rho_ref, in units of 1 / K
+    // incoming momentum populations: fp32, the stored f_q; fp16, deviations in
+    // units of 1 / K, at even steps the stored ones (all relative to the site's
+    // own reference density), at odd steps from rest
     float f[Q19];
-    float ref_own = 0.0f;                                     // fp16: K times the reference density of the own slots
-    float ref_sum[9];                                    // fp16, odd steps: K t (ref_q + ref_o) of each pair
-    if constexpr (PAR == 0) {
-        if constexpr (S::kRef) ref_own = d.drho[n];
-        static_for<0, Q19>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;
-            f[q] = S::ld_s(F + q * P + n);
-        });
-    } else {
-        f[0] = S::ld_s(F + n);
-        if constexpr (S::kRef) ref_own = d.drho[n];
-        static_for<0, 9>([&](auto pc) {
-            constexpr int p = decltype(pc)::value;
-            float r[2];
-            static_for<0, 2>([&](auto hc) {
-                constexpr int h = decltype(hc)::value;
-                constexpr int q = 2 * p + 1 + h;     // direction of the downstream slot
-                constexpr int o = opp(q);            // direction read from it
+    static_for<0, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        if constexpr (PAR == 0 || q == 0) f[q] = in.f[q];
+    });
+    const float ref_own = in.ref;
+    if constexpr (PAR == 1) {
+        if constexpr (S::kRef) f[0] = fma(t19(0) * K, ref_own, f[0]);
+        static_for<1, Q19>([&](auto qc) {
+            constexpr int q = decltype(qc)::value;   // direction of the downstream slot
+            constexpr int o = opp(q);                // direction read from it
+            if constexpr (DENSE) {
                 const int m = __ldg(d.vsite + v + stencil_off(d, q));
-                const int s = m >= 0 ? m : n + (o - q) * d.pitch;
-                sc.slot[(q - 1) * sc.stride] = s;
-                f[o] = S::ld_s(F + q * P + s);
-                if constexpr (S::kRef) r[h] = d.drho[m >= 0 ? m : n];
-            });
+                sc.slot[(q - 1) * sc.stride] = m >= 0 ? m : n + (o - q) * pitch;
+            }
+            f[o] = S::ld_s(F + q * static_cast<size_t>(pitch) + slot(qc));
             if constexpr (S::kRef) {
-                // reference of the slot of direction o minus that of direction q, o = q + 1
-                constexpr float tk = t19(2 * p + 1) * K;
-                ref_sum[p] = mul(tk, add(r[0], r[1]));
-                sc.ref[p * sc.stride] = mul(tk, sub(r[1], r[0]));
+                const float r = d.drho[has(qc) ? id(qc) : n];
+                sc.ref[(q - 1) * sc.stride] = r;
+                f[o] = fma(t19(o) * K, r, f[o]);
             }
         });
     }
-    if constexpr (CF != 0 && PAR == 0) {
+    if constexpr (DENSE && CF != 0 && PAR == 0) {
         // sum form, even step: the face neighbours that receive the component values
         static_for<1, Q7>([&](auto qc) {
             constexpr int q = decltype(qc)::value;
             sc.slot[(q - 1) * sc.stride] = __ldg(d.vsite + v + stencil_off(d, q));
         });
     }
-    // sum form from the sums: the site's own Na, Nb (complete before the
-    // previous phase pass, like f)
-    unsigned long long own = 0;
-    if constexpr (CF == 2) own = ld_keep(d.acc[PAR] + n, pol);
+    unsigned long long own = in.own;
+    forget_ids();
+    const float (&cw)[3] = in.cw;
 
-    // Everything above (site and neighbour ids, f and the sums from the
-    // previous collision) is safe to read before the phase pass of this step
+    // Everything above (neighbour ids, f and the sums from the previous
+    // collision) is safe to read before the phase pass of this step
     // completes; phi and nsum are its outputs, and the A/B slots written below
     // are its inputs.
     allow_next_grid();
     wait_prior_grid();
 
-    // colour gradient C = sum_q g_q xi_q phi(x + xi_q) (solids hold phi_s),
-    // g = 1 on faces and 1/2 on edges, from the differences over opposite
-    // neighbours; twice C is what is used below (n does not depend on the scale)
-    const float* const pv = d.phi[PAR] + v;
+    // colour gradient C = sum_q g_q xi_q phi(x + xi_q), g = 1 on faces and 1/2
+    // on edges, from the differences over opposite neighbours plus the solids'
+    // part; twice C is what is used below (n does not depend on the scale)
+    const float* const phi = d.phi[PAR];
+    auto phi_at = [&](auto qc) { return has(qc) ? phi[id(qc)] : 0.0f; };
     float dphi[9];
     static_for<0, 9>([&](auto pc) {
         constexpr int p = decltype(pc)::value;
-        dphi[p] = sub(pv[stencil_off(d, 2 * p + 1)], pv[stencil_off(d, 2 * p + 2)]);
+        const std::integral_constant<int, 2 * p + 1> q;
+        const std::integral_constant<int, 2 * p + 2> o;
+        dphi[p] = sub(phi_at(q), phi_at(o));
     });
-    const float phi_c = *pv;
+    const float phi_c = phi[n];
     float Nt;
     if constexpr (CF == 2) {
         int a, b;
@@ -528,14 +519,11 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
         // references of the values the next phase pass reads at this site: the
         // phase of x - xi_q, which this step writes, or this site's own on a
         // bounce-back link; every face direction has the same weight
-        const unsigned wall = __ldg(d.wall6 + n);
         float Sf = 0.0f;
-        static_for<1, Q7>([&](auto qc) {
-            constexpr int q = decltype(qc)::value;
-            Sf += (wall >> (q - 1)) & 1u ? phi_c : pv[stencil_off(d, q)];
-        });
+        static_for<1, Q7>([&](auto qc) { Sf += has(qc) ? phi[id(qc)] : phi_c; });
         d.rsum[n] = fmaf(w7(1), Sf, w7(0) * phi_c);
     }
+    forget_ids();
 
     // pair sums of deviations S = (f_q - t) + (f_o - t) and differences
     // D = f_q - f_o (both exact or once rounded: f_q - 2t is exact for f near
@@ -548,23 +536,22 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     }
     auto pair_sum = [&](auto pc) {
         constexpr int p = decltype(pc)::value;
-        constexpr int q = 2 * p + 1, o = q + 1, c = p < 3 ? 0 : 1;
+        constexpr int q = 2 * p + 1, o = q + 1;
+        [[maybe_unused]] constexpr int c = p < 3 ? 0 : 1;
         if constexpr (!S::kRef) return add(add(f[q], mt[c]), f[o]);
         else if constexpr (PAR == 0) return add(add(f[q], f[o]), two_ref[c]);
-        else return add(add(f[q], f[o]), ref_sum[p]);
+        else return add(f[q], f[o]);
     };
-    // fp16, odd steps: difference of the references, for D and the results
-    auto pair_ref = [&](auto pc) { return sc.ref[decltype(pc)::value * sc.stride]; };
     auto pair_diff = [&](auto pc) {
         constexpr int q = 2 * decltype(pc)::value + 1;
-        if constexpr (S::kRef && PAR == 1) return add(sub(f[q], f[q + 1]), pair_ref(pc));
-        else return sub(f[q], f[q + 1]);
+        return sub(f[q], f[q + 1]);
     };
     // drho = rho - 1 and j, in working units
     float drho, jx, jy, jz;
     {
         if constexpr (!S::kRef) drho = add(f[0], -t19(0));
-        else drho = fma(t19(0) * K, ref_own, f[0]);
+        else if constexpr (PAR == 0) drho = fma(t19(0) * K, ref_own, f[0]);
+        else drho = f[0];
         float s = pair_sum(std::integral_constant<int, 0>{});
         static_for<1, 9>([&](auto pc) { s = add(s, pair_sum(pc)); });
         drho = add(drho, s);
@@ -580,9 +567,9 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     static_for<1, Q19>([&](auto qc) { asm volatile("" : "+f"(f[decltype(qc)::value])); });
 
     // 2 C, its inverse length (0 where C vanishes) and the normal n
-    const float Cx = add(add(dphi[0], dphi[0]), add(add(dphi[3], dphi[4]), add(dphi[5], dphi[6])));
-    const float Cy = add(add(dphi[1], dphi[1]), add(sub(dphi[3], dphi[4]), add(dphi[7], dphi[8])));
-    const float Cz = add(add(dphi[2], dphi[2]), add(sub(dphi[5], dphi[6]), sub(dphi[7], dphi[8])));
+    const float Cx = add(cw[0], add(add(dphi[0], dphi[0]), add(add(dphi[3], dphi[4]), add(dphi[5], dphi[6]))));
+    const float Cy = add(cw[1], add(add(dphi[1], dphi[1]), add(sub(dphi[3], dphi[4]), add(dphi[7], dphi[8]))));
+    const float Cz = add(cw[2], add(add(dphi[2], dphi[2]), add(sub(dphi[5], dphi[6]), sub(dphi[7], dphi[8]))));
     const float C2 = fma(Cx, Cx, fma(Cy, Cy, mul(Cz, Cz)));
     const float inv = C2 > 0.0f ? rsqrtf(C2) : 0.0f;
 
@@ -650,11 +637,11 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     const float Ux = mul(b_m, add(jx, gx)), Uy = mul(b_m, add(jy, gy)), Uz = mul(b_m, add(jz, gz));
 
     // destination of direction q (q >= 1): row opp(q) at n (even step) or the
-    // cached slot of row q (odd step)
+    // slot of row q it was read from (odd step)
     auto store = [&](auto qc, T* base, float x) {
         constexpr int q = decltype(qc)::value;
-        if constexpr (PAR == 0) S::st_s(base + opp(q) * P + n, x);
-        else S::st_s(base + q * P + sc.slot[(q - 1) * sc.stride], x);
+        if constexpr (PAR == 0) S::st_s(base + opp(q) * static_cast<size_t>(pitch) + n, x);
+        else S::st_s(base + q * static_cast<size_t>(pitch) + slot(qc), x);
     };
 
     // fp16, even steps: the results are relative to this site's new density
@@ -671,7 +658,8 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     float esum;
     static_for<0, 9>([&](auto pc) {
         constexpr int p = decltype(pc)::value;
-        constexpr int q = 2 * p + 1, o = q + 1, c = p < 3 ? 0 : 1;
+        constexpr int q = 2 * p + 1, o = q + 1;
+        [[maybe_unused]] constexpr int c = p < 3 ? 0 : 1;
         float e, u;
         if constexpr (p == 0) { e = add(bF, add(qx, Gx)); u = add(Ux, Ux); }
         if constexpr (p == 1) { e = add(bF, add(qy, Gy)); u = add(Uy, Uy); }
@@ -685,12 +673,18 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
         e = sub(e, pair_sum(pc));
         if constexpr (p == 0) esum = e;
         else esum = add(esum, e);
-        float even, odd = fma(h_m, pair_diff(pc), u);
+        const float odd = fma(h_m, pair_diff(pc), u);
+        float even;
         if constexpr (S::kRef && PAR == 0) even = fma(h_nu, e, moved[c]);
         else even = mul(h_nu, e);
-        if constexpr (S::kRef && PAR == 1) odd = add(odd, pair_ref(pc));
-        store(std::integral_constant<int, q>{}, F, add(f[q], add(even, odd)));
-        store(std::integral_constant<int, o>{}, F, add(f[o], sub(even, odd)));
+        float vq = add(f[q], add(even, odd)), vo = add(f[o], sub(even, odd));
+        if constexpr (S::kRef && PAR == 1) {
+            // relative to the destination's density of the last even step
+            vq = fma(-t19(q) * K, sc.ref[(q - 1) * sc.stride], vq);
+            vo = fma(-t19(q) * K, sc.ref[(o - 1) * sc.stride], vo);
+        }
+        store(std::integral_constant<int, q>{}, F, vq);
+        store(std::integral_constant<int, o>{}, F, vo);
     });
     {
         const float m2 = mul(-2.0f, h_nu);
@@ -699,6 +693,7 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
             r0 = fma(t19(0), rref, r0);
             d.drho[n] = mul(iK, drho);
         }
+        if constexpr (S::kRef && PAR == 1) r0 = fma(-t19(0) * K, ref_own, r0);
         S::st_s(F + n, r0);
     }
 
@@ -735,10 +730,10 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
                 const unsigned long long x = pack_sums(__float2int_rn(q & 1 ? add(PA, dA) : sub(PA, dA)),
                                                        __float2int_rn(q & 1 ? add(PB, dB) : sub(PB, dB)));
                 // receiver: x + xi_q if it is a pore site, else x itself (bounce-back)
-                const int m = sc.slot[(q - 1) * sc.stride];
-                if (static_cast<unsigned>(m) < static_cast<unsigned>(d.n_sites)) {
+                const std::integral_constant<int, q> Q;
+                if (has(Q)) {
                     own -= x;
-                    red_add(acc + m, x, pol);
+                    red_add(acc + id(Q), x, pol);
                 }
             });
         });
@@ -801,6 +796,26 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
     }
 }
 
+// The loads that need no neighbour come first, then one path per warp: through
+// the records if all of them are regular, else through the dense grid of ids.
+template <int PAR, class S, int CF>
+__device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotCache sc) {
+    using T = typename S::T;
+    const size_t P = static_cast<size_t>(d.pitch);
+    const T* const F = static_cast<const T*>(d.f);
+    SiteState<S> in;
+    in.l = SiteLinks{__ldg(d.link_a + n), __ldg(d.link_b + n)};
+    static_for<0, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        if constexpr (PAR == 0 || q == 0) in.f[q] = S::ld_s(F + q * P + n);
+    });
+    if constexpr (S::kRef) in.ref = d.drho[n];
+    if constexpr (CF == 2) in.own = ld_keep(d.acc[PAR] + n, l2_keep());
+    for (int i = 0; i < 3; ++i) in.cw[i] = __ldg(d.wall_c + i * P + n);
+    if (__any_sync(__activemask(), in.l.a.w & kIrregular)) collide_site<PAR, S, CF, true>(d, n, in, sc);
+    else collide_site<PAR, S, CF, false>(d, n, in, sc);
+}
+
 // ---------------------------------------------------------------------------
 // reservoir reset (unsteady protocol, Sec. 4.1): write the rest state into
 // the slots the NEXT step (parity PAR) reads.
@@ -820,7 +835,7 @@ __device__ __forceinline__ void reservoir_thread(const DomainView& d, int n, int
         });
     }
     // fp16: the component references of the next step's reads (see StoreF16)
-    const unsigned wall = S::kRef ? __ldg(d.wall6 + n) : 0u;
+    if constexpr (S::kRef && PAR == 0) face_neighbours(d, n, nb);
     const float rho = side == 1 ? rho_in : rho_out;
     const float na = side == 1 ? 1.0f : 0.0f;
     static_for<0, Q19>([&](auto qc) {
@@ -835,7 +850,7 @@ __device__ __forceinline__ void reservoir_thread(const DomainView& d, int n, int
         if constexpr (q < Q7 && !SUMS) {
             float av = w7(q) * na, bv = w7(q) * (1.0f - na);
             if constexpr (S::kRef) {
-                const float pw = writer_phase<PAR, q>(d, v, wall);
+                const float pw = writer_phase<PAR, q>(d, n, nb);
                 av -= w7(q) * 0.5f * (1.0f + pw);
                 bv -= w7(q) * 0.5f * (1.0f - pw);
             }
@@ -942,7 +957,8 @@ __device__ __forceinline__ void pressure_face_thread(const DomainView& d, int n,
             float av = side == 1 ? eq : 0.0f, bv = side == 1 ? 0.0f : eq;
             if constexpr (S::kRef) {
                 // the reference the next step reads it with (see StoreF16)
-                const float pw = writer_phase<PAR, q>(d, d.site_vox[n], __ldg(d.wall6 + n));
+                if constexpr (PAR == 0) face_neighbours(d, n, nb);
+                const float pw = writer_phase<PAR, q>(d, n, nb);
                 av -= w7(q) * 0.5f * (1.0f + pw);
                 bv -= w7(q) * 0.5f * (1.0f - pw);
             }
