@@ -116,7 +116,7 @@ lbpm_status alloc_state(lbpm_ctx* c) {
     c->d_b = dalloc(c, state_bytes(c, 7));
     const size_t P = static_cast<size_t>(pitch_of(c->N));
     c->d_nsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
-    c->d_acc = static_cast<unsigned long long*>(dalloc(c, sizeof(unsigned long long) * 2 * P));
+    c->d_acc = static_cast<unsigned long long*>(dalloc(c, sizeof(unsigned long long) * P));
     c->d_phi = static_cast<float*>(dalloc(c, sizeof(float) * P));
     bool ok = c->d_f && c->d_a && c->d_b && c->d_nsum && c->d_acc && c->d_phi;
     if (c->params.precision == LBPM_FP16) {
@@ -236,12 +236,12 @@ enum StepKind { kStepPop = 0, kStepSumFirst = 1, kStepSumMid = 2, kStepSumLast =
 
 // The two kernels of one timestep of the given kind.
 cudaError_t launch_step_phase(lbpm_ctx* c, int kind, int par, cudaStream_t s) {
-    if (kind == kStepPop || kind == kStepSumFirst) return launch_phase(c, par, s);
-    return launch_phase_sum(c, par, kind == kStepSumLast, s);
+    if (kind == kStepPop || kind == kStepSumFirst) return launch_phase(c, par, kind == kStepSumFirst, s);
+    return launch_phase_sum(c, par, s);
 }
 cudaError_t launch_step_collide(lbpm_ctx* c, int kind, int par, cudaStream_t s) {
     if (kind == kStepPop || kind == kStepSumLast) return launch_collide(c, par, s);
-    return launch_collide_sum(c, par, kind == kStepSumMid, s);
+    return launch_collide_sum(c, par, s);
 }
 // The boundary kernel after the collision of a step of the given kind (reservoir
 // slabs, pressure faces); it writes what the next step (parity par ^ 1) reads.
@@ -253,7 +253,7 @@ cudaError_t launch_step_boundary(lbpm_ctx* c, int kind, int par, cudaStream_t s)
 
 // One timestep: phase pass, fused collide-stream, reservoir reset.
 cudaError_t enqueue_step(lbpm_ctx* c, int par, cudaStream_t s) {
-    cudaError_t e = launch_phase(c, par, s);
+    cudaError_t e = launch_phase(c, par, false, s);
     if (e == cudaSuccess) e = launch_collide(c, par, s);
     if (e == cudaSuccess && c->n_slab) e = launch_reservoir(c, par ^ 1, s);
     return e;
@@ -319,11 +319,6 @@ namespace lbm {
 
 bool sum_form_capable(const lbpm_ctx* c) {
     return c->step_form == LBPM_STEP_AUTO && c->params.reservoir_z <= 1 && c->d_acc != nullptr;
-}
-
-cudaError_t clear_sums(const lbpm_ctx* c, int par, cudaStream_t s) {
-    return cudaMemsetAsync(c->d_acc + static_cast<size_t>(par) * static_cast<size_t>(pitch_of(c->N)), 0,
-                           sizeof(unsigned long long) * static_cast<size_t>(c->N), s);
 }
 
 void* dalloc(lbpm_ctx* c, size_t bytes) {
@@ -640,12 +635,11 @@ lbpm_status plain_step(lbpm_ctx* c, int kind) {
     return LBPM_OK;
 }
 
-// lbpm_advance in the sum form (nsteps >= 2, no reservoirs): the first step
-// reads the populations, the middle steps carry the components as per-site
+// lbpm_advance in the sum form (nsteps >= 2): the first step reads the
+// populations and sets the sums, the middle steps carry the components as per-site
 // sums (replayed from CUDA graphs in bundles of 16 and 2), the last step
 // writes the populations again.
 lbpm_status advance_sum(lbpm_ctx* c, long long nsteps) {
-    LBPM_CK(c, clear_sums(c, static_cast<int>((c->step + 1) & 1), c->stream));
     lbpm_status st = plain_step(c, kStepSumFirst);
     if (st) return st;
     long long mid = nsteps - 2;
@@ -719,7 +713,7 @@ lbpm_status lbpm_advance(lbpm_ctx* c, long long nsteps) {
             e3 = next_event(c);
         }
         if (e0 >= 0) cudaEventRecord(c->ev_pool[e0], c->stream);
-        LBPM_CK(c, launch_phase(c, par, c->stream));
+        LBPM_CK(c, launch_phase(c, par, false, c->stream));
         if (e1 >= 0) cudaEventRecord(c->ev_pool[e1], c->stream);
         if (e2 >= 0) cudaEventRecord(c->ev_pool[e2], c->stream);
         LBPM_CK(c, launch_collide(c, par, c->stream));

@@ -50,25 +50,25 @@ __device__ __forceinline__ int job_of_tile(const BatchLaunch& p, int t) {
     return lo;
 }
 
-template <int PAR, class S, int BT>
+template <int PAR, class S, bool SUMS, int BT>
 __global__ void __launch_bounds__(BT) k_batch_phase(const __grid_constant__ BatchLaunch p) {
     const int nt = p.tile_begin[p.n_jobs];
     for (int t = blockIdx.x; t < nt; t += gridDim.x) {
         const int j = job_of_tile(p, t);
         const int i0 = (t - p.tile_begin[j]) * BT * kBatchPhasePer + static_cast<int>(threadIdx.x);
 #pragma unroll
-        for (int k = 0; k < kBatchPhasePer; ++k) phase_thread<PAR, S>(p.v[j], i0 + k * BT);
+        for (int k = 0; k < kBatchPhasePer; ++k) phase_thread<PAR, S, SUMS>(p.v[j], i0 + k * BT);
     }
 }
 
 // Phase pass of the sum form (see phase_sum_thread), kBatchPhasePer entries
 // per thread.
-template <int PAR, bool WRITE_N, int BT>
+template <int PAR, int BT>
 __global__ void __launch_bounds__(BT) k_batch_phase_sum(const __grid_constant__ BatchLaunch p) {
     const int nt = p.tile_begin[p.n_jobs];
     for (int t = blockIdx.x; t < nt; t += gridDim.x) {
         const int j = job_of_tile(p, t);
-        phase_sum_thread<PAR, WRITE_N, kBatchPhasePer>(
+        phase_sum_thread<PAR, kBatchPhasePer>(
             p.v[j], (t - p.tile_begin[j]) * BT * kBatchPhasePer + static_cast<int>(threadIdx.x), BT);
     }
 }
@@ -108,16 +108,18 @@ struct Launch {
     }
 };
 
-// phase pass: form 0 = populations, 1 = sums, 2 = sums writing N (last step of a run)
+// phase pass: form 0 = populations, 1 = sums, 2 = populations setting the sums (first step of a run)
 template <int BT, int PAR>
 cudaError_t batch_phase_par(int form, bool fp16, unsigned grid, cudaStream_t s, const BatchLaunch& p) {
-    if (form == 1) return Launch<BT>::go(k_batch_phase_sum<PAR, false, BT>, grid, s, p);
-    if (form == 2) return Launch<BT>::go(k_batch_phase_sum<PAR, true, BT>, grid, s, p);
-    return fp16 ? Launch<BT>::go(k_batch_phase<PAR, StoreF16, BT>, grid, s, p)
-                : Launch<BT>::go(k_batch_phase<PAR, StoreF32, BT>, grid, s, p);
+    if (form == 1) return Launch<BT>::go(k_batch_phase_sum<PAR, BT>, grid, s, p);
+    if (form == 2)
+        return fp16 ? Launch<BT>::go(k_batch_phase<PAR, StoreF16, true, BT>, grid, s, p)
+                    : Launch<BT>::go(k_batch_phase<PAR, StoreF32, true, BT>, grid, s, p);
+    return fp16 ? Launch<BT>::go(k_batch_phase<PAR, StoreF16, false, BT>, grid, s, p)
+                : Launch<BT>::go(k_batch_phase<PAR, StoreF32, false, BT>, grid, s, p);
 }
 
-// collision: form = component form CF (0 populations, 1 / 2 sums)
+// collision: form = component form CF (0 populations, 1 sums)
 template <int BT, int PAR, int CF>
 cudaError_t batch_collide_cf(bool fp16, unsigned grid, cudaStream_t s, const BatchLaunch& p) {
     return fp16 ? Launch<BT>::go(k_batch_collide<PAR, StoreF16, CF, BT>, grid, s, p)
@@ -125,9 +127,7 @@ cudaError_t batch_collide_cf(bool fp16, unsigned grid, cudaStream_t s, const Bat
 }
 template <int BT, int PAR>
 cudaError_t batch_collide_par(int form, bool fp16, unsigned grid, cudaStream_t s, const BatchLaunch& p) {
-    if (form == 1) return batch_collide_cf<BT, PAR, 1>(fp16, grid, s, p);
-    if (form == 2) return batch_collide_cf<BT, PAR, 2>(fp16, grid, s, p);
-    return batch_collide_cf<BT, PAR, 0>(fp16, grid, s, p);
+    return form == 1 ? batch_collide_cf<BT, PAR, 1>(fp16, grid, s, p) : batch_collide_cf<BT, PAR, 0>(fp16, grid, s, p);
 }
 
 template <int BT>
@@ -213,9 +213,9 @@ int batch_max_blocks(int kernel, bool fp16, int bt) {
     int nb = 0;
     const void* f = nullptr;
 #define LBPM_PICK(BT)                                                                                        \
-    f = kernel == 0 ? (fp16 ? (const void*)k_batch_phase<1, StoreF16, BT> : (const void*)k_batch_phase<1, StoreF32, BT>) \
-                    : (fp16 ? (const void*)k_batch_collide<1, StoreF16, 2, BT>                                \
-                            : (const void*)k_batch_collide<1, StoreF32, 2, BT>);
+    f = kernel == 0 ? (fp16 ? (const void*)k_batch_phase<1, StoreF16, false, BT> : (const void*)k_batch_phase<1, StoreF32, false, BT>) \
+                    : (fp16 ? (const void*)k_batch_collide<1, StoreF16, 1, BT>                                \
+                            : (const void*)k_batch_collide<1, StoreF32, 1, BT>);
     if (bt == 128) { LBPM_PICK(128) } else if (bt == 192) { LBPM_PICK(192) } else if (bt == 512) { LBPM_PICK(512) } else { LBPM_PICK(256) }
 #undef LBPM_PICK
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, bt, 0) != cudaSuccess) {

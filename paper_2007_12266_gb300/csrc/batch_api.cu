@@ -230,12 +230,9 @@ enum BatchStep { kBPop = 0, kBSumFirst = 1, kBSumMid = 2, kBSumLast = 3 };
 cudaError_t enqueue_step(lbpm_batch* b, int kind, int par, cudaStream_t s) {
     const bool h = b->precision == LBPM_FP16;
     // kernel forms (see launch_batch) of each kind: phase pass, collision
-    const int phase_form[4] = {0, 0, 1, 2};
-    const int collide_form[4] = {0, 1, 2, 0};
+    const int phase_form[4] = {0, 2, 1, 1};
+    const int collide_form[4] = {0, 1, 1, 0};
     cudaError_t e = cudaSuccess;
-    if (kind == kBSumFirst)
-        for (lbpm_ctx* c : b->jobs)
-            if (e == cudaSuccess) e = clear_sums(c, par ^ 1, s);
     for (size_t i = 0; i < b->launch[0].size() && e == cudaSuccess; ++i) {
         e = launch_batch(0, phase_form[kind], par, h, b->bt, grid_for(b, 0, b->launch[0][i]), s, b->launch[0][i]);
         if (e == cudaSuccess)

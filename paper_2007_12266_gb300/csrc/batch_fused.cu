@@ -102,14 +102,14 @@ __device__ __forceinline__ void fused_pass(const FusedLaunch& p, int pass, const
 }
 
 // Forms of each pass by kind of step (as in the graph path): the phase pass
-// 0 = populations, 1 = sums, 2 = sums writing N; the collision's component
-// form CF; the reservoir reset writing sums or populations.
+// from the sums, or from the populations (setting the sums at the first step of
+// a run); the collision's component form CF; the reservoir reset writing sums
+// or populations.
 template <int KIND>
 struct FusedKind {
-    static constexpr int kPhase = KIND == kFusedSumMid ? 1 : (KIND == kFusedSumLast ? 2 : 0);
-    static constexpr int kCollide = KIND == kFusedSumFirst ? 1 : (KIND == kFusedSumMid ? 2 : 0);
-    static constexpr bool kClearTargets = KIND == kFusedSumFirst;
-    static constexpr bool kResetSums = KIND == kFusedSumFirst || KIND == kFusedSumMid;
+    static constexpr bool kPhaseSums = KIND == kFusedSumMid || KIND == kFusedSumLast;
+    static constexpr int kCollide = KIND == kFusedSumFirst || KIND == kFusedSumMid ? 1 : 0;
+    static constexpr bool kResetSums = kCollide == 1;
 };
 
 // NS timesteps of the given kind, the first at parity PAR0.
@@ -124,25 +124,18 @@ __global__ void __launch_bounds__(BT, 1024 / BT) k_batch_fused(const __grid_cons
     static_for<0, NS>([&](auto kc) {
         constexpr int PAR = PAR0 ^ (decltype(kc)::value & 1);
         if (!go) return;
-        // phase pass (and, at the first step of a sum-form run, clearing the
-        // sums the collision accumulates into)
-        // (fused_phase_per(BT) independent entries per thread: the pass is
-        // latency-bound, and the fused kernel runs fewer warps than the
+        // phase pass (fused_phase_per(BT) independent entries per thread: the pass
+        // is latency-bound, and the fused kernel runs fewer warps than the
         // separate phase kernel because it holds the collision's registers)
         fused_pass(p, pass++, p.tiles[0], [&](int j, int tj) {
             const DomainView& d = p.v[j];
             constexpr int PER = fused_phase_per(BT);
             const int i0 = tj * BT * PER + static_cast<int>(threadIdx.x);
-            if constexpr (K::kPhase == 0) {
+            if constexpr (!K::kPhaseSums) {
                 #pragma unroll
-                for (int k = 0; k < PER; ++k) phase_thread<PAR, S>(d, i0 + k * BT);
+                for (int k = 0; k < PER; ++k) phase_thread<PAR, S, KIND == kFusedSumFirst>(d, i0 + k * BT);
             } else {
-                phase_sum_thread<PAR, K::kPhase == 2, PER>(d, i0, BT);
-            }
-            if constexpr (K::kClearTargets) {
-                #pragma unroll
-                for (int k = 0; k < PER; ++k)
-                    if (i0 + k * BT < d.n_sites) d.acc[PAR ^ 1][i0 + k * BT] = 0ull;
+                phase_sum_thread<PAR, PER>(d, i0, BT);
             }
         });
         go = grid_barrier(p.ctl, p.err, nblocks, p.limit_ns);

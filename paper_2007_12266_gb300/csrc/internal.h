@@ -57,8 +57,7 @@ struct DomainView {
     void* f;               // [19][P] momentum distributions (AA in place)
     void* a;               // [7][P]  component A
     void* b;               // [7][P]  component B
-    unsigned long long* acc[2];  // [N] sum form: packed fixed-point (Na, Nb) of each site at the step of
-                                 //     parity p, accumulated by the previous collision (see pack_sums)
+    unsigned long long* acc;     // [N] sum form: packed fixed-point (Na, Nb) of each site (see pack_sums)
     float tau_a, tau_b, alpha, beta;
     float fx, fy, fz;
     float fs[3];           // F / s_m when tau_a == tau_b, in the collision's working units (times 2^14
@@ -119,7 +118,7 @@ struct lbpm_ctx {
     void* d_f = nullptr;
     void* d_a = nullptr;
     void* d_b = nullptr;
-    unsigned long long* d_acc = nullptr;   // [2N] sum form: packed component sums by step parity
+    unsigned long long* d_acc = nullptr;   // [N] sum form: packed component sums
     int step_form = LBPM_STEP_AUTO;        // lbpm_set_step_form
     int* d_slab_site = nullptr;     // reservoir sites
     signed char* d_slab_side = nullptr;
@@ -170,23 +169,21 @@ cudaError_t noalloc_setup(int device);
 DomainView make_view(const lbpm_ctx* c);
 cudaError_t launch_init_fluids(const lbpm_ctx* c, const float* phi0, cudaStream_t s);
 cudaError_t launch_ref_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
-cudaError_t launch_phase(const lbpm_ctx* c, int parity, cudaStream_t s);
+// Phase pass from the populations (sums: also set the component sums, for a
+// collision of the sum form next) and the collision storing populations.
+cudaError_t launch_phase(const lbpm_ctx* c, int parity, bool sums, cudaStream_t s);
 cudaError_t launch_collide(const lbpm_ctx* c, int parity, cudaStream_t s);
 // Sum form of a timestep (components carried as per-site sums, see pack_sums):
-// phase pass from the sums (write_nsum: also Na + Nb for a population-form
-// collision), and the collision scattering its recolored values into the
-// receivers' sums (from_sums: the site's own Na, Nb come from its sums,
-// otherwise from the phase pass of the population form).
-cudaError_t launch_phase_sum(const lbpm_ctx* c, int parity, bool write_nsum, cudaStream_t s);
-cudaError_t launch_collide_sum(const lbpm_ctx* c, int parity, bool from_sums, cudaStream_t s);
+// phase pass from the sums, and the collision moving its recolored values
+// between the sums.
+cudaError_t launch_phase_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
+cudaError_t launch_collide_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
 // Reservoir slabs (reservoir_z = 1) in the sum form: the reset state goes into
 // the sums the next step (parity `parity`) reads, and into its f slots.
 cudaError_t launch_reservoir_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
 // Whether a context can run the sum form (no pressure or flux faces, the
 // population form not forced).
 bool sum_form_capable(const lbpm_ctx* c);
-// Clear the sums that the first step of a sum-form run (parity `par`) accumulates into.
-cudaError_t clear_sums(const lbpm_ctx* c, int par, cudaStream_t s);
 cudaError_t launch_reservoir(const lbpm_ctx* c, int parity, cudaStream_t s);
 // flux inlet: blocks of the fixed-order face reduction
 constexpr int kFaceBlocks = 64;
@@ -215,8 +212,8 @@ struct BatchLaunch {
     int tile_begin[kBatchLaunchJobs + 1];
     DomainView v[kBatchLaunchJobs];
 };
-// form: phase pass 0 = populations, 1 = sums, 2 = sums writing N; collision
-// 0 = populations, 1 = sums from the phase pass, 2 = sums from the sums.
+// form: phase pass 0 = populations, 1 = sums, 2 = populations setting the sums;
+// collision 0 = populations, 1 = sums.
 cudaError_t launch_batch(int kernel, int form, int par, bool fp16, int bt, unsigned grid, cudaStream_t s,
                          const BatchLaunch& p);
 cudaError_t launch_batch_measure(bool fp16, unsigned grid, cudaStream_t s, const DomainView* v, const int* parity,

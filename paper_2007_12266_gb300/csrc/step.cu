@@ -28,17 +28,17 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, cudaStream_t s, 
     return launch_pdl_bt(kernel, grid, kBlock, s, args...);
 }
 
-template <int PAR, class S>
+template <int PAR, class S, bool SUMS>
 __global__ void __launch_bounds__(kBlock) k_phase(DomainView d) {
     const int t = blockIdx.x * kBlock + threadIdx.x;
-    phase_thread<PAR, S>(d, t);
+    phase_thread<PAR, S, SUMS>(d, t);
 }
 
-constexpr int kPhaseSumPer = 2;   // entries per thread of the sum-form phase pass (1, 2, 4, 8 measured; 2 fastest)
+constexpr int kPhaseSumPer = 2;   // sites per thread of the sum-form phase pass (1, 2, 4, 8 measured; 2 fastest)
 
-template <int PAR, bool WRITE_N>
+template <int PAR>
 __global__ void __launch_bounds__(kBlock) k_phase_sum(DomainView d) {
-    phase_sum_thread<PAR, WRITE_N, kPhaseSumPer>(d, blockIdx.x * kBlock * kPhaseSumPer + threadIdx.x, kBlock);
+    phase_sum_thread<PAR, kPhaseSumPer>(d, blockIdx.x * kBlock * kPhaseSumPer + threadIdx.x, kBlock);
 }
 
 // Launch shape of the collision: 64 registers and 32 resident warps per SM.
@@ -211,8 +211,7 @@ DomainView make_view(const lbpm_ctx* c) {
     d.f = c->d_f;
     d.a = c->d_a;
     d.b = c->d_b;
-    d.acc[0] = c->d_acc;
-    d.acc[1] = c->d_acc ? c->d_acc + d.pitch : nullptr;
+    d.acc = c->d_acc;
     const lbpm_params& p = c->params;
     d.tau_a = static_cast<float>(p.tau_a);
     d.tau_b = static_cast<float>(p.tau_b);
@@ -253,13 +252,18 @@ cudaError_t launch_ref_sum(const lbpm_ctx* c, int parity, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_phase(const lbpm_ctx* c, int parity, cudaStream_t s) {
-    DomainView d = make_view(c);
+template <class S, bool SUMS>
+cudaError_t launch_phase_form(const lbpm_ctx* c, int parity, cudaStream_t s) {
     const unsigned g = blocks_for(c->N);
     if (g == 0) return cudaSuccess;
-    const bool h = c->params.precision == LBPM_FP16;
-    if (parity == 0) return h ? launch_pdl(k_phase<0, StoreF16>, g, s, d) : launch_pdl(k_phase<0, StoreF32>, g, s, d);
-    return h ? launch_pdl(k_phase<1, StoreF16>, g, s, d) : launch_pdl(k_phase<1, StoreF32>, g, s, d);
+    DomainView d = make_view(c);
+    return parity == 0 ? launch_pdl(k_phase<0, S, SUMS>, g, s, d) : launch_pdl(k_phase<1, S, SUMS>, g, s, d);
+}
+
+cudaError_t launch_phase(const lbpm_ctx* c, int parity, bool sums, cudaStream_t s) {
+    if (c->params.precision == LBPM_FP16)
+        return sums ? launch_phase_form<StoreF16, true>(c, parity, s) : launch_phase_form<StoreF16, false>(c, parity, s);
+    return sums ? launch_phase_form<StoreF32, true>(c, parity, s) : launch_phase_form<StoreF32, false>(c, parity, s);
 }
 
 // one collision launch of the given parity, storage and component form
@@ -279,16 +283,14 @@ cudaError_t launch_collide(const lbpm_ctx* c, int parity, cudaStream_t s) {
     return parity == 0 ? launch_collide_form<0, 0>(c, s) : launch_collide_form<1, 0>(c, s);
 }
 
-cudaError_t launch_phase_sum(const lbpm_ctx* c, int parity, bool write_nsum, cudaStream_t s) {
-    DomainView d = make_view(c);
+cudaError_t launch_phase_sum(const lbpm_ctx* c, int parity, cudaStream_t s) {
     const unsigned g = blocks_for((c->N + kPhaseSumPer - 1) / kPhaseSumPer);
     if (g == 0) return cudaSuccess;
-    if (parity == 0) return write_nsum ? launch_pdl(k_phase_sum<0, true>, g, s, d) : launch_pdl(k_phase_sum<0, false>, g, s, d);
-    return write_nsum ? launch_pdl(k_phase_sum<1, true>, g, s, d) : launch_pdl(k_phase_sum<1, false>, g, s, d);
+    DomainView d = make_view(c);
+    return parity == 0 ? launch_pdl(k_phase_sum<0>, g, s, d) : launch_pdl(k_phase_sum<1>, g, s, d);
 }
 
-cudaError_t launch_collide_sum(const lbpm_ctx* c, int parity, bool from_sums, cudaStream_t s) {
-    if (from_sums) return parity == 0 ? launch_collide_form<0, 2>(c, s) : launch_collide_form<1, 2>(c, s);
+cudaError_t launch_collide_sum(const lbpm_ctx* c, int parity, cudaStream_t s) {
     return parity == 0 ? launch_collide_form<0, 1>(c, s) : launch_collide_form<1, 1>(c, s);
 }
 

@@ -151,9 +151,11 @@ __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol
 // The recolored populations of Eqs. LBE-mass-a/b are a function of the
 // writing site's Na, Nb, velocity and colour normal, and the next step uses
 // the populations a site receives only through their sums Na, Nb. In the sum
-// form the collision adds each recolored value A*_q, B*_q straight into the
-// sums of the site that receives it (x + xi_q, or x itself on a bounce-back
-// link). A site's (Na, Nb) is one 64-bit word: Na in the high and Nb in the
+// form the collision moves each recolored value A*_q, B*_q from the sums of its
+// site to the sums of the site that receives it, x + xi_q (on a bounce-back link
+// it stays). The sums are updated in place: the collision itself reads N and phi,
+// which the phase pass formed from them, and only adds to them. A site's (Na, Nb)
+// is one 64-bit word: Na in the high and Nb in the
 // low 32 bits, each in units of 2^-28 (|N| < 8). Adding packed words adds both
 // halves exactly as long as the low sum stays within 32 bits, and integer sums
 // do not depend on the order of the additions, so the result is deterministic
@@ -171,17 +173,15 @@ __device__ __forceinline__ void unpack_sums(unsigned long long s, int& a, int& b
 }
 // N = Na + Nb and phi = (Na - Nb)/(Na + Nb) of a site from its sums, in fp32
 // (32-bit integer to float conversions: a 64-bit conversion runs on the fp64
-// pipe, which is slow on this GPU); the phase pass and the collision both use
-// this function, so they agree bit for bit.
+// pipe, which is slow on this GPU).
 __device__ __forceinline__ void sums_phase(int a, int b, float& Nt, float& phi) {
     const float fa = static_cast<float>(a), fb = static_cast<float>(b);
     const float nt = fa + fb;
     Nt = nt * kSumInv;
     phi = nt > 0.0f ? (fa - fb) / nt : 0.0f;
 }
-// The sums and the site -> voxel map (8 + 4 bytes per site, read by the phase
-// pass and again by the collision) are accessed with an L2 evict-last policy,
-// so that they stay in L2 between the two kernels while the populations
+// The sums (8 bytes per site, touched by both kernels of every step) are accessed
+// with an L2 evict-last policy, so that they stay in L2 while the populations
 // stream through it.
 __device__ __forceinline__ unsigned long long l2_keep() {
     unsigned long long pol;
@@ -198,11 +198,6 @@ __device__ __forceinline__ unsigned long long ld_keep(const unsigned long long* 
 }
 __device__ __forceinline__ void st_keep(unsigned long long* p, unsigned long long v, unsigned long long pol) {
     asm volatile("st.global.L2::cache_hint.u64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol) : "memory");
-}
-__device__ __forceinline__ int ldg_keep(const int* p, unsigned long long pol) {
-    int v;
-    asm("ld.global.nc.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
-    return v;
 }
 
 // ---------------------------------------------------------------------------
@@ -299,7 +294,9 @@ constexpr bool need_face_nb() { return PAR == 1 || S::kRef; }
 // the previous collision) are written, only after it. Dependents are released
 // after the wait, so the next collision never starts before the previous
 // one has completed.
-template <int PAR, class S>
+// SUMS: the first step of a run of the sum form, whose collision finds the
+// site's sums set to its Na, Nb.
+template <int PAR, class S, bool SUMS = false>
 __device__ __forceinline__ void phase_thread(const DomainView& d, int n) {
     const bool ok = n < d.n_sites;
     int nb[Q7];
@@ -332,15 +329,21 @@ __device__ __forceinline__ void phase_thread(const DomainView& d, int n) {
         });
     }
     const float Nt = Na + Nb;
-    d.phi[PAR][n] = Nt > 0.0f ? (Na - Nb) / Nt : 0.0f;
+    const float phi = Nt > 0.0f ? (Na - Nb) / Nt : 0.0f;
+    d.phi[PAR][n] = phi;
     d.nsum[n] = Nt;
+    if constexpr (SUMS) {
+        const float half = mul(0.5f * kSumOne, Nt);
+        st_keep(d.acc + n,
+                pack_sums(__float2int_rn(mul(half, add(1.0f, phi))), __float2int_rn(mul(half, sub(1.0f, phi)))),
+                l2_keep());
+    }
 }
 
-// Phase pass of the sum form: phi (and, for a population-form collision
-// next, N) from the site's component sums, for PER sites per thread (t0 + k *
-// stride). Ordering as in phase_thread: the sums were completed by the
-// collision before the previous phase pass.
-template <int PAR, bool WRITE_N, int PER>
+// Phase pass of the sum form: phi and N from the site's component sums, for
+// PER sites per thread (t0 + k * stride). Ordering as in phase_thread: the sums
+// were completed by the collision before.
+template <int PAR, int PER>
 __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, int stride) {
     const unsigned long long pol = l2_keep();
     wait_prior_grid();
@@ -349,7 +352,7 @@ __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, in
     #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int n = t0 + k * stride;
-        s[k] = n < d.n_sites ? ld_keep(d.acc[PAR] + n, pol) : 0ull;
+        s[k] = n < d.n_sites ? ld_keep(d.acc + n, pol) : 0ull;
     }
     #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -360,7 +363,7 @@ __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, in
         float Nt, phi;
         sums_phase(a, b, Nt, phi);
         d.phi[PAR][n] = phi;
-        if constexpr (WRITE_N) d.nsum[n] = Nt;
+        d.nsum[n] = Nt;
     }
 }
 
@@ -368,9 +371,8 @@ __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, in
 // fused collide + stream                                            Sec. 3.1
 // ---------------------------------------------------------------------------
 // Component forms of the collision (CF): 0 stores the recolored populations
-// (AA slots); 1 and 2 add them into the receivers' sums (sum form), with the
-// site's own Na, Nb taken from the phase pass (1, first step of a run) or
-// from its own sums (2).
+// (AA slots); 1 moves them between the sites' sums (sum form). Both take Na, Nb
+// from the phase pass, as N and phi.
 // At an odd step site n reads direction opp(q) from, and writes direction q
 // to, the same slot: row q at the downstream neighbour x + xi_q, or row
 // opp(q) at n itself when that voxel is solid. With fp16 storage both also
@@ -396,7 +398,6 @@ struct SiteState {
     SiteLinks l;
     float f[Q19];                   // even steps: the populations in the own slots (stored numbers); odd: f[0]
     float ref = 0.0f;               // fp16: the own slots' reference density (deviation)
-    unsigned long long own = 0;     // sum form from the sums: own Na, Nb
     float cw[3];                    // the solids' part of twice the colour gradient
 };
 
@@ -404,18 +405,21 @@ struct SiteState {
 // explicitly rounded operations (no contraction is left to the compiler), so a
 // site's result is the same bit for bit in every kernel this is compiled into.
 //
-// What bounds it: DRAM at even steps with fp32 storage (6.1 TB/s, 92 % of a
-// plain copy, on 3.69 M sites of a 256^3 pack), elsewhere the latency of the
-// loads, with 32 warps per SM resident, and the instructions (605 and 854 per
-// site at even and odd steps in fp32, 667 and 1093 in fp16). So neighbours come
-// from a 24-byte record per site and the phase is kept per site: against
-// gathering 18 phases and 18 (odd) or 6 site ids from dense voxel grids, where
-// the 32 sites of a warp span about 150 voxels, a warp touches half the cache
-// lines (L1 data-pipe wavefronts per warp 289 -> 175 odd, 171 -> 122 even), and
-// the phase pass needs no site -> voxel map and no scattered stores: 161 -> 146 us
-// per step in fp32, 154 -> 135 in fp16, 7.7 -> 6.3 on 79 k sites. Two sites per
-// thread on fma.rn.f32x2 took 463 instructions per site in an earlier form but
-// ran slower: twice the registers left fewer warps to cover the latency.
+// What bounds it: DRAM with fp32 storage (live, 202 B per site at 5.9 TB/s at even
+// and 5.4 TB/s at odd steps, of 6.7 for a plain copy, on 3.69 M sites of a 256^3
+// pack), with fp16 the latency of the loads, with 32 warps per SM resident, and
+// the instructions (595 and 785 per site at even and odd steps in fp32, 651 and
+// 972 in fp16). So neighbours come from a 24-byte record per site and the phase
+// is kept per site: against gathering 18 phases and 18 (odd) or 6 site ids from
+// dense voxel grids, where the 32 sites of a warp span about 150 voxels, a warp
+// touches half the cache lines (L1 data-pipe wavefronts per warp 289 -> 175 odd,
+// 171 -> 122 even), and the phase pass needs no site -> voxel map and no
+// scattered stores: 161 -> 146 us per step in fp32, 154 -> 135 in fp16, 7.7 ->
+// 6.3 on 79 k sites. And the component sums are updated in place, in one array
+// that stays in L2 instead of two of which the collision reads one and clears it:
+// 143 -> 136 us in fp32 (15 B per site less from DRAM), 135 -> 131 in fp16. Two
+// sites per thread on fma.rn.f32x2 took 463 instructions per site in an earlier
+// form but ran slower: twice the registers left fewer warps to cover the latency.
 template <int PAR, class S, int CF, bool DENSE>
 __device__ __forceinline__ void collide_site(const DomainView& d, int n, const SiteState<S>& in, SlotCache sc) {
     SiteLinks l = in.l;
@@ -483,12 +487,10 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
             sc.slot[(q - 1) * sc.stride] = __ldg(d.vsite + v + stencil_off(d, q));
         });
     }
-    unsigned long long own = in.own;
     forget_ids();
     const float (&cw)[3] = in.cw;
 
-    // Everything above (neighbour ids, f and the sums from the previous
-    // collision) is safe to read before the phase pass of this step
+    // Everything above (neighbour ids and f from the previous collision) is safe to read before the phase pass of this step
     // completes; phi and nsum are its outputs, and the A/B slots written below
     // are its inputs.
     allow_next_grid();
@@ -507,14 +509,7 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
         dphi[p] = sub(phi_at(q), phi_at(o));
     });
     const float phi_c = phi[n];
-    float Nt;
-    if constexpr (CF == 2) {
-        int a, b;
-        unpack_sums(own, a, b);
-        Nt = mul(add(static_cast<float>(a), static_cast<float>(b)), kSumInv);
-    } else {
-        Nt = d.nsum[n];
-    }
+    const float Nt = d.nsum[n];
     if constexpr (S::kRef && CF == 0) {
         // references of the values the next phase pass reads at this site: the
         // phase of x - xi_q, which this step writes, or this site's own on a
@@ -711,15 +706,11 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
     const float rA[3] = {fma(bxa, nx, wx), fma(bxa, ny, wy), fma(bxa, nz, wz)};
     const float rB[3] = {fma(bxb, nx, wx), fma(bxb, ny, wy), fma(bxb, nz, wz)};
     if constexpr (CF != 0) {
-        // Sum form: the values in fixed point, added into the sums of the site
-        // that receives them; what stays (the rest value, and the values of
-        // bounce-back links) is the remainder of the site's own Na (Nb), so all
-        // seven add up to it exactly.
-        if constexpr (CF == 1) {
-            const float half = mul(0.5f * kSumOne, Nt);
-            own = pack_sums(__float2int_rn(mul(half, pa1)), __float2int_rn(mul(half, pb1)));
-        }
-        unsigned long long* const acc = d.acc[PAR ^ 1];
+        // Sum form: the values in fixed point, moved from the site's sums to those
+        // of the site that receives them; the rest value, and the values of
+        // bounce-back links, stay.
+        unsigned long long out = 0;
+        unsigned long long* const acc = d.acc;
         const float wN = mul(w7(1) * 0.5f * kSumOne, Nt);
         const float PA = mul(wN, pa1), PB = mul(wN, pb1);
         static_for<0, 3>([&](auto ic) {
@@ -729,18 +720,14 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
                 constexpr int q = 2 * i + 1 + decltype(hc)::value;
                 const unsigned long long x = pack_sums(__float2int_rn(q & 1 ? add(PA, dA) : sub(PA, dA)),
                                                        __float2int_rn(q & 1 ? add(PB, dB) : sub(PB, dB)));
-                // receiver: x + xi_q if it is a pore site, else x itself (bounce-back)
                 const std::integral_constant<int, q> Q;
                 if (has(Q)) {
-                    own -= x;
+                    out -= x;
                     red_add(acc + id(Q), x, pol);
                 }
             });
         });
-        red_add(acc + n, own, pol);
-        // this step's sums of the site are consumed (the phase pass before this
-        // collision was their last other reader): they receive the step after next
-        st_keep(d.acc[PAR] + n, 0ull, pol);
+        red_add(acc + n, out, pol);
     } else {
         // Populations. With fp16 storage the stored quantity is the deviation
         // from w_q (1 +- phi_c)/2: the deviation from w_q Na (w_q Nb), which is
@@ -810,7 +797,6 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
         if constexpr (PAR == 0 || q == 0) in.f[q] = S::ld_s(F + q * P + n);
     });
     if constexpr (S::kRef) in.ref = d.drho[n];
-    if constexpr (CF == 2) in.own = ld_keep(d.acc[PAR] + n, l2_keep());
     for (int i = 0; i < 3; ++i) in.cw[i] = __ldg(d.wall_c + i * P + n);
     if (__any_sync(__activemask(), in.l.a.w & kIrregular)) collide_site<PAR, S, CF, true>(d, n, in, sc);
     else collide_site<PAR, S, CF, false>(d, n, in, sc);
@@ -860,7 +846,7 @@ __device__ __forceinline__ void reservoir_thread(const DomainView& d, int n, int
     });
     if constexpr (SUMS) {
         constexpr int one = 1 << 28;   // kSumOne
-        d.acc[PAR][n] = side == 1 ? pack_sums(one, 0) : pack_sums(0, one);
+        d.acc[n] = side == 1 ? pack_sums(one, 0) : pack_sums(0, one);
     }
 }
 
