@@ -743,13 +743,11 @@ lbpm_status lbpm_measure(lbpm_ctx* c, lbpm_measures* out) {
     if (s) return s;
     if (!out) return fail(c, LBPM_E_INVALID, "out is NULL");
     if (!c->have_fluids) return fail(c, LBPM_E_STATE, "initialise the fluids first");
-    double* d_out;
-    LBPM_ALLOC(c, d_out, double, NSUM);
+    const double* d_out = nullptr;
     double S[NSUM];
-    cudaError_t e = launch_measure(c, static_cast<int>(c->step & 1), d_out, c->stream);
+    cudaError_t e = launch_measure(c, static_cast<int>(c->step & 1), &d_out, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(S, d_out, sizeof S, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    dfree(c, d_out);
     if (e != cudaSuccess) return fail_cuda(c, "measure", e);
     c->launches += 2;
     fill_measures(c, S, out);
@@ -769,7 +767,7 @@ lbpm_status lbpm_read_field(lbpm_ctx* c, int which, float* out) {
     float* d;
     LBPM_ALLOC(c, d, float, c->V);
     cudaError_t e = launch_field(c, static_cast<int>(c->step & 1), which, d, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, sizeof(float) * c->V, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = copy_to_host(out, d, sizeof(float) * c->V, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d);
     if (e != cudaSuccess) return fail_cuda(c, "read_field", e);
@@ -787,7 +785,7 @@ lbpm_status lbpm_read_distributions(lbpm_ctx* c, int which, float* out) {
     float* d;
     LBPM_ALLOC(c, d, float, count);
     cudaError_t e = launch_export_dist(c, static_cast<int>(c->step & 1), which, d, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, sizeof(float) * count, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = copy_to_host(out, d, sizeof(float) * count, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d);
     if (e != cudaSuccess) return fail_cuda(c, "read_distributions", e);
@@ -811,7 +809,7 @@ lbpm_status lbpm_read_box(lbpm_ctx* c, int which, const int* lo, const int* hi, 
     float* d;
     LBPM_ALLOC(c, d, float, count);
     cudaError_t e = launch_read_box(c, static_cast<int>(c->step & 1), which, lo, hi, d, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, sizeof(float) * count, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = copy_to_host(out, d, sizeof(float) * count, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d);
     if (e != cudaSuccess) return fail_cuda(c, "read_box", e);
@@ -866,9 +864,9 @@ lbpm_status lbpm_get_index(lbpm_ctx* c, int64_t* site2vox, int32_t* nbr) {
     }
     cudaError_t e = launch_export_index(c, d_s, d_n, c->stream);
     if (e == cudaSuccess && site2vox)
-        e = cudaMemcpyAsync(site2vox, d_s, sizeof(long long) * c->N, cudaMemcpyDeviceToHost, c->stream);
+        e = copy_to_host(site2vox, d_s, sizeof(long long) * c->N, c->stream);
     if (e == cudaSuccess && nbr)
-        e = cudaMemcpyAsync(nbr, d_n, sizeof(int) * 18 * c->N, cudaMemcpyDeviceToHost, c->stream);
+        e = copy_to_host(nbr, d_n, sizeof(int) * 18 * c->N, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d_s);
     dfree(c, d_n);

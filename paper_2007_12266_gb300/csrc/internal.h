@@ -149,6 +149,10 @@ namespace lbm {
 void* dalloc(lbpm_ctx* c, size_t bytes);
 void dfree(lbpm_ctx* c, void* p);
 
+// Enqueue the copy of `bytes` device bytes to the caller's host buffer on `s`
+// (host_copy.cu; the caller synchronizes the stream).
+cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s);
+
 // launchers (return cudaError_t of the launch)
 cudaError_t launch_flag_pore(const uint16_t* labels, long long V, int* flags, cudaStream_t s);
 cudaError_t exclusive_scan(lbpm_ctx* c, const int* in, int* out, long long n);
@@ -220,7 +224,7 @@ cudaError_t launch_batch_measure(bool fp16, unsigned grid, cudaStream_t s, const
                                  const BatchTile* t, int nt, double* partials, const int* tile_begin, int n_jobs,
                                  double* out);
 int batch_max_blocks(int kernel, bool fp16, int bt);
-cudaError_t launch_measure(lbpm_ctx* c, int parity, double* d_out, cudaStream_t s);
+cudaError_t launch_measure(lbpm_ctx* c, int parity, const double** out, cudaStream_t s);
 cudaError_t launch_field(const lbpm_ctx* c, int parity, int which, float* dense, cudaStream_t s);
 cudaError_t launch_export_dist(const lbpm_ctx* c, int parity, int which, float* out, cudaStream_t s);
 cudaError_t launch_read_box(const lbpm_ctx* c, int parity, int which, const int* lo, const int* hi, float* out,

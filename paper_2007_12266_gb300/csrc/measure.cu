@@ -220,8 +220,9 @@ struct ImportK {
 
 }  // namespace
 
-// d_out receives NSUM doubles. Uses c->d_partials (allocated on demand).
-cudaError_t launch_measure(lbpm_ctx* c, int parity, double* d_out, cudaStream_t s) {
+// *out receives the address of the NSUM results, which lie behind the partial
+// sums in c->d_partials (allocated on demand, kept by the context).
+cudaError_t launch_measure(lbpm_ctx* c, int parity, const double** out, cudaStream_t s) {
     // enough blocks that no thread sums more than kMeasureSitesPerThread sites
     long long nb = (c->N + kBlock - 1) / kBlock;
     const long long need = (c->N + kBlock * kMeasureSitesPerThread - 1) / (kBlock * kMeasureSitesPerThread);
@@ -229,13 +230,16 @@ cudaError_t launch_measure(lbpm_ctx* c, int parity, double* d_out, cudaStream_t 
     if (nb < 1) nb = 1;
     if (c->n_partials < nb) {
         dfree(c, c->d_partials);
-        c->d_partials = static_cast<double*>(dalloc(c, sizeof(double) * NSUM * nb));
+        c->n_partials = 0;
+        c->d_partials = static_cast<double*>(dalloc(c, sizeof(double) * NSUM * (nb + 1)));
         if (!c->d_partials) return cudaErrorMemoryAllocation;
         c->n_partials = nb;
     }
     cudaError_t e = dispatch<MeasureK>(c, parity, static_cast<unsigned>(nb), s, make_view(c), c->d_partials);
     if (e != cudaSuccess) return e;
-    k_reduce_partials<<<1, 32 * NSUM, 0, s>>>(c->d_partials, static_cast<int>(nb), d_out);
+    double* const res = c->d_partials + NSUM * c->n_partials;
+    k_reduce_partials<<<1, 32 * NSUM, 0, s>>>(c->d_partials, static_cast<int>(nb), res);
+    *out = res;
     return cudaGetLastError();
 }
 
