@@ -164,8 +164,10 @@ lbpm_status build_boundaries(lbpm_ctx* c) {
     c->n_slab = 0;
     if (c->params.reservoir_z == 3 && !c->d_face_part) {
         c->d_face_part = static_cast<double*>(dalloc(c, sizeof(double) * 2 * kFaceBlocks));
-        c->d_face_rho = static_cast<float*>(dalloc(c, sizeof(float) * 2));
-        if (!c->d_face_part || !c->d_face_rho) return fail(c, LBPM_E_OOM, "device allocation of the flux inlet failed");
+        c->d_face_rho = static_cast<float*>(dalloc(c, sizeof(float) * kFaceWords));
+        if (!c->d_face_part || !c->d_face_rho ||
+            cudaMemsetAsync(c->d_face_rho, 0, sizeof(float) * kFaceWords, c->stream) != cudaSuccess)
+            return fail(c, LBPM_E_OOM, "device allocation of the flux inlet failed");
     }
     if (c->params.reservoir_z) {
         LBPM_ALLOC(c, flags, int, c->N);
@@ -247,15 +249,14 @@ cudaError_t launch_step_collide(lbpm_ctx* c, int kind, int par, cudaStream_t s) 
 // slabs, pressure faces); it writes what the next step (parity par ^ 1) reads.
 cudaError_t launch_step_boundary(lbpm_ctx* c, int kind, int par, cudaStream_t s) {
     if (!c->n_slab) return cudaSuccess;
-    if (kind == kStepPop || kind == kStepSumLast) return launch_reservoir(c, par ^ 1, s);
-    return launch_reservoir_sum(c, par ^ 1, s);
+    return launch_reservoir(c, par ^ 1, kind == kStepSumFirst || kind == kStepSumMid, s);
 }
 
 // One timestep: phase pass, fused collide-stream, reservoir reset.
 cudaError_t enqueue_step(lbpm_ctx* c, int par, cudaStream_t s) {
     cudaError_t e = launch_phase(c, par, false, s);
     if (e == cudaSuccess) e = launch_collide(c, par, s);
-    if (e == cudaSuccess && c->n_slab) e = launch_reservoir(c, par ^ 1, s);
+    if (e == cudaSuccess && c->n_slab) e = launch_reservoir(c, par ^ 1, false, s);
     return e;
 }
 
@@ -592,7 +593,7 @@ lbpm_status lbpm_init_fluids(lbpm_ctx* c, const float* phi0) {
     LBPM_ALLOC(c, d_p, float, c->V);
     cudaError_t e = cudaMemcpyAsync(d_p, phi0, sizeof(float) * c->V, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = launch_init_fluids(c, d_p, c->stream);
-    if (e == cudaSuccess) e = launch_reservoir(c, 0, c->stream);
+    if (e == cudaSuccess) e = launch_reservoir(c, 0, false, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d_p);
     if (e != cudaSuccess) return fail_cuda(c, "fluid initialisation", e);
@@ -722,7 +723,7 @@ lbpm_status lbpm_advance(lbpm_ctx* c, long long nsteps) {
         if (e2 >= 0 && e3 >= 0) c->ev_collide.emplace_back(e2, e3);
         c->launches += 2;
         if (c->n_slab) {
-            LBPM_CK(c, launch_reservoir(c, par ^ 1, c->stream));
+            LBPM_CK(c, launch_reservoir(c, par ^ 1, false, c->stream));
             c->launches += 1;
         }
         c->step += 1;

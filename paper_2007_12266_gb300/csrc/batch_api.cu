@@ -242,7 +242,7 @@ cudaError_t enqueue_step(lbpm_batch* b, int kind, int par, cudaStream_t s) {
     const bool sums_next = kind == kBSumFirst || kind == kBSumMid;
     for (lbpm_ctx* c : b->jobs)
         if (e == cudaSuccess && c->n_slab)
-            e = sums_next ? launch_reservoir_sum(c, par ^ 1, s) : launch_reservoir(c, par ^ 1, s);
+            e = launch_reservoir(c, par ^ 1, sums_next, s);
     return e;
 }
 

@@ -113,7 +113,7 @@ struct lbpm_ctx {
     float* d_nsum = nullptr;        // [N]
     float* d_rsum = nullptr;        // [N] fp16 storage
     double* d_face_part = nullptr;          // flux inlet: per-block sums (2 * kFaceBlocks)
-    float* d_face_rho = nullptr;            // flux inlet: (rho, rho - 1) of the inlet face
+    float* d_face_rho = nullptr;            // flux inlet: (rho, rho - 1) of the inlet face, block counter (kFaceWords)
     float* d_drho = nullptr;                // [N] fp16 store
     void* d_f = nullptr;
     void* d_a = nullptr;
@@ -182,15 +182,16 @@ cudaError_t launch_collide(const lbpm_ctx* c, int parity, cudaStream_t s);
 // between the sums.
 cudaError_t launch_phase_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
 cudaError_t launch_collide_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
-// Reservoir slabs (reservoir_z = 1) in the sum form: the reset state goes into
-// the sums the next step (parity `parity`) reads, and into its f slots.
-cudaError_t launch_reservoir_sum(const lbpm_ctx* c, int parity, cudaStream_t s);
 // Whether a context can run the sum form (no pressure or flux faces, the
 // population form not forced).
 bool sum_form_capable(const lbpm_ctx* c);
-cudaError_t launch_reservoir(const lbpm_ctx* c, int parity, cudaStream_t s);
+// Reservoir slabs or faces after a collision, for the next step (parity `parity`):
+// the reset state (slabs; sums: the components' into the sums) or what enters
+// (faces, population form only).
+cudaError_t launch_reservoir(const lbpm_ctx* c, int parity, bool sums, cudaStream_t s);
 // flux inlet: blocks of the fixed-order face reduction
 constexpr int kFaceBlocks = 64;
+constexpr int kFaceWords = 4;   // (rho, rho - 1) of the inlet and the counter of finished blocks
 cudaError_t launch_morph(const lbpm_ctx* c, int parity, float delta, int R, int apply, float* phi_grid,
                          float* dist_grid, float* ntot, int3* off, long long* off_lin, float* off_len, int n_off,
                          unsigned long long* counts, cudaStream_t s);

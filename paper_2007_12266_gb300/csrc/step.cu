@@ -65,63 +65,92 @@ __global__ void __launch_bounds__(CollideShape<S>::kThreads, CollideShape<S>::kB
     if (n < d.n_sites) collide_thread<PAR, S, CF>(d, n, SlotCache{slot + threadIdx.x, ref + threadIdx.x, BT});
 }
 
+// The boundary kernels run after the collision with programmatic launch: the
+// next phase pass, which waits for them, must not start before the collision has
+// completed, so every thread waits first.
 template <int PAR, class S>
 __global__ void __launch_bounds__(kBlock) k_pressure_faces(DomainView d, const int* sites,
                                                            const signed char* side, int n_face,
                                                            float rho_in, float rho_out, float drho_in,
                                                            float drho_out, const float* face) {
+    wait_prior_grid();
+    allow_next_grid();
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i < n_face) pressure_face_thread<PAR, S>(d, sites[i], side[i], rho_in, rho_out, drho_in, drho_out, face);
 }
 
-// Flux inlet, first half: per-block sums (fixed grid, fixed order: the result
-// does not depend on scheduling) of D_s over the inlet sites and their count.
+__device__ __forceinline__ double warp_total(double v) {
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Flux inlet: per-block sums (fixed grid, fixed order: the result does not
+// depend on scheduling) of D_s over the inlet sites and their count; the block
+// that finishes last adds them up, again in a fixed order, and sets the inlet's
+// density,
+//   rho_in - 1 = (sum D + Q) / (n_in - Q), from sum_s (1 + D_s) / (n_in - Q).
+// A few thousand sites: latency is all of it, so the sums are warp trees (one
+// thread's 64 dependent fp64 additions took longer than the rest).
 template <int PAR, class S>
-__global__ void __launch_bounds__(kBlock) k_face_sum(DomainView d, const int* sites, const signed char* side,
-                                                     int n_face, double* part) {
-    __shared__ double sd[kBlock];
-    __shared__ double sc[kBlock];
-    double acc = 0.0, cnt = 0.0;
+__global__ void __launch_bounds__(kBlock) k_face_rho(DomainView d, const int* sites, const signed char* side,
+                                                     int n_face, double* part, double flux, float* face) {
+    constexpr int kWarps = kBlock / 32;
+    __shared__ double sd[kWarps];
+    __shared__ int sc[kWarps];
+    __shared__ bool last;
+    static_assert(kFaceBlocks == 64 && kWarps >= 1, "the last block's first warp adds two partial sums per lane");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    wait_prior_grid();
+    allow_next_grid();
+    double acc = 0.0;
+    int cnt = 0;
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < n_face; i += kFaceBlocks * kBlock) {
         if (side[i] != 1) continue;
         int nb[Q19];
         float dv[Q19], nx, ny;
         acc += face_deviations<PAR, S>(d, sites[i], 1.0f, nb, dv, nx, ny);
-        cnt += 1.0;
+        ++cnt;
     }
-    sd[threadIdx.x] = acc;
-    sc[threadIdx.x] = cnt;
+    acc = warp_total(acc);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) {
+        sd[warp] = acc;
+        sc[warp] = cnt;
+    }
     __syncthreads();
-    for (int w = kBlock / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            sd[threadIdx.x] += sd[threadIdx.x + w];
-            sc[threadIdx.x] += sc[threadIdx.x + w];
-        }
-        __syncthreads();
-    }
+    unsigned* const finished = reinterpret_cast<unsigned*>(face + 2);
     if (threadIdx.x == 0) {
-        part[2 * blockIdx.x] = sd[0];
-        part[2 * blockIdx.x + 1] = sc[0];
+        double D = 0.0;
+        int n = 0;
+        for (int w = 0; w < kWarps; ++w) {
+            D += sd[w];
+            n += sc[w];
+        }
+        part[2 * blockIdx.x] = D;
+        part[2 * blockIdx.x + 1] = static_cast<double>(n);
+        __threadfence();
+        last = atomicAdd(finished, 1u) + 1u == kFaceBlocks;
     }
-}
-
-// Second half: rho_in - 1 = (sum D + Q) / (n_in - Q), from sum_s (1 + D_s) / (n_in - Q).
-__global__ void k_face_rho(const double* part, double flux, float* face) {
-    if (threadIdx.x != 0) return;
-    double D = 0.0, n = 0.0;
-    for (int b = 0; b < kFaceBlocks; ++b) {
-        D += part[2 * b];
-        n += part[2 * b + 1];
-    }
+    __syncthreads();
+    if (!last || warp != 0) return;
+    __threadfence();
+    const volatile double* const p = part;
+    const double D = warp_total(p[2 * lane] + p[2 * (lane + 32)]);
+    const double n = warp_total(p[2 * lane + 1] + p[2 * (lane + 32) + 1]);
+    if (lane != 0) return;
     const double drho = n > flux ? (D + flux) / (n - flux) : 0.0;
     face[0] = static_cast<float>(1.0 + drho);
     face[1] = static_cast<float>(drho);
+    *finished = 0u;                        // for the next launch
 }
 
 template <int PAR, class S, bool SUMS>
 __global__ void __launch_bounds__(kBlock) k_reservoir(DomainView d, const int* sites,
                                                       const signed char* side, int n_slab,
                                                       float rho_in, float rho_out) {
+    wait_prior_grid();
+    allow_next_grid();
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i < n_slab) reservoir_thread<PAR, S, SUMS>(d, sites[i], side[i], rho_in, rho_out);
 }
@@ -295,66 +324,38 @@ cudaError_t launch_collide_sum(const lbpm_ctx* c, int parity, cudaStream_t s) {
 }
 
 // parity = parity of the step that will READ the reset values; reservoir slabs
-// (reservoir_z = 1) or the pressure boundary at the z faces (reservoir_z = 2)
-cudaError_t launch_reservoir(const lbpm_ctx* c, int parity, cudaStream_t s) {
-    if (c->n_slab == 0) return cudaSuccess;
-    DomainView d = make_view(c);
+// (reservoir_z = 1) or the boundary at the z faces (2: pressure, 3: flux inlet)
+template <int PAR, class S, bool SUMS>
+cudaError_t launch_reservoir_form(const lbpm_ctx* c, cudaStream_t s) {
+    const DomainView d = make_view(c);
     const unsigned g = blocks_for(c->n_slab);
     const int ns = static_cast<int>(c->n_slab);
-    const float ri = static_cast<float>(c->params.rho_in), ro = static_cast<float>(c->params.rho_out);
-    const bool h = c->params.precision == LBPM_FP16;
-    if (c->params.reservoir_z >= 2) {   // pressure faces; flux inlet (3)
-        // rho - 1 formed in double, so the small difference keeps full fp32 precision
-        const float di = static_cast<float>(c->params.rho_in - 1.0), dout = static_cast<float>(c->params.rho_out - 1.0);
-        const int* st = c->d_slab_site;
-        const signed char* sd = c->d_slab_side;
-        float* face = nullptr;
-        if (c->params.reservoir_z == 3) {
-            face = c->d_face_rho;
-            double* part = c->d_face_part;
-            if (parity == 0) {
-                if (h) k_face_sum<0, StoreF16><<<kFaceBlocks, kBlock, 0, s>>>(d, st, sd, ns, part);
-                else k_face_sum<0, StoreF32><<<kFaceBlocks, kBlock, 0, s>>>(d, st, sd, ns, part);
-            } else {
-                if (h) k_face_sum<1, StoreF16><<<kFaceBlocks, kBlock, 0, s>>>(d, st, sd, ns, part);
-                else k_face_sum<1, StoreF32><<<kFaceBlocks, kBlock, 0, s>>>(d, st, sd, ns, part);
-            }
-            k_face_rho<<<1, 32, 0, s>>>(part, c->params.flux_in, face);
-        }
-        if (parity == 0) {
-            if (h) k_pressure_faces<0, StoreF16><<<g, kBlock, 0, s>>>(d, st, sd, ns, ri, ro, di, dout, face);
-            else k_pressure_faces<0, StoreF32><<<g, kBlock, 0, s>>>(d, st, sd, ns, ri, ro, di, dout, face);
-        } else {
-            if (h) k_pressure_faces<1, StoreF16><<<g, kBlock, 0, s>>>(d, st, sd, ns, ri, ro, di, dout, face);
-            else k_pressure_faces<1, StoreF32><<<g, kBlock, 0, s>>>(d, st, sd, ns, ri, ro, di, dout, face);
-        }
-        return cudaGetLastError();
+    const lbpm_params& p = c->params;
+    const float ri = static_cast<float>(p.rho_in), ro = static_cast<float>(p.rho_out);
+    const int* const st = c->d_slab_site;
+    const signed char* const sd = c->d_slab_side;
+    if (p.reservoir_z == 1) return launch_pdl(k_reservoir<PAR, S, SUMS>, g, s, d, st, sd, ns, ri, ro);
+    // rho - 1 formed in double, so the small difference keeps full fp32 precision
+    const float di = static_cast<float>(p.rho_in - 1.0), dout = static_cast<float>(p.rho_out - 1.0);
+    const float* face = nullptr;
+    if (p.reservoir_z == 3) {
+        const cudaError_t e = launch_pdl(k_face_rho<PAR, S>, kFaceBlocks, s, d, st, sd, ns, c->d_face_part, p.flux_in,
+                                         c->d_face_rho);
+        if (e != cudaSuccess) return e;
+        face = c->d_face_rho;
     }
-    if (parity == 0) {
-        if (h) k_reservoir<0, StoreF16, false><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-        else k_reservoir<0, StoreF32, false><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-    } else {
-        if (h) k_reservoir<1, StoreF16, false><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-        else k_reservoir<1, StoreF32, false><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-    }
-    return cudaGetLastError();
+    return launch_pdl(k_pressure_faces<PAR, S>, g, s, d, st, sd, ns, ri, ro, di, dout, face);
+}
+template <int PAR>
+cudaError_t launch_reservoir_par(const lbpm_ctx* c, bool sums, cudaStream_t s) {
+    if (c->params.precision == LBPM_FP16)
+        return sums ? launch_reservoir_form<PAR, StoreF16, true>(c, s) : launch_reservoir_form<PAR, StoreF16, false>(c, s);
+    return sums ? launch_reservoir_form<PAR, StoreF32, true>(c, s) : launch_reservoir_form<PAR, StoreF32, false>(c, s);
 }
 
-cudaError_t launch_reservoir_sum(const lbpm_ctx* c, int parity, cudaStream_t s) {
-    if (c->n_slab == 0 || c->params.reservoir_z != 1) return cudaSuccess;
-    DomainView d = make_view(c);
-    const unsigned g = blocks_for(c->n_slab);
-    const int ns = static_cast<int>(c->n_slab);
-    const float ri = static_cast<float>(c->params.rho_in), ro = static_cast<float>(c->params.rho_out);
-    const bool h = c->params.precision == LBPM_FP16;
-    if (parity == 0) {
-        if (h) k_reservoir<0, StoreF16, true><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-        else k_reservoir<0, StoreF32, true><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-    } else {
-        if (h) k_reservoir<1, StoreF16, true><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-        else k_reservoir<1, StoreF32, true><<<g, kBlock, 0, s>>>(d, c->d_slab_site, c->d_slab_side, ns, ri, ro);
-    }
-    return cudaGetLastError();
+cudaError_t launch_reservoir(const lbpm_ctx* c, int parity, bool sums, cudaStream_t s) {
+    if (c->n_slab == 0) return cudaSuccess;
+    return parity == 0 ? launch_reservoir_par<0>(c, sums, s) : launch_reservoir_par<1>(c, sums, s);
 }
 
 }  // namespace lbm
