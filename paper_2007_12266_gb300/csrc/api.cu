@@ -750,7 +750,7 @@ lbpm_status lbpm_measure(lbpm_ctx* c, lbpm_measures* out) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(S, d_out, sizeof S, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return fail_cuda(c, "measure", e);
-    c->launches += 2;
+    c->launches += 1;
     fill_measures(c, S, out);
     if (out->status) {
         c->unstable = true;

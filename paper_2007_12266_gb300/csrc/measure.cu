@@ -3,8 +3,8 @@
 // instability check), field export and distribution import/export.
 //
 // The reductions run in a fixed order: each thread walks a fixed strided set
-// of sites (compensated fp32, fp64 accuracy, see AccF64), blocks reduce in
-// fp64 with warp shuffles and shared memory, and one block reduces the
+// of sites (compensated fp32, fp64 accuracy, see AccF64), warps add those up
+// pairwise, blocks add their warps in fp64, and the last block adds the
 // per-block partials in fp64. The result depends
 // only on the domain, never on timing.
 #include <algorithm>
@@ -22,21 +22,37 @@ constexpr long long kMeasureSitesPerThread = 64;   // at most this many sites pe
 
 inline unsigned blocks_for(long long n) { return static_cast<unsigned>((n + kBlock - 1) / kBlock); }
 
+// The block that finishes last adds up the blocks' sums in a fixed order (a launch
+// of its own for that cost 4 us and a gap). Two blocks per SM: one, as the fp16
+// form's 144 registers would have it, leaves too few loads in flight.
 template <int PAR, class S>
-__global__ void __launch_bounds__(kBlock) k_measure(DomainView d, double* partials) {
+__global__ void __launch_bounds__(kBlock, 2) k_measure(DomainView d, double* partials, unsigned* finished, double* out) {
+    __shared__ bool last;
     AccF64 acc[NSUM];
     for (int n = blockIdx.x * kBlock + threadIdx.x; n < d.n_sites; n += gridDim.x * kBlock)
         measure_site<PAR, S>(d, n, acc);
     block_reduce_sums<kBlock>(acc, partials + static_cast<size_t>(blockIdx.x) * NSUM);
-}
-
-__global__ void k_reduce_partials(const double* partials, int nblocks, double* out) {
-    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (i >= NSUM) return;
-    double s = 0.0;
-    for (int k = lane; k < nblocks; k += 32) s += partials[static_cast<size_t>(k) * NSUM + i];
-    s = warp_sum(s);
-    if (lane == 0) out[i] = s;
+    if (threadIdx.x < NSUM) __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(finished, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // a warp's four quantities together, so that their loads overlap
+    constexpr int kWarps = kBlock / 32, kEach = (NSUM + kWarps - 1) / kWarps;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double s[kEach] = {};
+    #pragma unroll 4
+    for (unsigned k = lane; k < gridDim.x; k += 32)
+        #pragma unroll
+        for (int j = 0; j < kEach; ++j)
+            if (w + j * kWarps < NSUM) s[j] += __ldcg(partials + static_cast<size_t>(k) * NSUM + w + j * kWarps);
+    #pragma unroll
+    for (int j = 0; j < kEach; ++j) {
+        const double v = warp_sum(s[j]);
+        if (lane == 0 && w + j * kWarps < NSUM) out[w + j * kWarps] = v;
+    }
+    if (threadIdx.x == 0) *finished = 0u;   // for the next launch
 }
 
 __global__ void k_fill(float* p, long long n, float v) {
@@ -188,8 +204,8 @@ cudaError_t dispatch(const lbpm_ctx* c, int parity, unsigned grid, cudaStream_t 
 
 template <int PAR, class S>
 struct MeasureK {
-    static void launch(unsigned g, cudaStream_t s, DomainView d, double* p) {
-        k_measure<PAR, S><<<g, kBlock, 0, s>>>(d, p);
+    static void launch(unsigned g, cudaStream_t s, DomainView d, double* p, unsigned* finished, double* out) {
+        k_measure<PAR, S><<<g, kBlock, 0, s>>>(d, p, finished, out);
     }
 };
 template <int PAR, class S>
@@ -231,16 +247,19 @@ cudaError_t launch_measure(lbpm_ctx* c, int parity, const double** out, cudaStre
     if (c->n_partials < nb) {
         dfree(c, c->d_partials);
         c->n_partials = 0;
-        c->d_partials = static_cast<double*>(dalloc(c, sizeof(double) * NSUM * (nb + 1)));
+        // the blocks' sums, the results, the counter of finished blocks
+        const size_t words = NSUM * (static_cast<size_t>(nb) + 1) + 1;
+        c->d_partials = static_cast<double*>(dalloc(c, sizeof(double) * words));
         if (!c->d_partials) return cudaErrorMemoryAllocation;
+        const cudaError_t e = cudaMemsetAsync(c->d_partials + words - 1, 0, sizeof(double), s);
+        if (e != cudaSuccess) return e;
         c->n_partials = nb;
     }
-    cudaError_t e = dispatch<MeasureK>(c, parity, static_cast<unsigned>(nb), s, make_view(c), c->d_partials);
-    if (e != cudaSuccess) return e;
     double* const res = c->d_partials + NSUM * c->n_partials;
-    k_reduce_partials<<<1, 32 * NSUM, 0, s>>>(c->d_partials, static_cast<int>(nb), res);
+    const cudaError_t e = dispatch<MeasureK>(c, parity, static_cast<unsigned>(nb), s, make_view(c), c->d_partials,
+                                             reinterpret_cast<unsigned*>(res + NSUM), res);
     *out = res;
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_field(const lbpm_ctx* c, int parity, int which, float* dense, cudaStream_t s) {

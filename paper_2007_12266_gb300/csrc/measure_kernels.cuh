@@ -121,16 +121,55 @@ __device__ __forceinline__ void measure_site(const DomainView& d, int n, AccF64 
     if (Na < -1e-2f || Nb < -1e-2f || Nt <= 0.0f || rho <= 0.0f) acc[26].add(1.0);
 }
 
-// Block-wide fp64 reduction of the accumulators into out[0..NSUM) (thread 0..NSUM-1 write).
+// s + err = a + b exactly (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float s = a + b;
+    const float bp = s - a;
+    err = (a - (s - bp)) + (b - bp);
+    return s;
+}
+
+// Sums of a warp's accumulators: lane i receives the warp's sum of acc[i]. Each
+// exchange halves the number of quantities a lane still holds: 31 sums per lane
+// where a tree per quantity takes 135. The sums are unevaluated triples of fp32
+// values, which keep the rounding errors of both parts (72 bits, more than
+// fp64's 53), since the fp64 pipe takes 16 cycles per warp instruction: adding 27
+// quantities there one by one was most of the analysis of a small domain (a call
+// on 11 k sites 53 us before and 39 now with the blocks' total below, 3.7 M sites
+// 180 and 138, a batch of 5.4 M 360 and 315). The order is fixed.
+__device__ __forceinline__ double warp_sums(const AccF64 (&acc)[NSUM]) {
+    const int lane = threadIdx.x & 31;
+    float hi[32], lo[32], rest[32];
+    #pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        hi[i] = i < NSUM ? acc[i < NSUM ? i : 0].hi : 0.0f;
+        lo[i] = i < NSUM ? acc[i < NSUM ? i : 0].lo : 0.0f;
+        rest[i] = 0.0f;
+    }
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool upper = (lane & o) != 0;
+        #pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const float h = __shfl_xor_sync(0xffffffffu, upper ? hi[i] : hi[i + o], o);
+            const float l = __shfl_xor_sync(0xffffffffu, upper ? lo[i] : lo[i + o], o);
+            const float r = o == 16 ? 0.0f : __shfl_xor_sync(0xffffffffu, upper ? rest[i] : rest[i + o], o);
+            float eh, el, em;
+            hi[i] = two_sum(upper ? hi[i + o] : hi[i], h, eh);
+            lo[i] = two_sum(two_sum(upper ? lo[i + o] : lo[i], l, el), eh, em);
+            rest[i] = ((upper ? rest[i + o] : rest[i]) + r) + (el + em);
+        }
+    }
+    return static_cast<double>(hi[0]) + (static_cast<double>(lo[0]) + static_cast<double>(rest[0]));
+}
+
+// Block-wide reduction of the accumulators into out[0..NSUM) (thread 0..NSUM-1
+// write), fp64 across the warps.
 template <int BT>
 __device__ __forceinline__ void block_reduce_sums(AccF64 (&acc)[NSUM], double* out) {
-    __shared__ double red[BT / 32][NSUM];
+    __shared__ double red[BT / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NSUM; ++i) {
-        const double s = warp_sum(acc[i].value());
-        if (lane == 0) red[w][i] = s;
-    }
+    red[w][lane] = warp_sums(acc);
     __syncthreads();
     if (threadIdx.x < NSUM) {
         double s = 0.0;
