@@ -35,6 +35,18 @@ struct FusedSlab {
     int n;
     float rho_in, rho_out;
 };
+// Reservoir slabs of up to kBatchSlabJobs jobs, reset by one launch: job j owns
+// the tiles of kBatchSlabTile slab sites from tile_begin[j].
+constexpr int kBatchSlabJobs = 32;
+constexpr int kBatchSlabTile = 256;
+struct BatchSlabs {
+    int n_jobs;
+    int tile_begin[kBatchSlabJobs + 1];
+    FusedSlab slab[kBatchSlabJobs];
+    DomainView v[kBatchSlabJobs];
+};
+// par = parity of the step that reads the reset state; sums: it reads the component sums
+cudaError_t launch_batch_reservoir(int par, bool sums, bool fp16, cudaStream_t s, const BatchSlabs& p);
 struct FusedLaunch {
     int n_jobs;
     int tiles[3][kFusedJobs + 1];    // first tile of each job: phase entries, sites, slab sites

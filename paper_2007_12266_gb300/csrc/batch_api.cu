@@ -240,9 +240,26 @@ cudaError_t enqueue_step(lbpm_batch* b, int kind, int par, cudaStream_t s) {
                              b->launch[1][i]);
     }
     const bool sums_next = kind == kBSumFirst || kind == kBSumMid;
-    for (lbpm_ctx* c : b->jobs)
-        if (e == cudaSuccess && c->n_slab)
+    BatchSlabs slabs = {};
+    for (const lbpm_ctx* c : b->jobs) {
+        if (e != cudaSuccess) return e;
+        if (!c->n_slab) continue;
+        if (c->params.reservoir_z != 1) {           // pressure and flux faces
             e = launch_reservoir(c, par ^ 1, sums_next, s);
+            continue;
+        }
+        const int k = slabs.n_jobs++;
+        slabs.tile_begin[k + 1] =
+            slabs.tile_begin[k] + static_cast<int>((c->n_slab + kBatchSlabTile - 1) / kBatchSlabTile);
+        slabs.slab[k] = FusedSlab{c->d_slab_site, c->d_slab_side, static_cast<int>(c->n_slab),
+                                  static_cast<float>(c->params.rho_in), static_cast<float>(c->params.rho_out)};
+        slabs.v[k] = make_view(c);
+        if (slabs.n_jobs == kBatchSlabJobs) {
+            e = launch_batch_reservoir(par ^ 1, sums_next, h, s, slabs);
+            slabs.n_jobs = 0;
+        }
+    }
+    if (e == cudaSuccess) e = launch_batch_reservoir(par ^ 1, sums_next, h, s, slabs);
     return e;
 }
 
@@ -328,8 +345,12 @@ lbpm_status batch_advance_fused(lbpm_batch* b, long long nsteps) {
 }
 
 int kernels_per_bundle(const lbpm_batch* b) {
-    int k = 4 * static_cast<int>(b->launch[0].size());
-    for (const lbpm_ctx* c : b->jobs) k += c->n_slab ? 2 : 0;
+    int k = 4 * static_cast<int>(b->launch[0].size()), slabs = 0;
+    for (const lbpm_ctx* c : b->jobs) {
+        if (c->n_slab && c->params.reservoir_z == 1) ++slabs;
+        else k += c->n_slab ? 2 : 0;
+    }
+    k += 2 * ((slabs + kBatchSlabJobs - 1) / kBatchSlabJobs);
     return k;
 }
 
