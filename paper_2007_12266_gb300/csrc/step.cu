@@ -41,20 +41,18 @@ __global__ void __launch_bounds__(kBlock) k_phase_sum(DomainView d) {
     phase_sum_thread<PAR, kPhaseSumPer>(d, blockIdx.x * kBlock * kPhaseSumPer + threadIdx.x, kBlock);
 }
 
-// Launch shape of the collision: 64 registers and 32 resident warps per SM.
-// Blocks of 256 in FP32 and 128 in FP16 measured 146 and 135 us per step on the
-// 256^3 workload; 56 registers and 36 warps (192 and 128 threads) spill and took
-// 152-155 and 153 us.
-template <class S>
-struct CollideShape {
-    static constexpr int kThreads = S::kRef ? 128 : 256;
-    static constexpr int kBlocksPerSm = 1024 / kThreads;
-};
+// Launch shape of the collision: 64 registers and 32 resident warps per SM; 56
+// registers and 36 warps spill and are slower. Blocks of 128 threads in FP16, and in
+// FP32 below kSmallSites: there a launch is a few waves out of L2, which smaller
+// blocks end more evenly (256 / 128 threads, us per step: 3.65 / 3.24 at 7 k sites,
+// 10.1 / 9.7 at 247 k, 21.9 / 21.6 at 657 k, 34.2 / 34.1 at 901 k). Above it the step
+// runs from DRAM and 256 threads are as fast or faster (59.8 / 59.8 at 1.6 M, 91.9 /
+// 92.0 at 2.5 M, 135.6 / 136.5 at 3.7 M).
+constexpr long long kSmallSites = 1LL << 20;
 
 // CF: component form of the collision (see collide_site)
-template <int PAR, class S, int CF>
-__global__ void __launch_bounds__(CollideShape<S>::kThreads, CollideShape<S>::kBlocksPerSm) k_collide(DomainView d) {
-    constexpr int BT = CollideShape<S>::kThreads;
+template <int PAR, class S, int CF, int BT>
+__global__ void __launch_bounds__(BT, 1024 / BT) k_collide(DomainView d) {
     // odd steps: slot (and fp16 reference) cache, see SlotCache; even steps of
     // the sum form: the six face neighbours
     constexpr int kSlots = PAR == 1 ? (Q19 - 1) * BT : (CF != 0 ? (Q7 - 1) * BT : 1);
@@ -295,17 +293,17 @@ cudaError_t launch_phase(const lbpm_ctx* c, int parity, bool sums, cudaStream_t 
     return sums ? launch_phase_form<StoreF32, true>(c, parity, s) : launch_phase_form<StoreF32, false>(c, parity, s);
 }
 
-// one collision launch of the given parity, storage and component form
+// one collision launch of the given parity, storage, component form and block size
+template <int PAR, class S, int CF, int BT>
+cudaError_t launch_collide_shape(const lbpm_ctx* c, cudaStream_t s) {
+    return launch_pdl_bt(k_collide<PAR, S, CF, BT>, static_cast<unsigned>((c->N + BT - 1) / BT), BT, s, make_view(c));
+}
 template <int PAR, int CF>
 cudaError_t launch_collide_form(const lbpm_ctx* c, cudaStream_t s) {
     if (c->N == 0) return cudaSuccess;
-    DomainView d = make_view(c);
-    if (c->params.precision == LBPM_FP16) {
-        constexpr int bt = CollideShape<StoreF16>::kThreads;
-        return launch_pdl_bt(k_collide<PAR, StoreF16, CF>, static_cast<unsigned>((c->N + bt - 1) / bt), bt, s, d);
-    }
-    constexpr int bt = CollideShape<StoreF32>::kThreads;
-    return launch_pdl_bt(k_collide<PAR, StoreF32, CF>, static_cast<unsigned>((c->N + bt - 1) / bt), bt, s, d);
+    if (c->params.precision == LBPM_FP16) return launch_collide_shape<PAR, StoreF16, CF, 128>(c, s);
+    return c->N < kSmallSites ? launch_collide_shape<PAR, StoreF32, CF, 128>(c, s)
+                              : launch_collide_shape<PAR, StoreF32, CF, 256>(c, s);
 }
 
 cudaError_t launch_collide(const lbpm_ctx* c, int parity, cudaStream_t s) {
