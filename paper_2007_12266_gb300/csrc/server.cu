@@ -101,7 +101,11 @@ size_t estimate_footprint(const lbpm_job_spec& sp, long long n_pore) {
     const bool h = sp.params.precision == LBPM_FP16;
     // populations, nsum (+ drho, rsum and the second phase grid with fp16 storage)
     const double state = 33.0 * es * N + (h ? 12.0 : 4.0) * N + (h ? 4.0 * Vp : 0.0);
-    // labels, vsite, phi, site_vox, wall mask
+    // labels, vsite, the solids' phase, site_vox. With the indexer's transient grids
+    // (freed before the state is allocated) this also covers, at porosities of rocks,
+    // the per-site records, phase and sums: at porosity 0.22 224 bytes per site in
+    // fp32 (estimated 213) and 170 in fp16 (173), at 0.35 211 (187) and 157 (140).
+    // A job for which it falls short waits, see lbpm_server_run.
     const double grids = 2.0 * V + 8.0 * Vp + 5.0 * N;
     const double transient = 8.0 * Vp;
     return static_cast<size_t>(state + grids + transient + (1 << 20));
@@ -259,7 +263,20 @@ lbpm_status lbpm_server_run(lbpm_server* s, int* n_running, int* n_queued, int* 
         Job* j = s->queue.front();
         s->queue.pop_front();
         s->used += j->footprint;
-        if ((st = build_job(s, j)) || (st = lbpm_batch_add(s->batch, j->ctx))) {
+        st = build_job(s, j);
+        if (st == LBPM_E_OOM && !(s->running.empty() && s->finished.empty())) {
+            // the estimate fell short of what the device can give: the job waits
+            // for the others' memory (a finished job's at once)
+            if (j->ctx) release_job_device(s, j);
+            else s->used -= j->footprint;
+            s->err.clear();
+            s->queue.push_front(j);
+            if (s->finished.empty()) break;
+            release_job_device(s, s->finished.front());
+            s->finished.pop_front();
+            continue;
+        }
+        if (st || (st = lbpm_batch_add(s->batch, j->ctx))) {
             j->state = LBPM_JOB_FAILED;
             j->note = s->err.empty() ? lbpm_batch_last_error(s->batch) : s->err;
             j->t_done = now_s();
