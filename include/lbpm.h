@@ -302,8 +302,8 @@ lbpm_status lbpm_restore(lbpm_ctx* ctx, const void* host_buf, size_t bytes);
  *     collision adds its recolored values straight into the component
  *     densities Na, Nb of the sites that receive them (the streaming
  *     destinations, or the site itself on a bounce-back link), kept per site
- *     as one 64-bit fixed-point pair (2^-28 units); the next phase pass and
- *     collision read those sums instead of 14 populations. This is exact
+ *     as one 64-bit fixed-point pair (2^-28 units); the next phase pass reads
+ *     those sums instead of 14 populations. This is exact
  *     algebra: the recolored populations depend only on the writer's Na, Nb,
  *     velocity and colour normal, and the next step uses only their sums.
  *     Integer sums are independent of the order of the additions (results
@@ -329,17 +329,18 @@ lbpm_status lbpm_kernel_timing(lbpm_ctx* ctx, double* ms_collide, long long* n_c
 
 /*
  * Batched form: several jobs (independent contexts on one GPU, same storage
- * precision) advanced together. Every timestep of the whole batch is ONE
- * launch of the phase pass and ONE of the fused collide-stream kernel, both
+ * precision) advanced together. With the default launch shape, jobs of 2^16
+ * sites or more on average and every job in the sum form, each job's steps are
+ * a chain of launches of its own, three of them in flight at a time (on streams
+ * that start after the earlier work of the batch's stream, which waits for them).
+ * Otherwise every timestep of the whole batch is ONE launch of the phase pass and ONE of the fused collide-stream kernel, both
  * over a list of tiles that covers all jobs' sites (or, with the fused launch
  * shape of lbpm_batch_set_launch, one kernel runs every pass of a bundle);
  * bundles of two steps are replayed from a CUDA graph. Inside a call of two or more steps the
  * components travel as per-site sums when every job allows it (see
  * lbpm_set_step_form). Each job's results agree with
  * advancing it alone to fp32 rounding (1e-5 relative per distribution after
- * 24 steps in the tests: the batched and single-domain kernels are compiled
- * separately and the compiler may contract multiply-adds differently); two
- * batched runs of the same jobs are bit-identical. Jobs keep their own state and every per-job call
+ * 24 steps in the tests); two batched runs of the same jobs are bit-identical. Jobs keep their own state and every per-job call
  * (lbpm_measure, lbpm_read_field, ...) stays valid; a job joins at an even
  * step and must be removed before it is destroyed. After changing a job's
  * parameters, call lbpm_batch_refresh. Work runs on the batch's stream: use

@@ -667,6 +667,26 @@ lbpm_status advance_sum(lbpm_ctx* c, long long nsteps) {
 
 }  // namespace
 
+namespace lbm {
+
+lbpm_status advance_job(lbpm_ctx* c, long long nsteps, cudaStream_t s, long long* launches) {
+    const cudaStream_t own = c->stream;
+    const long long count = c->launches;
+    const bool timing = c->timing, graphs = c->use_graphs;
+    c->stream = s;
+    c->timing = false;
+    c->use_graphs = true;
+    const lbpm_status st = advance_sum(c, nsteps);
+    *launches += c->launches - count;
+    c->stream = own;
+    c->launches = count;
+    c->timing = timing;
+    c->use_graphs = graphs;
+    return st;
+}
+
+}  // namespace lbm
+
 extern "C" {
 
 lbpm_status lbpm_set_step_form(lbpm_ctx* c, int form) {

@@ -1,6 +1,8 @@
 // Batched form: many independent domains (jobs) advanced together.
 //
-// Each job keeps its own context and device arrays. A batch builds a table of
+// Each job keeps its own context and device arrays. Batches of large jobs run as
+// single-domain launches, job by job (batch_advance_jobs in batch_api.cu says
+// when and why); what follows is for all others. A batch builds a table of
 // the jobs' views and of the first tile of each job (passed by value in the
 // kernel's parameter space), and advances every job with ONE launch per pass:
 // the phase kernel, then the fused collide-stream kernel, over the tiles of

@@ -16,6 +16,11 @@
 
 using namespace lbm;
 
+// Job-by-job form (see by_job): streams that the jobs' chains share, and the mean
+// number of sites per job from which it is taken.
+constexpr int kJobStreams = 3;
+constexpr long long kByJobMean = 1 << 16;
+
 struct lbpm_batch {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -52,6 +57,9 @@ struct lbpm_batch {
     cudaGraphExec_t graph = nullptr;
     cudaGraphExec_t sum_graph = nullptr;
     long long launches = 0;
+    // job-by-job form (see batch_advance_jobs): the streams beside the batch's own
+    cudaStream_t job_stream[kJobStreams - 1] = {};
+    cudaEvent_t job_start = nullptr, job_done[kJobStreams - 1] = {};
     // fused persistent form (blocks per SM -2 for both passes, see batch_fused.cu):
     // the job table, the barrier and tile-counter words, the error flag, and the
     // graph of two steps (two middle steps in the sum form)
@@ -373,6 +381,59 @@ lbpm_status batch_advance_sum(lbpm_batch* b, long long nsteps) {
     return LBPM_OK;
 }
 
+// Whether the batch runs job by job (batch_advance_jobs) instead of one launch per
+// pass over all jobs: with the default launch shape, in the sum form, and with jobs
+// large enough that two or three fill the GPU. A pass over all jobs leaves nothing of
+// a job in L2 for the next pass, where a job of some 100 k sites keeps its whole state
+// there from step to step; and the chains cover each other's tails, where a pass ends
+// for all jobs at once. Us per step of one launch per pass (256 threads) and job by
+// job: 12 jobs of 221 k sites on average 116 and 92 (fp32), 114 and 89 (fp16); 12 of
+// 446 k 225 and 190, 227 and 182; 32 of 83 k 119 and 97, 116 and 99; but 12 of 49 k
+// 23 and 27, 26 and 28, and 12 of 28 k 15 and 21, where a job's launches are too small
+// to fill the GPU three at a time. One, two and four streams: 217, 192, 193 against
+// 190 us on the second set.
+bool by_job(const lbpm_batch* b) {
+    if (b->bt != 192 || b->bps[0] != -1 || b->bps[1] != -1) return false;
+    long long n = 0;
+    for (const lbpm_ctx* c : b->jobs) n += c->N;
+    return n >= kByJobMean * static_cast<long long>(b->jobs.size()) && batch_sum_form(b);
+}
+
+// lbpm_batch_advance job by job: each job's whole run is a chain of its own (the
+// single-domain launches and graphs) on one of kJobStreams streams, the largest
+// jobs first and each to the stream with the fewest sites so far. The batch's
+// stream is one of them; the others start after its earlier work, and it waits
+// for them at the end.
+lbpm_status batch_advance_jobs(lbpm_batch* b, long long nsteps) {
+    for (int k = 0; k < kJobStreams - 1; ++k) {
+        if (!b->job_stream[k]) LBPM_BCK(b, cudaStreamCreateWithFlags(&b->job_stream[k], cudaStreamNonBlocking));
+        if (!b->job_done[k]) LBPM_BCK(b, cudaEventCreateWithFlags(&b->job_done[k], cudaEventDisableTiming));
+    }
+    if (!b->job_start) LBPM_BCK(b, cudaEventCreateWithFlags(&b->job_start, cudaEventDisableTiming));
+    std::vector<lbpm_ctx*> order(b->jobs.begin(), b->jobs.end());
+    std::stable_sort(order.begin(), order.end(), [](const lbpm_ctx* x, const lbpm_ctx* y) { return x->N > y->N; });
+    cudaStream_t stream[kJobStreams];
+    long long sites[kJobStreams] = {};
+    for (int k = 0; k < kJobStreams; ++k) stream[k] = k == 0 ? b->stream : b->job_stream[k - 1];
+    LBPM_BCK(b, cudaEventRecord(b->job_start, b->stream));
+    for (int k = 1; k < kJobStreams; ++k) LBPM_BCK(b, cudaStreamWaitEvent(stream[k], b->job_start, 0));
+    lbpm_status st = LBPM_OK;
+    for (lbpm_ctx* c : order) {
+        const long long k = std::min_element(sites, sites + kJobStreams) - sites;
+        sites[k] += c->N;
+        if ((st = advance_job(c, nsteps, stream[k], &b->launches))) {
+            bfail(b, st, c->err);
+            break;
+        }
+    }
+    // joined also after an error: nothing of the batch is in flight beside its stream
+    for (int k = 1; k < kJobStreams; ++k) {
+        LBPM_BCK(b, cudaEventRecord(b->job_done[k - 1], stream[k]));
+        LBPM_BCK(b, cudaStreamWaitEvent(b->stream, b->job_done[k - 1], 0));
+    }
+    return st;
+}
+
 // launch-shape cache: (gpu, precision, log2 of the site count) -> (bt, bps0, bps1)
 std::mutex g_tune_mu;
 std::map<std::string, std::vector<int>> g_tune_cache;
@@ -416,6 +477,11 @@ lbpm_status lbpm_batch_destroy(lbpm_batch* b) {
     else cudaDeviceSynchronize();
     drop_graph(b);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+    for (cudaStream_t t : b->job_stream)
+        if (t) cudaStreamDestroy(t);
+    for (cudaEvent_t e : b->job_done)
+        if (e) cudaEventDestroy(e);
+    if (b->job_start) cudaEventDestroy(b->job_start);
     bfree(b, b->d_views);
     bfree(b, b->d_parity);
     bfree(b, b->d_mtiles);
@@ -502,6 +568,7 @@ lbpm_status lbpm_batch_advance(lbpm_batch* b, long long nsteps) {
     if (b->jobs.empty() || nsteps == 0) return LBPM_OK;
     if (b->dirty && (s = rebuild(b))) return s;
     if (use_fused(b)) return batch_advance_fused(b, nsteps);
+    if (by_job(b)) return batch_advance_jobs(b, nsteps);
     if (batch_sum_form(b)) return batch_advance_sum(b, nsteps);
     if (!b->graph && (s = capture(b, kBPop, 0, &b->graph))) return s;
     for (long long k = 0; k < nsteps; k += 2) LBPM_BCK(b, cudaGraphLaunch(b->graph, b->stream));

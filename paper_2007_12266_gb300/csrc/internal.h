@@ -225,6 +225,9 @@ cudaError_t launch_batch_measure(bool fp16, unsigned grid, cudaStream_t s, const
                                  const BatchTile* t, int nt, double* partials, const int* tile_begin, int n_jobs,
                                  double* out);
 int batch_max_blocks(int kernel, bool fp16, int bt);
+// nsteps (>= 2) timesteps of one job of a batch in the sum form, enqueued on s
+// instead of the context's own stream; adds the kernels launched to *launches.
+lbpm_status advance_job(lbpm_ctx* c, long long nsteps, cudaStream_t s, long long* launches);
 cudaError_t launch_measure(lbpm_ctx* c, int parity, const double** out, cudaStream_t s);
 cudaError_t launch_field(const lbpm_ctx* c, int parity, int which, float* dense, cudaStream_t s);
 cudaError_t launch_export_dist(const lbpm_ctx* c, int parity, int which, float* out, cudaStream_t s);
