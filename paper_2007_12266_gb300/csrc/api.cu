@@ -685,6 +685,14 @@ lbpm_status advance_job(lbpm_ctx* c, long long nsteps, cudaStream_t s, long long
     return st;
 }
 
+lbpm_status capture_job(lbpm_ctx* c, long long nsteps) {
+    const int sizes[2] = {2, 16};
+    for (int gi = 0; gi < 2; ++gi)   // first, second and last step are plain launches
+        if (nsteps - 3 >= sizes[gi] && !c->sum_graphs[gi])
+            LBPM_CK(c, capture_sum_bundle(c, sizes[gi], &c->sum_graphs[gi]));
+    return LBPM_OK;
+}
+
 }  // namespace lbm
 
 extern "C" {

@@ -665,6 +665,13 @@ lbpm_status lbpm_batch_tune(lbpm_batch* b, int steps_per_candidate, int* threads
                 const int bps = frac < 0 ? frac : std::max(1, occ * frac / 4);
                 if ((s = lbpm_batch_set_launch(b, bt, bps, bps))) break;
                 if ((s = lbpm_batch_advance(b, 2))) break;  // capture + warm up
+                if (by_job(b))   // their graphs, which two steps do not use
+                    for (lbpm_ctx* c : b->jobs)
+                        if ((s = capture_job(c, steps_per_candidate))) {
+                            bfail(b, s, c->err);
+                            break;
+                        }
+                if (s) break;
                 cudaEventRecord(e0, b->stream);
                 if ((s = lbpm_batch_advance(b, steps_per_candidate))) break;
                 cudaEventRecord(e1, b->stream);

@@ -228,6 +228,8 @@ int batch_max_blocks(int kernel, bool fp16, int bt);
 // nsteps (>= 2) timesteps of one job of a batch in the sum form, enqueued on s
 // instead of the context's own stream; adds the kernels launched to *launches.
 lbpm_status advance_job(lbpm_ctx* c, long long nsteps, cudaStream_t s, long long* launches);
+// Capture the graphs that such a run uses, without advancing the job.
+lbpm_status capture_job(lbpm_ctx* c, long long nsteps);
 cudaError_t launch_measure(lbpm_ctx* c, int parity, const double** out, cudaStream_t s);
 cudaError_t launch_field(const lbpm_ctx* c, int parity, int which, float* dense, cudaStream_t s);
 cudaError_t launch_export_dist(const lbpm_ctx* c, int parity, int which, float* out, cudaStream_t s);
