@@ -96,7 +96,7 @@ def kernel_hash(precision: str) -> str:
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2007_12266_gb300", "csrc")
-    for name in ("step_kernels.cuh", "step.cu", "lattice.cuh", "internal.h"):
+    for name in ("step_kernels.cuh", "step.cu", "lattice.cuh", "links.cuh", "internal.h"):
         with open(os.path.join(csrc, name)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)

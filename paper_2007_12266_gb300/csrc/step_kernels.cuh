@@ -408,8 +408,8 @@ struct SiteState {
 // What bounds it: DRAM with fp32 storage (live, 202 B per site at 5.9 TB/s at even
 // and 5.4 TB/s at odd steps, of 6.7 for a plain copy, on 3.69 M sites of a 256^3
 // pack), with fp16 the latency of the loads, with 32 warps per SM resident, and
-// the instructions (595 and 785 per site at even and odd steps in fp32, 651 and
-// 972 in fp16). So neighbours come from a 24-byte record per site and the phase
+// the instructions (581 and 769 per site at even and odd steps in fp32, 644 and
+// 954 in fp16). So neighbours come from a 24-byte record per site and the phase
 // is kept per site: against gathering 18 phases and 18 (odd) or 6 site ids from
 // dense voxel grids, where the 32 sites of a warp span about 150 voxels, a warp
 // touches half the cache lines (L1 data-pipe wavefronts per warp 289 -> 175 odd,
@@ -417,7 +417,8 @@ struct SiteState {
 // scattered stores: 161 -> 146 us per step in fp32, 154 -> 135 in fp16, 7.7 ->
 // 6.3 on 79 k sites. And the component sums are updated in place, in one array
 // that stays in L2 instead of two of which the collision reads one and clears it:
-// 143 -> 136 us in fp32 (15 B per site less from DRAM), 135 -> 131 in fp16. Two
+// 143 -> 136 us in fp32 (15 B per site less from DRAM), 135 -> 131 in fp16, 129
+// with two fused multiply-adds per pair and fewer fixed-point conversions. Two
 // sites per thread on fma.rn.f32x2 took 463 instructions per site in an earlier
 // form but ran slower: twice the registers left fewer warps to cover the latency.
 template <int PAR, class S, int CF, bool DENSE>
