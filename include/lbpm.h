@@ -329,7 +329,7 @@ lbpm_status lbpm_kernel_timing(lbpm_ctx* ctx, double* ms_collide, long long* n_c
 
 /*
  * Batched form: several jobs (independent contexts on one GPU, same storage
- * precision) advanced together. With the default launch shape, jobs of 2^16
+ * precision) advanced together. With the default launch shape, jobs of 81920
  * sites or more on average and every job in the sum form, each job's steps are
  * a chain of launches of its own, three of them in flight at a time (on streams
  * that start after the earlier work of the batch's stream, which waits for them).

@@ -19,7 +19,7 @@ using namespace lbm;
 // Job-by-job form (see by_job): streams that the jobs' chains share, and the mean
 // number of sites per job from which it is taken.
 constexpr int kJobStreams = 3;
-constexpr long long kByJobMean = 1 << 16;
+constexpr long long kByJobMean = 80 << 10;
 
 struct lbpm_batch {
     int device = 0;
@@ -390,7 +390,10 @@ lbpm_status batch_advance_sum(lbpm_batch* b, long long nsteps) {
 // job: 12 jobs of 221 k sites on average 116 and 92 (fp32), 114 and 89 (fp16); 12 of
 // 446 k 225 and 190, 227 and 182; 32 of 83 k 119 and 97, 116 and 99; but 12 of 49 k
 // 23 and 27, 26 and 28, and 12 of 28 k 15 and 21, where a job's launches are too small
-// to fill the GPU three at a time. One, two and four streams: 217, 192, 193 against
+// to fill the GPU three at a time; and 48 of 71 k, 40 steps a call 147 and 136, lose in
+// calls of 6 to 16 steps (152 and 161, where launching them takes the host as long),
+// which 32 of 83 k do not (calls of 2, 8, 16 steps: 133 and 128, 122 and 118, 120 and
+// 116), so the line lies between. One, two and four streams: 217, 192, 193 against
 // 190 us on the second set.
 bool by_job(const lbpm_batch* b) {
     if (b->bt != 192 || b->bps[0] != -1 || b->bps[1] != -1) return false;

@@ -8,7 +8,7 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-EDGES = [(40, 40, 36), (64, 32, 32), (41, 41, 41), (40, 64, 28), (33, 64, 31)]   # 65,400 sites on average
+EDGES = [(40, 40, 36), (64, 32, 32), (41, 41, 41), (40, 64, 28), (33, 64, 31)]
 
 
 def _domains(precision, grow):
@@ -26,7 +26,7 @@ def _domains(precision, grow):
 
 
 @pytest.mark.parametrize("precision", ["fp32", "fp16"])
-@pytest.mark.parametrize("grow", [0, 24])
+@pytest.mark.parametrize("grow", [8, 9])         # layers more
 def test_by_job_is_the_same(grow, precision):
     import paper_2007_12266_gb300 as lbm
     runs = []
@@ -43,7 +43,7 @@ def test_by_job_is_the_same(grow, precision):
         launches = b.launch_count - n0
         mean = b.n_sites / len(doms)
         # two kernels per step and job, one more for the reservoirs; or per step
-        assert launches == 32 * (2 * len(doms) + 1 if not shape and mean >= 1 << 16 else 3)
+        assert launches == 32 * (2 * len(doms) + 1 if not shape and mean >= 80 << 10 else 3)
         m = b.measure()
         runs.append([[d.distributions(k) for k in ("f", "a", "b")] for d in doms] + [m])
         b.close()
