@@ -86,10 +86,8 @@ void free_image(lbpm_ctx* c) {
     dfree(c, c->d_phis);
     dfree(c, c->d_link_a);
     dfree(c, c->d_link_b);
-    dfree(c, c->d_wall_c);
     c->d_link_a = nullptr;
     c->d_link_b = nullptr;
-    c->d_wall_c = nullptr;
     dfree(c, c->d_slab_site);
     dfree(c, c->d_slab_side);
     dfree(c, c->d_face_part);
@@ -137,19 +135,16 @@ lbpm_status alloc_state(lbpm_ctx* c) {
 }
 
 // what depends on the periodic axes and the boundaries: the grids' halo, each
-// site's neighbour record and the solids' part of its colour gradient, and the
-// reservoir site list
+// site's neighbour record, and the reservoir site list
 lbpm_status build_boundaries(lbpm_ctx* c) {
     drop_graphs(c);
     LBPM_CK(c, launch_fill_halo(c, c->stream));
     const size_t P = static_cast<size_t>(pitch_of(c->N));
     if (!c->d_link_a) c->d_link_a = static_cast<int4*>(dalloc(c, sizeof(int4) * P));
     if (!c->d_link_b) c->d_link_b = static_cast<int2*>(dalloc(c, sizeof(int2) * P));
-    if (!c->d_wall_c) c->d_wall_c = static_cast<float*>(dalloc(c, sizeof(float) * 3 * P));
-    if (!c->d_link_a || !c->d_link_b || !c->d_wall_c)
+    if (!c->d_link_a || !c->d_link_b)
         return fail(c, LBPM_E_OOM, "device allocation of the neighbour records failed");
     LBPM_CK(c, launch_links(c, c->stream));
-    LBPM_CK(c, launch_wall_gradient(c, c->stream));
     LBPM_CK(c, cudaStreamSynchronize(c->stream));
     int* flags;
     int* scan;
@@ -558,11 +553,10 @@ lbpm_status lbpm_set_affinity_table(lbpm_ctx* c, const float* table, int n_label
     cudaError_t e = cudaMemcpyAsync(d_t, table, sizeof(float) * n_labels, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = launch_affinity_table(c, d_t, n_labels, c->stream);
     if (e == cudaSuccess) e = launch_fill_halo(c, c->stream);
-    if (e == cudaSuccess) e = launch_wall_gradient(c, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d_t);
     if (e != cudaSuccess) return fail_cuda(c, "affinity table", e);
-    c->launches += 3;
+    c->launches += 2;
     return LBPM_OK;
 }
 
@@ -576,11 +570,10 @@ lbpm_status lbpm_set_affinity_map(lbpm_ctx* c, const float* map) {
     cudaError_t e = cudaMemcpyAsync(d_m, map, sizeof(float) * c->V, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = launch_affinity_map(c, d_m, c->stream);
     if (e == cudaSuccess) e = launch_fill_halo(c, c->stream);
-    if (e == cudaSuccess) e = launch_wall_gradient(c, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     dfree(c, d_m);
     if (e != cudaSuccess) return fail_cuda(c, "affinity map", e);
-    c->launches += 3;
+    c->launches += 2;
     return LBPM_OK;
 }
 

@@ -8,8 +8,7 @@
 // complement of the voxel's rank, or wall, -1) and phis[pv] holds phi_s
 // (Sec. 3.2, Eq. phi_s) at solids and 0 elsewhere. Halo voxels of periodic axes
 // copy the voxel they wrap to. The steps themselves read what is derived from
-// these grids per site: the neighbour ids (SiteLinks) and the solids' part of
-// the colour gradient.
+// the first per site, the neighbour ids (SiteLinks), and phi_s from the second.
 #include "internal.h"
 #include "lattice.cuh"
 #include "links.cuh"
@@ -253,24 +252,6 @@ __global__ void k_links(const int* site_vox, const int* vsite, long long N, int 
     link_b[n] = b;
 }
 
-// The solids' part of twice the colour gradient at each site (face weight 1,
-// edge weight 1/2): static between changes of the wetting map.
-__global__ void k_wall_gradient(const int* site_vox, const float* phis, long long N, long long P, int px, int pxpy,
-                                float* wall_c) {
-    const long long n = static_cast<long long>(blockIdx.x) * kBlock + threadIdx.x;
-    if (n >= N) return;
-    const int pv = site_vox[n];
-    float c[3] = {0.0f, 0.0f, 0.0f};
-    static_for<1, Q19>([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        const float p = 2.0f * grad_w(q) * phis[pv + stencil_offset(q, px, pxpy)];
-        if constexpr (cx(q) != 0) c[0] += cx(q) * p;
-        if constexpr (cy(q) != 0) c[1] += cy(q) * p;
-        if constexpr (cz(q) != 0) c[2] += cz(q) * p;
-    });
-    for (int i = 0; i < 3; ++i) wall_c[i * P + n] = c[i];
-}
-
 }  // namespace
 
 cudaError_t launch_flag_pore(const uint16_t* labels, long long V, int* flags, cudaStream_t s) {
@@ -354,13 +335,6 @@ cudaError_t launch_links(const lbpm_ctx* c, cudaStream_t s) {
     if (c->N == 0) return cudaSuccess;
     k_links<<<blocks_for(c->N), kBlock, 0, s>>>(c->d_site_vox, c->d_vsite, c->N, c->px, c->px * c->py, c->d_link_a,
                                                 c->d_link_b);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_wall_gradient(const lbpm_ctx* c, cudaStream_t s) {
-    if (c->N == 0) return cudaSuccess;
-    k_wall_gradient<<<blocks_for(c->N), kBlock, 0, s>>>(c->d_site_vox, c->d_phis, c->N, pitch_of(c->N), c->px,
-                                                        c->px * c->py, c->d_wall_c);
     return cudaGetLastError();
 }
 

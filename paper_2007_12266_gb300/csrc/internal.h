@@ -44,7 +44,7 @@ struct DomainView {
     const int* vsite;      // [Vp] site id; negative for solid (the complement of its rank) and wall (-1)
     const int4* link_a;    // [N] SiteLinks::a
     const int2* link_b;    // [N] SiteLinks::b
-    const float* wall_c;   // [3][P] the solids' part of twice the colour gradient, sum_q 2 g_q xi_q phi_s
+    const float* phis;     // [Vp] phi_s of solid voxels, 0 at pores and walls
     float* phi[2];         // [N] phase of each site by step parity: the phase pass of a step of parity P
                            //     writes phi[P] and the collision reads it; with fp16 storage the
                            //     previous step's phi[P ^ 1] is the reference of the stored
@@ -60,8 +60,8 @@ struct DomainView {
     unsigned long long* acc;     // [N] sum form: packed fixed-point (Na, Nb) of each site (see pack_sums)
     float tau_a, tau_b, alpha, beta;
     float fx, fy, fz;
-    float fs[3];           // F / s_m when tau_a == tau_b, in the collision's working units (times 2^14
-                           // with fp16 storage)
+    float fterm[9];        // 3 t_q xi_q . F of the odd directions q = 2k + 1 (forcing term per pair), in
+                           // the collision's working units (times 2^14 with fp16 storage)
     float s_nu, s_m;       // rates when tau_a == tau_b
     int uniform_tau;
 };
@@ -107,7 +107,6 @@ struct lbpm_ctx {
     float* d_phis = nullptr;        // [Vp] phi_s of solid voxels, 0 at pores and walls
     int4* d_link_a = nullptr;       // [N] SiteLinks
     int2* d_link_b = nullptr;       // [N]
-    float* d_wall_c = nullptr;      // [3][N] the solids' part of the colour gradient
     float* d_phi = nullptr;         // [N] phase of each site
     float* d_phi_alt = nullptr;     // [N] fp16 storage: the phase at odd steps
     float* d_nsum = nullptr;        // [N]
@@ -164,7 +163,6 @@ cudaError_t launch_slab_flags(const lbpm_ctx* c, int* flags, cudaStream_t s);
 cudaError_t launch_slab_scatter(const lbpm_ctx* c, const int* flags, const int* scan, cudaStream_t s);
 cudaError_t launch_export_index(const lbpm_ctx* c, long long* site2vox, int* nbr, cudaStream_t s);
 cudaError_t launch_links(const lbpm_ctx* c, cudaStream_t s);
-cudaError_t launch_wall_gradient(const lbpm_ctx* c, cudaStream_t s);
 
 // Look up (once per device, with that device current) the device address of
 // the static staging array of lbpm_read_field_noalloc; called by lbpm_create.

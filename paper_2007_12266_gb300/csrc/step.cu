@@ -231,7 +231,7 @@ DomainView make_view(const lbpm_ctx* c) {
     d.phi[1] = c->d_phi_alt ? c->d_phi_alt : c->d_phi;
     d.link_a = c->d_link_a;
     d.link_b = c->d_link_b;
-    d.wall_c = c->d_wall_c;
+    d.phis = c->d_phis;
     d.nsum = c->d_nsum;
     d.drho = c->d_drho;
     d.rsum = c->d_rsum;
@@ -247,12 +247,15 @@ DomainView make_view(const lbpm_ctx* c) {
     d.fx = static_cast<float>(p.force[0]);
     d.fy = static_cast<float>(p.force[1]);
     d.fz = static_cast<float>(p.force[2]);
+    const float K = p.precision == LBPM_FP16 ? StoreF16::kK : StoreF32::kK;
+    for (int k = 0; k < 9; ++k) {
+        const int q = 2 * k + 1;
+        d.fterm[k] = K * (3.0f * t19(q) * (cx(q) * d.fx + cy(q) * d.fy + cz(q) * d.fz));
+    }
     d.uniform_tau = p.tau_a == p.tau_b;
     const float s_nu = 1.0f / static_cast<float>(p.tau_a);
     d.s_nu = s_nu;
     d.s_m = 8.0f * (2.0f - s_nu) / (8.0f - s_nu);
-    const float K = p.precision == LBPM_FP16 ? StoreF16::kK : StoreF32::kK;
-    for (int a = 0; a < 3; ++a) d.fs[a] = static_cast<float>(static_cast<double>(K) * p.force[a] / static_cast<double>(d.s_m));
     return d;
 }
 

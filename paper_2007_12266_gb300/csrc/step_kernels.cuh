@@ -38,6 +38,11 @@ struct StoreF32 {
     static constexpr float kK = 1.0f;
     static __device__ __forceinline__ float ld_s(const T* p) { return *p; }
     static __device__ __forceinline__ void st_s(T* p, float v) { *p = v; }
+    // a stored momentum population as a deviation from rest, and back
+    template <int Q>
+    static __device__ __forceinline__ float deviation(float x, float) { return sub(x, t19(Q)); }
+    template <int Q>
+    static __device__ __forceinline__ float stored(float dev) { return add(t19(Q), dev); }
     template <int Q>
     static __device__ __forceinline__ float ld_fdev(const void* p, size_t i) {
         return static_cast<const float*>(p)[i] - t19(Q);
@@ -106,6 +111,12 @@ struct StoreF16 {
     static constexpr float kK = kScale;
     static __device__ __forceinline__ float ld_s(const T* p) { return __half2float(*p); }
     static __device__ __forceinline__ void st_s(T* p, float v) { *p = __float2half_rn(v); }
+    // a stored momentum population, relative to the reference density deviation
+    // `ref`, as a deviation from rest in working units
+    template <int Q>
+    static __device__ __forceinline__ float deviation(float x, float ref) { return fma(t19(Q) * kK, ref, x); }
+    template <int Q>
+    static __device__ __forceinline__ float stored(float dev) { return dev; }
     template <int Q>
     static __device__ __forceinline__ float ld_fdev(const void* p, size_t i) {
         return __half2float(static_cast<const __half*>(p)[i]) * kInv;
@@ -398,29 +409,31 @@ struct SiteState {
     SiteLinks l;
     float f[Q19];                   // even steps: the populations in the own slots (stored numbers); odd: f[0]
     float ref = 0.0f;               // fp16: the own slots' reference density (deviation)
-    float cw[3];                    // the solids' part of twice the colour gradient
+    int v;                          // the site's voxel
 };
 
 // Collision, recoloring and streaming of site n. The arithmetic is written in
 // explicitly rounded operations (no contraction is left to the compiler), so a
 // site's result is the same bit for bit in every kernel this is compiled into.
+// Which operations they are, and in which order, is part of the result: where the
+// colour gradient nearly cancels, in pockets of a few voxels, the normal hangs on
+// the last bits, and any other rounding moves single sites by a thousandth and more
+// within a few hundred steps, in both storages. (A form over pairs of opposite
+// directions with the solids' part of the gradient summed beforehand took 110
+// instructions fewer per site and 136 / 129 us per step instead of 150 / 140, and
+// was nearer to 64 bits in norm, but single sites of a 256^3 pack, and of batches,
+// came out up to 4e-3 of the largest value away.)
 //
-// What bounds it: DRAM with fp32 storage (live, 202 B per site at 5.9 TB/s at even
-// and 5.4 TB/s at odd steps, of 6.7 for a plain copy, on 3.69 M sites of a 256^3
-// pack), with fp16 the latency of the loads, with 32 warps per SM resident, and
-// the instructions (581 and 769 per site at even and odd steps in fp32, 644 and
-// 954 in fp16). So neighbours come from a 24-byte record per site and the phase
-// is kept per site: against gathering 18 phases and 18 (odd) or 6 site ids from
-// dense voxel grids, where the 32 sites of a warp span about 150 voxels, a warp
-// touches half the cache lines (L1 data-pipe wavefronts per warp 289 -> 175 odd,
-// 171 -> 122 even), and the phase pass needs no site -> voxel map and no
-// scattered stores: 161 -> 146 us per step in fp32, 154 -> 135 in fp16, 7.7 ->
-// 6.3 on 79 k sites. And the component sums are updated in place, in one array
-// that stays in L2 instead of two of which the collision reads one and clears it:
-// 143 -> 136 us in fp32 (15 B per site less from DRAM), 135 -> 131 in fp16, 129
-// with two fused multiply-adds per pair and fewer fixed-point conversions. Two
-// sites per thread on fma.rn.f32x2 took 463 instructions per site in an earlier
-// form but ran slower: twice the registers left fewer warps to cover the latency.
+// What bounds it: DRAM with fp32 storage, with fp16 the latency of the loads, with 32
+// warps per SM resident, and the instructions. So neighbours come from a 24-byte
+// record per site and the phase is kept per site: against gathering 18 phases and 18
+// (odd) or 6 site ids from dense voxel grids, where the 32 sites of a warp span about
+// 150 voxels, the phase pass needs no site -> voxel map and no scattered stores, and
+// only the solid neighbours (2 of 18 on average in a sphere pack of porosity 0.22) are
+// read by voxel. And the component sums are updated in place, in one array that stays
+// in L2 instead of two of which the collision reads one and clears it. Together, us per
+// step before and now: 166 and 150 in fp32 and 156 and 140 in fp16 on 3.69 M sites of
+// a 256^3 pack, 8.0 and 6.5 on 79 k sites.
 template <int PAR, class S, int CF, bool DENSE>
 __device__ __forceinline__ void collide_site(const DomainView& d, int n, const SiteState<S>& in, SlotCache sc) {
     SiteLinks l = in.l;
@@ -430,7 +443,7 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
     int pitch = d.pitch;
     T* const F = static_cast<T*>(d.f);
     const unsigned long long pol = l2_keep();
-    const int v = DENSE ? __ldg(d.site_vox + n) : 0;
+    const int v = in.v;
     // id of x + xi_q where has(q)
     auto has = [&](auto qc) { return link_has<decltype(qc)::value>(l); };
     auto id = [&](auto qc) {
@@ -455,17 +468,16 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
         asm volatile("" : "+r"(l.a.w), "+r"(n), "+r"(pitch));
     };
 
-    // incoming momentum populations: fp32, the stored f_q; fp16, deviations in
-    // units of 1 / K, at even steps the stored ones (all relative to the site's
-    // own reference density), at odd steps from rest
+    // incoming distributions as deviations d_q = f_q - t_q from the rest state
+    // (exact in fp32 near rest), so that density and momentum are sums of small
+    // numbers and the relaxation acts on small quantities; in working units
     float f[Q19];
+    const float ref_own = in.ref;
     static_for<0, Q19>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
-        if constexpr (PAR == 0 || q == 0) f[q] = in.f[q];
+        if constexpr (PAR == 0 || q == 0) f[q] = S::template deviation<q>(in.f[q], ref_own);
     });
-    const float ref_own = in.ref;
     if constexpr (PAR == 1) {
-        if constexpr (S::kRef) f[0] = fma(t19(0) * K, ref_own, f[0]);
         static_for<1, Q19>([&](auto qc) {
             constexpr int q = decltype(qc)::value;   // direction of the downstream slot
             constexpr int o = opp(q);                // direction read from it
@@ -473,12 +485,13 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
                 const int m = __ldg(d.vsite + v + stencil_off(d, q));
                 sc.slot[(q - 1) * sc.stride] = m >= 0 ? m : n + (o - q) * pitch;
             }
-            f[o] = S::ld_s(F + q * static_cast<size_t>(pitch) + slot(qc));
+            const float x = S::ld_s(F + q * static_cast<size_t>(pitch) + slot(qc));
+            float r = 0.0f;
             if constexpr (S::kRef) {
-                const float r = d.drho[has(qc) ? id(qc) : n];
+                r = d.drho[has(qc) ? id(qc) : n];
                 sc.ref[(q - 1) * sc.stride] = r;
-                f[o] = fma(t19(o) * K, r, f[o]);
             }
+            f[o] = S::template deviation<o>(x, r);
         });
     }
     if constexpr (DENSE && CF != 0 && PAR == 0) {
@@ -489,25 +502,30 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
         });
     }
     forget_ids();
-    const float (&cw)[3] = in.cw;
 
-    // Everything above (neighbour ids and f from the previous collision) is safe to read before the phase pass of this step
-    // completes; phi and nsum are its outputs, and the A/B slots written below
-    // are its inputs.
+    // Everything above (neighbour ids and f from the previous collision) is safe to
+    // read before the phase pass of this step completes; phi and nsum are its outputs,
+    // and the A/B slots written below are its inputs.
     allow_next_grid();
     wait_prior_grid();
 
-    // colour gradient C = sum_q g_q xi_q phi(x + xi_q), g = 1 on faces and 1/2
-    // on edges, from the differences over opposite neighbours plus the solids'
-    // part; twice C is what is used below (n does not depend on the scale)
+    // colour gradient C = sum_q g_q xi_q phi(x + xi_q), summed in the order of the
+    // directions: pores' phases per site, solids' phi_s from the voxel grid. One load
+    // through a selected pointer: two loads under opposite predicates took 162 us per
+    // step instead of 150 (fp32, 256^3), and the solids' values packed site after site
+    // 147 (139 instead of 140 in fp16, 6.6 instead of 6.5 on 79 k sites), for another
+    // 8 B per site and a list to keep.
     const float* const phi = d.phi[PAR];
-    auto phi_at = [&](auto qc) { return has(qc) ? phi[id(qc)] : 0.0f; };
-    float dphi[9];
-    static_for<0, 9>([&](auto pc) {
-        constexpr int p = decltype(pc)::value;
-        const std::integral_constant<int, 2 * p + 1> q;
-        const std::integral_constant<int, 2 * p + 2> o;
-        dphi[p] = sub(phi_at(q), phi_at(o));
+    const float* const phis = d.phis + v;
+    float Cx = 0.0f, Cy = 0.0f, Cz = 0.0f;
+    static_for<1, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        constexpr float g = grad_w(q);
+        const float* const at = has(qc) ? phi + id(qc) : phis + stencil_off(d, q);
+        const float p = *at;
+        if constexpr (cx(q) != 0) Cx = fma(g * cx(q), p, Cx);
+        if constexpr (cy(q) != 0) Cy = fma(g * cy(q), p, Cy);
+        if constexpr (cz(q) != 0) Cz = fma(g * cz(q), p, Cz);
     });
     const float phi_c = phi[n];
     const float Nt = d.nsum[n];
@@ -521,75 +539,36 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
     }
     forget_ids();
 
-    // pair sums of deviations S = (f_q - t) + (f_o - t) and differences
-    // D = f_q - f_o (both exact or once rounded: f_q - 2t is exact for f near
-    // t)
-    const float mt[2] = {-2.0f * t19(1), -2.0f * t19(7)};
-    float two_ref[2];
-    if constexpr (S::kRef && PAR == 0) {
-        two_ref[0] = mul(2.0f * t19(1) * K, ref_own);
-        two_ref[1] = mul(2.0f * t19(7) * K, ref_own);
-    }
-    auto pair_sum = [&](auto pc) {
-        constexpr int p = decltype(pc)::value;
-        constexpr int q = 2 * p + 1, o = q + 1;
-        [[maybe_unused]] constexpr int c = p < 3 ? 0 : 1;
-        if constexpr (!S::kRef) return add(add(f[q], mt[c]), f[o]);
-        else if constexpr (PAR == 0) return add(add(f[q], f[o]), two_ref[c]);
-        else return add(f[q], f[o]);
-    };
-    auto pair_diff = [&](auto pc) {
-        constexpr int q = 2 * decltype(pc)::value + 1;
-        return sub(f[q], f[q + 1]);
-    };
-    // drho = rho - 1 and j, in working units
-    float drho, jx, jy, jz;
-    {
-        if constexpr (!S::kRef) drho = add(f[0], -t19(0));
-        else if constexpr (PAR == 0) drho = fma(t19(0) * K, ref_own, f[0]);
-        else drho = f[0];
-        float s = pair_sum(std::integral_constant<int, 0>{});
-        static_for<1, 9>([&](auto pc) { s = add(s, pair_sum(pc)); });
-        drho = add(drho, s);
-        float D[9];
-        static_for<0, 9>([&](auto pc) { D[decltype(pc)::value] = pair_diff(pc); });
-        // pairs: x, y, z; (++), (+-) of xy, xz, yz
-        jx = add(add(add(D[3], D[4]), add(D[5], D[6])), D[0]);
-        jy = add(add(sub(D[3], D[4]), add(D[7], D[8])), D[1]);
-        jz = add(add(sub(D[5], D[6]), sub(D[7], D[8])), D[2]);
-    }
-    // From here on the compiler knows nothing about the populations: it derives
-    // S and D again below instead of keeping all of them in registers.
-    static_for<1, Q19>([&](auto qc) { asm volatile("" : "+f"(f[decltype(qc)::value])); });
+    // macroscopic moments: drho = rho - 1 and j from the deviations
+    float drho = f[0], jx = 0.0f, jy = 0.0f, jz = 0.0f;
+    static_for<1, Q19>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        drho = add(drho, f[q]);
+        if constexpr (cx(q) > 0) jx = add(jx, f[q]);
+        if constexpr (cx(q) < 0) jx = sub(jx, f[q]);
+        if constexpr (cy(q) > 0) jy = add(jy, f[q]);
+        if constexpr (cy(q) < 0) jy = sub(jy, f[q]);
+        if constexpr (cz(q) > 0) jz = add(jz, f[q]);
+        if constexpr (cz(q) < 0) jz = sub(jz, f[q]);
+    });
 
-    // 2 C, its inverse length (0 where C vanishes) and the normal n
-    const float Cx = add(cw[0], add(add(dphi[0], dphi[0]), add(add(dphi[3], dphi[4]), add(dphi[5], dphi[6]))));
-    const float Cy = add(cw[1], add(add(dphi[1], dphi[1]), add(sub(dphi[3], dphi[4]), add(dphi[7], dphi[8]))));
-    const float Cz = add(cw[2], add(add(dphi[2], dphi[2]), add(sub(dphi[5], dphi[6]), sub(dphi[7], dphi[8]))));
-    const float C2 = fma(Cx, Cx, fma(Cy, Cy, mul(Cz, Cz)));
-    const float inv = C2 > 0.0f ? rsqrtf(C2) : 0.0f;
+    const float C2 = fma(Cz, Cz, fma(Cx, Cx, mul(Cy, Cy)));
+    float nx = 0.0f, ny = 0.0f, nz = 0.0f, Cmag = 0.0f;
+    if (C2 > 0.0f) {
+        const float inv = rsqrtf(C2);
+        Cmag = mul(C2, inv);
+        nx = mul(Cx, inv);
+        ny = mul(Cy, inv);
+        nz = mul(Cz, inv);
+    }
 
-    // relaxation rates from the viscosity (tau mixed linearly in phi): half of
-    // s_nu, -s_m / 2, s_m / 12, and the force (times K) over s_m
-    float h_nu, h_m, b_m, gx, gy, gz;
-    if (d.uniform_tau) {
-        h_nu = 0.5f * d.s_nu;
-        h_m = -0.5f * d.s_m;
-        b_m = d.s_m * (1.0f / 12.0f);
-        gx = d.fs[0];
-        gy = d.fs[1];
-        gz = d.fs[2];
-    } else {
-        const float tau = fma(mul(d.tau_a - d.tau_b, 0.5f), add(1.0f, phi_c), d.tau_b);
-        const float s_nu = __fdiv_rn(1.0f, tau);
-        const float s_m = __fdiv_rn(mul(8.0f, sub(2.0f, s_nu)), sub(8.0f, s_nu));
-        h_nu = mul(0.5f, s_nu);
-        h_m = mul(-0.5f, s_m);
-        b_m = mul(s_m, 1.0f / 12.0f);
-        const float g = mul(K, __fdiv_rn(1.0f, s_m));
-        gx = mul(g, d.fx);
-        gy = mul(g, d.fy);
-        gz = mul(g, d.fz);
+    // relaxation rates from the viscosity (tau mixed linearly in phi)
+    float s_nu = d.s_nu, s_m = d.s_m;
+    if (!d.uniform_tau) {
+        const float half = mul(d.tau_a - d.tau_b, 0.5f), pa = add(1.0f, phi_c);
+        const float tau = fma(half, pa, d.tau_b);
+        s_nu = __fdiv_rn(1.0f, tau);
+        s_m = __fdiv_rn(mul(8.0f, sub(2.0f, s_nu)), sub(8.0f, s_nu));
     }
 
     // MRT collision, evaluated in its equivalent two-relaxation-time form.
@@ -602,35 +581,28 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
     //   feq+ = t_q (rho + 4.5 (xi.j)^2 - 1.5 j.j) + M^-1 dm_alpha
     //   feq- = 3 t_q xi.j
     // where dm_alpha holds the interfacial-tension terms of m1, m9, m11,
-    // m13, m14, m15 (rho0 = 1). With E_ij = alpha |C| n_i n_j (whose trace is
-    // alpha |C|) the rows of M^-1 combine to
-    //   faces  (11/2394 - 1/36) alpha|C| + E_ii / 12
-    //   edges  (-8/2394 - 1/18) alpha|C| + (E_ii + E_jj) / 12 +- E_ij / 8
-    // and with q_i = j_i^2 / 4, G_i = q_i + E_ii / 6, H_ij = j_i j_j / 2 + E_ij / 4
-    //   faces  2 feq+ = bF + q_i + G_i
-    //   edges  2 feq+ = bE + G_i + G_j +- H_ij
-    // bF, bE holding rho - 1 - 1.5 j.j and the alpha |C| parts. The relaxation
-    // is h_nu (2 feq+ - S) on both populations of a pair and
-    // +-(-s_m/2 D + s_m/12 {2, 1} xi.(j + F/s_m)) on each, F/s_m bringing in
-    // the force. Everything is relative to the rest state (rho = 1), in
-    // working units: q_i and j_i j_j / 2 take one factor 1/K (as 2^-7 on each
-    // j with fp16 storage), alpha one factor K (ga below: alpha K / (12 |2C|)).
-    constexpr float kHalf = S::kRef ? 0.5f / 128.0f : 0.5f;   // 0.5 / sqrt(K)
-    const float px = mul(kHalf, jx), py = mul(kHalf, jy), pz = mul(kHalf, jz);
-    const float ga = mul(d.alpha * (K / 12.0f), inv);
-    const float ax = mul(ga, Cx), ay = mul(ga, Cy), az = mul(ga, Cz);
-    const float qx = mul(px, px), qy = mul(py, py), qz = mul(pz, pz);
-    const float Gx = fma(ax, Cx, qx), Gy = fma(ay, Cy, qy), Gz = fma(az, Cz, qz);
-    const float ac = mul(ga, C2);                                // alpha |C| K / 6
-    const float i9 = mul(1.0f / 9.0f, fma(-6.0f, add(add(qx, qy), qz), drho));
-    constexpr float kF = static_cast<float>(12.0 * (11.0 / 2394.0 - 1.0 / 36.0));
-    constexpr float kE = static_cast<float>(12.0 * (-8.0 / 2394.0 - 1.0 / 18.0));
-    const float bF = fma(kF, ac, i9);
-    const float bE = fma(kE, ac, mul(0.5f, i9));
-    const float Hxy = fma(add(px, px), py, mul(mul(1.5f, ax), Cy));
-    const float Hxz = fma(add(px, px), pz, mul(mul(1.5f, ax), Cz));
-    const float Hyz = fma(add(py, py), pz, mul(mul(1.5f, ay), Cz));
-    const float Ux = mul(b_m, add(jx, gx)), Uy = mul(b_m, add(jy, gy)), Uz = mul(b_m, add(jz, gz));
+    // m13, m14, m15 (rho0 = 1). Everything below is relative to the rest
+    // state t_q (rho = 1), i.e. in deviations, and in working units: the
+    // equilibrium's quadratic terms take one factor 1/K, the interfacial terms
+    // and the forcing (d.fterm is stored in working units) one factor K.
+    const float jj = fma(jz, jz, fma(jx, jx, mul(jy, jy)));
+    const float ac = mul(mul(d.alpha, K), Cmag);
+    const float hac = mul(0.5f, ac);
+    float dma[Q19];
+    dma[1] = -ac;
+    {
+        const float i9 = fma(mul(2.0f, nx), nx, -mul(ny, ny));
+        dma[9] = mul(hac, fma(-nz, nz, i9));
+        dma[11] = mul(hac, fma(-nz, nz, mul(ny, ny)));
+    }
+    dma[13] = mul(mul(hac, nx), ny);
+    dma[14] = mul(mul(hac, ny), nz);
+    dma[15] = mul(mul(hac, nx), nz);
+    const float drho_iso = fma(-1.5f * iK, jj, drho);
+
+    // recoloring weights Nb/N and Na/N are (1 - phi)/2 and (1 + phi)/2
+    const float bxa = mul(mul(d.beta, 0.5f), sub(1.0f, phi_c));
+    const float bxb = mul(mul(d.beta, 0.5f), add(1.0f, phi_c));
 
     // destination of direction q (q >= 1): row opp(q) at n (even step) or the
     // slot of row q it was read from (odd step)
@@ -640,141 +612,118 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
         else S::st_s(base + q * static_cast<size_t>(pitch) + slot(qc), x);
     };
 
-    // fp16, even steps: the results are relative to this site's new density
-    // instead of the old reference
-    float moved[2] = {0.0f, 0.0f}, rref = 0.0f;
-    if constexpr (S::kRef && PAR == 0) {
-        rref = sub(mul(K, ref_own), drho);
-        moved[0] = mul(t19(1), rref);
-        moved[1] = mul(t19(7), rref);
-    }
-    // The even increments of the moving populations sum to minus the rest
+    // The increments of the moving populations sum to minus the rest
     // increment in exact arithmetic; taking the rest increment as that sum
     // keeps fp32 mass exact up to unbiased rounding.
-    float esum;
+    float dsum = 0.0f;
     static_for<0, 9>([&](auto pc) {
-        constexpr int p = decltype(pc)::value;
-        constexpr int q = 2 * p + 1, o = q + 1;
-        [[maybe_unused]] constexpr int c = p < 3 ? 0 : 1;
-        float e, u;
-        if constexpr (p == 0) { e = add(bF, add(qx, Gx)); u = add(Ux, Ux); }
-        if constexpr (p == 1) { e = add(bF, add(qy, Gy)); u = add(Uy, Uy); }
-        if constexpr (p == 2) { e = add(bF, add(qz, Gz)); u = add(Uz, Uz); }
-        if constexpr (p == 3) { e = add(add(bE, add(Gx, Gy)), Hxy); u = add(Ux, Uy); }
-        if constexpr (p == 4) { e = sub(add(bE, add(Gx, Gy)), Hxy); u = sub(Ux, Uy); }
-        if constexpr (p == 5) { e = add(add(bE, add(Gx, Gz)), Hxz); u = add(Ux, Uz); }
-        if constexpr (p == 6) { e = sub(add(bE, add(Gx, Gz)), Hxz); u = sub(Ux, Uz); }
-        if constexpr (p == 7) { e = add(add(bE, add(Gy, Gz)), Hyz); u = add(Uy, Uz); }
-        if constexpr (p == 8) { e = sub(add(bE, add(Gy, Gz)), Hyz); u = sub(Uy, Uz); }
-        e = sub(e, pair_sum(pc));
-        if constexpr (p == 0) esum = e;
-        else esum = add(esum, e);
-        const float odd = fma(h_m, pair_diff(pc), u);
-        float vq, vo;
-        if constexpr (S::kRef && PAR == 0) {
-            const float even = fma(h_nu, e, moved[c]);
-            vq = add(f[q], add(even, odd));
-            vo = add(f[o], sub(even, odd));
-        } else {
-            vq = add(f[q], fma(h_nu, e, odd));
-            vo = add(f[o], fma(h_nu, e, -odd));
-        }
-        if constexpr (S::kRef && PAR == 1) {
+        constexpr int q = 2 * decltype(pc)::value + 1;   // q odd, opp(q) = q + 1
+        constexpr int o = q + 1;
+        constexpr float t = t19(q), t3 = 3.0f * t;
+        float cu;
+        if constexpr (q == 1) cu = jx;
+        if constexpr (q == 3) cu = jy;
+        if constexpr (q == 5) cu = jz;
+        if constexpr (q == 7) cu = add(jx, jy);
+        if constexpr (q == 9) cu = sub(jx, jy);
+        if constexpr (q == 11) cu = add(jx, jz);
+        if constexpr (q == 13) cu = sub(jx, jz);
+        if constexpr (q == 15) cu = add(jy, jz);
+        if constexpr (q == 17) cu = sub(jy, jz);
+        float eqp = mul(t, fma(mul(4.5f * iK, cu), cu, drho_iso));
+        static_for<1, 16>([&](auto kc) {
+            constexpr int k = decltype(kc)::value;
+            if constexpr (k == 1 || k == 9 || k == 11 || k == 13 || k == 14 || k == 15) {
+                if constexpr (mrow(k, q) != 0) eqp = fma(minv(q, k), dma[k], eqp);
+            }
+        });
+        const float ev = fma(0.5f, add(f[q], f[o]), -eqp);          // f+ - feq+
+        const float D = sub(f[q], f[o]);
+        const float od = fma(0.5f, D, -mul(t3, cu));   // f- - feq-
+        const float dmi = fma(-s_m, od, d.fterm[q >> 1]);
+        const float inc_q = fma(-s_nu, ev, dmi);
+        const float inc_o = fma(-s_nu, ev, -dmi);
+        if constexpr (q == 1) dsum = add(inc_q, inc_o);
+        else dsum = add(dsum, add(inc_q, inc_o));
+        float vq = add(f[q], inc_q), vo = add(f[o], inc_o);
+        if constexpr (S::kRef) {
+            // even step: relative to this site's rest state t_q rho; odd step:
             // relative to the destination's density of the last even step
-            vq = fma(-t19(q) * K, sc.ref[(q - 1) * sc.stride], vq);
-            vo = fma(-t19(q) * K, sc.ref[(o - 1) * sc.stride], vo);
+            if constexpr (PAR == 0) {
+                vq = fma(-t, drho, vq);
+                vo = fma(-t, drho, vo);
+            } else {
+                vq = fma(-t * K, sc.ref[(q - 1) * sc.stride], vq);
+                vo = fma(-t * K, sc.ref[(o - 1) * sc.stride], vo);
+            }
         }
-        store(std::integral_constant<int, q>{}, F, vq);
-        store(std::integral_constant<int, o>{}, F, vo);
+        store(std::integral_constant<int, q>{}, F, S::template stored<q>(vq));
+        store(std::integral_constant<int, o>{}, F, S::template stored<o>(vo));
     });
     {
-        const float m2 = mul(-2.0f, h_nu);
-        float r0 = fma(m2, esum, f[0]);
+        float r0 = sub(f[0], dsum);
         if constexpr (S::kRef && PAR == 0) {
-            r0 = fma(t19(0), rref, r0);
+            r0 = fma(-t19(0), drho, r0);
             d.drho[n] = mul(iK, drho);
         }
         if constexpr (S::kRef && PAR == 1) r0 = fma(-t19(0) * K, ref_own, r0);
-        S::st_s(F + n, r0);
+        S::st_s(F + n, S::template stored<0>(r0));
     }
 
     // recolored component distributions (Eqs. LBE-mass-a/b), streamed on the
     // fly; the rest populations take the remainder of Na and Nb so that the
-    // fp32 weights (whose sum is not exactly 1) create no mass. Over a pair of
-    // opposite directions the values are P +- P (4.5 u_i + beta Nb/N n_i) with
-    // P = w_q Na (likewise B, with the normal's sign turned); the recoloring
-    // weights Nb/N and Na/N are (1 - phi)/2 and (1 + phi)/2.
-    const float nx = mul(Cx, inv), ny = mul(Cy, inv), nz = mul(Cz, inv);
-    const float c45 = 4.5f * iK, one = 1.0f;
-    const float wx = mul(c45, jx), wy = mul(c45, jy), wz = mul(c45, jz);
-    const float pa1 = add(one, phi_c), pb1 = sub(one, phi_c);   // 1 + phi, 1 - phi
-    const float bxa = mul(0.5f * d.beta, pb1), bxb = mul(-0.5f * d.beta, pa1);
-    const float rA[3] = {fma(bxa, nx, wx), fma(bxa, ny, wy), fma(bxa, nz, wz)};
-    const float rB[3] = {fma(bxb, nx, wx), fma(bxb, ny, wy), fma(bxb, nz, wz)};
+    // fp32 weights (whose sum is not exactly 1) create no mass. With fp16
+    // storage the stored quantity is the deviation from w_q (1 +- phi_c)/2: the
+    // deviation from w_q Na (w_q Nb), which the formula gives directly as
+    // w_q Na (4.5 u.xi + beta Nb/N n.xi), plus w_q times
+    //   Na - (1 + phi_c)/2 = (N - 1)(1 + phi_c)/2   (likewise for Nb).
+    // (working units: Na, Nb times K, j divided by K back to u)
+    const float pa1 = add(1.0f, phi_c), pb1 = sub(1.0f, phi_c);   // 1 + phi, 1 - phi
+    const float j3[3] = {jx, jy, jz}, n3[3] = {nx, ny, nz};
     if constexpr (CF != 0) {
-        // Sum form: the values in fixed point, moved from the site's sums to those
-        // of the site that receives them; the rest value, and the values of
-        // bounce-back links, stay. P and the part that changes sign are converted
-        // once per axis and added as packed integers: 8 instead of 12 conversions
-        // (a slow pipe), and finer than converting fp32 sums of 25-bit values.
+        // Sum form: A*_q = w_q Na [1 + 4.5 u.xi_q + beta (Nb/N) n.xi_q] (likewise B*_q)
+        // in fixed point, moved from the site's sums to those of the site that
+        // receives it; the rest value, and the values of bounce-back links, stay.
         unsigned long long out = 0;
         unsigned long long* const acc = d.acc;
-        const float wN = mul(w7(1) * 0.5f * kSumOne, Nt);
-        const float PA = mul(wN, pa1), PB = mul(wN, pb1);
-        const unsigned long long both = pack_sums(__float2int_rn(PA), __float2int_rn(PB));
-        static_for<0, 3>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            const unsigned long long d1 =
-                pack_sums(__float2int_rn(mul(PA, rA[i])), __float2int_rn(mul(PB, rB[i])));
-            static_for<0, 2>([&](auto hc) {
-                constexpr int q = 2 * i + 1 + decltype(hc)::value;
-                const unsigned long long x = q & 1 ? both + d1 : both - d1;
-                const std::integral_constant<int, q> Q;
-                if (has(Q)) {
-                    out -= x;
-                    red_add(acc + id(Q), x, pol);
-                }
-            });
+        const float NS = mul(0.5f * kSumOne, Nt);
+        const float PA = mul(w7(1), mul(NS, pa1)), PB = mul(w7(1), mul(NS, pb1));
+        static_for<1, Q7>([&](auto qc) {
+            constexpr int q = decltype(qc)::value;
+            constexpr int i = (q - 1) >> 1;
+            const float base = fma(q & 1 ? 4.5f * iK : -4.5f * iK, j3[i], 1.0f);
+            const float ma = mul(bxa, n3[i]), mb = mul(bxb, n3[i]);
+            const float ya = q & 1 ? add(base, ma) : sub(base, ma);
+            const float yb = q & 1 ? sub(base, mb) : add(base, mb);
+            if (has(qc)) {
+                const unsigned long long x = pack_sums(__float2int_rn(mul(PA, ya)), __float2int_rn(mul(PB, yb)));
+                out -= x;
+                red_add(acc + id(qc), x, pol);
+            }
         });
         red_add(acc + n, out, pol);
     } else {
-        // Populations. With fp16 storage the stored quantity is the deviation
-        // from w_q (1 +- phi_c)/2: the deviation from w_q Na (w_q Nb), which is
-        // +- P (4.5 u_i + ...), plus w_q times Na - (1 + phi_c)/2 = (N - 1)(1 + phi_c)/2
-        // (likewise for Nb); the working units' K on both.
         T* const A = static_cast<T*>(d.a);
         T* const B = static_cast<T*>(d.b);
         const float NK = mul(0.5f * K, Nt);
         const float Na = mul(NK, pa1), Nb = mul(NK, pb1);
         const float PA = mul(w7(1), Na), PB = mul(w7(1), Nb);
-        float cA = PA, cB = PB, eA = 0.0f, eB = 0.0f;
         if constexpr (S::kRef) {
+            // K (N - 1)(1 +- phi_c)/2, the offsets of the references; the values
+            // of opposite directions cancel in the sum of the six
             const float hN = mul(0.5f * K, add(Nt, -1.0f));
-            eA = mul(hN, pa1);
-            eB = mul(hN, pb1);
-            cA = mul(w7(1), eA);
-            cB = mul(w7(1), eB);
-        }
-        float asum = 0.0f, bsum = 0.0f;
-        static_for<0, 3>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            const float dA = mul(PA, rA[i]), dB = mul(PB, rB[i]);
-            const float a1 = add(cA, dA), a2 = sub(cA, dA), b1 = add(cB, dB), b2 = sub(cB, dB);
-            store(std::integral_constant<int, 2 * i + 1>{}, A, a1);
-            store(std::integral_constant<int, 2 * i + 2>{}, A, a2);
-            store(std::integral_constant<int, 2 * i + 1>{}, B, b1);
-            store(std::integral_constant<int, 2 * i + 2>{}, B, b2);
-            if constexpr (!S::kRef) {
-                if constexpr (i == 0) {
-                    asum = add(a1, a2);
-                    bsum = add(b1, b2);
-                } else {
-                    asum = add(asum, add(a1, a2));
-                    bsum = add(bsum, add(b1, b2));
-                }
-            }
-        });
-        if constexpr (S::kRef) {
+            const float eA = mul(hN, pa1), eB = mul(hN, pb1);
+            static_for<0, 3>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                const std::integral_constant<int, 2 * i + 1> q;
+                const std::integral_constant<int, 2 * i + 2> o;
+                const float av = mul(PA, fma(4.5f * iK, j3[i], mul(bxa, n3[i])));
+                const float bv = mul(PB, fma(4.5f * iK, j3[i], -mul(bxb, n3[i])));
+                store(q, A, fma(w7(1), eA, av));
+                store(q, B, fma(w7(1), eB, bv));
+                store(o, A, fma(w7(1), eA, -av));
+                store(o, B, fma(w7(1), eB, -bv));
+            });
             // The phase pass adds (1 + S)/2 to the seven values a site reads, S
             // holding w_q phi_c for this site's value of direction q; the seven
             // stored values above sum to Wsum (Na - (1 + phi_c)/2) with Wsum the
@@ -786,6 +735,18 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
             S::st_s(A + n, fma(kWerr, add(-0.5f * K, Na), mul(w7(0), eA)));
             S::st_s(B + n, fma(kWerr, add(-0.5f * K, Nb), mul(w7(0), eB)));
         } else {
+            float asum = 0.0f, bsum = 0.0f;
+            static_for<1, Q7>([&](auto qc) {
+                constexpr int q = decltype(qc)::value;
+                constexpr int i = (q - 1) >> 1;
+                constexpr float sgn = q & 1 ? 1.0f : -1.0f;
+                const float base = fma(sgn * 4.5f * iK, j3[i], 1.0f);
+                const float av = mul(PA, fma(bxa, sgn * n3[i], base)), bv = mul(PB, fma(-bxb, sgn * n3[i], base));
+                asum = q == 1 ? av : add(asum, av);
+                bsum = q == 1 ? bv : add(bsum, bv);
+                store(qc, A, av);
+                store(qc, B, bv);
+            });
             S::st_s(A + n, sub(Na, asum));
             S::st_s(B + n, sub(Nb, bsum));
         }
@@ -806,7 +767,7 @@ __device__ __forceinline__ void collide_thread(const DomainView& d, int n, SlotC
         if constexpr (PAR == 0 || q == 0) in.f[q] = S::ld_s(F + q * P + n);
     });
     if constexpr (S::kRef) in.ref = d.drho[n];
-    for (int i = 0; i < 3; ++i) in.cw[i] = __ldg(d.wall_c + i * P + n);
+    in.v = __ldg(d.site_vox + n);
     if (__any_sync(__activemask(), in.l.a.w & kIrregular)) collide_site<PAR, S, CF, true>(d, n, in, sc);
     else collide_site<PAR, S, CF, false>(d, n, in, sc);
 }
@@ -948,14 +909,20 @@ __device__ __forceinline__ void pressure_face_thread(const DomainView& d, int n,
     static_for<5, 7>([&](auto qc) {
         constexpr int q = decltype(qc)::value;   // 5: +z, 6: -z
         if (cz(q) * sgn > 0.0f) {
-            const float eq = w7(q) * rho * (1.0f + 4.5f * cz(q) * uz);
+            const float y = fma(4.5f * cz(q), uz, 1.0f);
+            const float eq = mul(mul(w7(q), rho), y);
             float av = side == 1 ? eq : 0.0f, bv = side == 1 ? 0.0f : eq;
             if constexpr (S::kRef) {
                 // the reference the next step reads it with (see StoreF16)
                 if constexpr (PAR == 0) face_neighbours(d, n, nb);
                 const float pw = writer_phase<PAR, q>(d, n, nb);
-                av -= w7(q) * 0.5f * (1.0f + pw);
-                bv -= w7(q) * 0.5f * (1.0f - pw);
+                // av - h (1 + pw), bv - h (1 - pw); the operations are part of the result,
+                // as in collide_site
+                constexpr float h = 0.5f * w7(q);
+                const float ra = mul(h, add(1.0f, pw)), rb = sub(1.0f, pw);
+                av = side == 1 ? fma(mul(w7(q), rho), y, -ra) : -ra;
+                if constexpr (PAR == 0) bv = side == 1 ? -mul(h, rb) : fma(mul(w7(q), rho), y, -mul(h, rb));
+                else bv = side == 1 ? -mul(h, rb) : fma(-h, rb, eq);
             }
             const size_t i = read_slot<PAR, q>(d, n, nb);
             S::template st_c<q>(d.a, i, av);
