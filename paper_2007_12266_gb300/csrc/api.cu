@@ -65,13 +65,10 @@ void free_state(lbpm_ctx* c) {
     dfree(c, c->d_b);
     dfree(c, c->d_nsum);
     dfree(c, c->d_drho);
-    dfree(c, c->d_phi);
-    dfree(c, c->d_phi_alt);
     dfree(c, c->d_rsum);
     dfree(c, c->d_acc);
     c->d_acc = nullptr;
     c->d_drho = nullptr;
-    c->d_phi = c->d_phi_alt = nullptr;
     c->d_rsum = nullptr;
     c->d_f = c->d_a = c->d_b = nullptr;
     c->d_nsum = nullptr;
@@ -83,7 +80,7 @@ void free_image(lbpm_ctx* c) {
     dfree(c, c->d_labels);
     dfree(c, c->d_site_vox);
     dfree(c, c->d_vsite);
-    dfree(c, c->d_phis);
+    dfree(c, c->d_phases);
     dfree(c, c->d_link_a);
     dfree(c, c->d_link_b);
     c->d_link_a = nullptr;
@@ -96,7 +93,7 @@ void free_image(lbpm_ctx* c) {
     c->d_face_rho = nullptr;
     c->d_labels = nullptr;
     c->d_site_vox = c->d_vsite = c->d_slab_site = nullptr;
-    c->d_phis = nullptr;
+    c->d_phases = c->d_phis = c->d_phi = c->d_phi_alt = nullptr;
     c->d_slab_side = nullptr;
     c->N = c->n_slab = 0;
     c->have_image = false;
@@ -107,6 +104,29 @@ size_t state_bytes(const lbpm_ctx* c, int q) {
     return e * static_cast<size_t>(q) * static_cast<size_t>(pitch_of(c->N));
 }
 
+// The phases of the sites and the grid of phi_s in one block (see DomainView::phis_at);
+// the grid's values are kept when the storage changes.
+lbpm_status alloc_phases(lbpm_ctx* c) {
+    const size_t P = static_cast<size_t>(pitch_of(c->N)), G = static_cast<size_t>(pitch_of(c->Vp));
+    const size_t alt = c->params.precision == LBPM_FP16 ? P : 0;
+    float* const block = static_cast<float*>(dalloc(c, sizeof(float) * (alt + G + P)));
+    if (!block) return fail(c, LBPM_E_OOM, "device allocation of the phases failed");
+    if (c->d_phases) {
+        const cudaError_t e = cudaMemcpyAsync(block + alt, c->d_phis, sizeof(float) * c->Vp, cudaMemcpyDeviceToDevice,
+                                              c->stream);
+        if (e != cudaSuccess) {
+            dfree(c, block);
+            return fail_cuda(c, "copy of the solids' phases", e);
+        }
+        dfree(c, c->d_phases);
+    }
+    c->d_phases = block;
+    c->d_phi_alt = alt ? block : nullptr;
+    c->d_phis = block + alt;
+    c->d_phi = c->d_phis + G;
+    return LBPM_OK;
+}
+
 lbpm_status alloc_state(lbpm_ctx* c) {
     free_state(c);
     c->d_f = dalloc(c, state_bytes(c, 19));
@@ -115,13 +135,11 @@ lbpm_status alloc_state(lbpm_ctx* c) {
     const size_t P = static_cast<size_t>(pitch_of(c->N));
     c->d_nsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
     c->d_acc = static_cast<unsigned long long*>(dalloc(c, sizeof(unsigned long long) * P));
-    c->d_phi = static_cast<float*>(dalloc(c, sizeof(float) * P));
-    bool ok = c->d_f && c->d_a && c->d_b && c->d_nsum && c->d_acc && c->d_phi;
+    bool ok = c->d_f && c->d_a && c->d_b && c->d_nsum && c->d_acc;
     if (c->params.precision == LBPM_FP16) {
         c->d_drho = static_cast<float*>(dalloc(c, sizeof(float) * P));
         c->d_rsum = static_cast<float*>(dalloc(c, sizeof(float) * P));
-        c->d_phi_alt = static_cast<float*>(dalloc(c, sizeof(float) * P));
-        ok = ok && c->d_drho && c->d_rsum && c->d_phi_alt;
+        ok = ok && c->d_drho && c->d_rsum;
         // a state restored without an initialisation takes its references from these
         if (ok && (cudaMemsetAsync(c->d_phi, 0, sizeof(float) * P, c->stream) != cudaSuccess ||
                    cudaMemsetAsync(c->d_phi_alt, 0, sizeof(float) * P, c->stream) != cudaSuccess))
@@ -471,6 +489,10 @@ lbpm_status lbpm_set_params(lbpm_ctx* c, const lbpm_params* p) {
         if (per_changed) c->have_fluids = false;
     }
     if (old.precision != p->precision) {
+        if ((s = alloc_phases(c))) {
+            free_state(c);
+            return s;
+        }
         if ((s = alloc_state(c))) return s;
     }
     return LBPM_OK;
@@ -522,8 +544,7 @@ lbpm_status lbpm_load_image(lbpm_ctx* c, const uint16_t* labels, int nx, int ny,
     }
     c->d_site_vox = static_cast<int*>(dalloc(c, sizeof(int) * pitch_of(c->N)));
     c->d_vsite = static_cast<int*>(dalloc(c, sizeof(int) * c->Vp));
-    c->d_phis = static_cast<float*>(dalloc(c, sizeof(float) * c->Vp));
-    if (!c->d_site_vox || !c->d_vsite || !c->d_phis) {
+    if (!c->d_site_vox || !c->d_vsite || alloc_phases(c) != LBPM_OK) {
         dfree(c, flags);
         dfree(c, scan);
         return fail(c, LBPM_E_OOM, "device allocation of the index failed");

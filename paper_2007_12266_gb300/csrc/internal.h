@@ -44,11 +44,13 @@ struct DomainView {
     const int* vsite;      // [Vp] site id; negative for solid (the complement of its rank) and wall (-1)
     const int4* link_a;    // [N] SiteLinks::a
     const int2* link_b;    // [N] SiteLinks::b
-    const float* phis;     // [Vp] phi_s of solid voxels, 0 at pores and walls
     float* phi[2];         // [N] phase of each site by step parity: the phase pass of a step of parity P
                            //     writes phi[P] and the collision reads it; with fp16 storage the
                            //     previous step's phi[P ^ 1] is the reference of the stored
                            //     components (with fp32 storage both point to one array)
+    unsigned phis_at[2];   // where the grid of phi_s (phi_s of solid voxels, 0 at pores and walls) lies
+                           //     relative to phi[P], in entries modulo 2^32: behind phi[1] with fp16
+                           //     storage, otherwise before
     float* nsum;           // [N] Na + Nb of the current step (phase pass -> collision)
     float* rsum;           // [N] fp16 store: sum_q w_q phi_w(q) of the component references that the
                            //     next phase pass reads (collision -> phase pass, see StoreF16)
@@ -104,6 +106,7 @@ struct lbpm_ctx {
     uint16_t* d_labels = nullptr;   // [V]
     int* d_site_vox = nullptr;      // [N]
     int* d_vsite = nullptr;         // [Vp]
+    float* d_phases = nullptr;      // one block: d_phi_alt (fp16 storage), d_phis, d_phi
     float* d_phis = nullptr;        // [Vp] phi_s of solid voxels, 0 at pores and walls
     int4* d_link_a = nullptr;       // [N] SiteLinks
     int2* d_link_b = nullptr;       // [N]

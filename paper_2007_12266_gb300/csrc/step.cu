@@ -231,7 +231,7 @@ DomainView make_view(const lbpm_ctx* c) {
     d.phi[1] = c->d_phi_alt ? c->d_phi_alt : c->d_phi;
     d.link_a = c->d_link_a;
     d.link_b = c->d_link_b;
-    d.phis = c->d_phis;
+    for (int k = 0; k < 2; ++k) d.phis_at[k] = static_cast<unsigned>(c->d_phis - d.phi[k]);
     d.nsum = c->d_nsum;
     d.drho = c->d_drho;
     d.rsum = c->d_rsum;

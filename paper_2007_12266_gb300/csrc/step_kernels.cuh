@@ -419,21 +419,24 @@ struct SiteState {
 // colour gradient nearly cancels, in pockets of a few voxels, the normal hangs on
 // the last bits, and any other rounding moves single sites by a thousandth and more
 // within a few hundred steps, in both storages. (A form over pairs of opposite
-// directions with the solids' part of the gradient summed beforehand took 110
-// instructions fewer per site and 136 / 129 us per step instead of 150 / 140, and
-// was nearer to 64 bits in norm, but single sites of a 256^3 pack, and of batches,
-// came out up to 4e-3 of the largest value away.)
+// directions with the solids' part of the gradient summed beforehand took a hundred
+// instructions fewer per site and 137 / 130 us per step (fp32 / fp16) instead of 151 /
+// 136, and was nearer to 64 bits in norm, but single sites of a 256^3 pack, and of
+// batches, came out up to 4e-3 of the largest value away.)
 //
 // What bounds it: DRAM with fp32 storage, with fp16 the latency of the loads, with 32
-// warps per SM resident, and the instructions. So neighbours come from a 24-byte
+// warps per SM resident, and the instructions (689 and 870 per site at even and odd
+// steps in fp32, 738 and 1043 in fp16). So neighbours come from a 24-byte
 // record per site and the phase is kept per site: against gathering 18 phases and 18
 // (odd) or 6 site ids from dense voxel grids, where the 32 sites of a warp span about
 // 150 voxels, the phase pass needs no site -> voxel map and no scattered stores, and
 // only the solid neighbours (2 of 18 on average in a sphere pack of porosity 0.22) are
 // read by voxel. And the component sums are updated in place, in one array that stays
 // in L2 instead of two of which the collision reads one and clears it. Together, us per
-// step before and now: 166 and 150 in fp32 and 156 and 140 in fp16 on 3.69 M sites of
-// a 256^3 pack, 8.0 and 6.5 on 79 k sites.
+// step before and now: 167 and 151 in fp32 and 157 and 136 in fp16 on 3.69 M sites of
+// a 256^3 pack, 8.1 and 6.3 in fp32 on 79 k sites. Not everywhere a gain in fp32: on
+// 734 k sites with a periodic x axis 29.2 and 30.8, on 1.02 M 44.7 and 46.3, where the
+// step runs out of L2 and 36 instead of 32 warps cover its latency better.
 template <int PAR, class S, int CF, bool DENSE>
 __device__ __forceinline__ void collide_site(const DomainView& d, int n, const SiteState<S>& in, SlotCache sc) {
     SiteLinks l = in.l;
@@ -510,19 +513,19 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
     wait_prior_grid();
 
     // colour gradient C = sum_q g_q xi_q phi(x + xi_q), summed in the order of the
-    // directions: pores' phases per site, solids' phi_s from the voxel grid. One load
-    // through a selected pointer: two loads under opposite predicates took 162 us per
-    // step instead of 150 (fp32, 256^3), and the solids' values packed site after site
-    // 147 (139 instead of 140 in fp16, 6.6 instead of 6.5 on 79 k sites), for another
-    // 8 B per site and a list to keep.
+    // directions: pores' phases per site, solids' phi_s from the voxel grid, which lies
+    // within 32-bit reach of the phases so that one load takes either, at a selected
+    // index. On 256^3 in fp32 / fp16: 151 / 136 us per step; loads under opposite
+    // predicates took 162 / 145, one through a selected pointer 151 / 141, the solids'
+    // values packed site after site (8 B per site more) 147 / 139.
     const float* const phi = d.phi[PAR];
-    const float* const phis = d.phis + v;
+    const unsigned vs = static_cast<unsigned>(v) + d.phis_at[PAR];
     float Cx = 0.0f, Cy = 0.0f, Cz = 0.0f;
     static_for<1, Q19>([&](auto qc) {
         constexpr int q = decltype(qc)::value;
         constexpr float g = grad_w(q);
-        const float* const at = has(qc) ? phi + id(qc) : phis + stencil_off(d, q);
-        const float p = *at;
+        const unsigned i = has(qc) ? static_cast<unsigned>(id(qc)) : vs + static_cast<unsigned>(stencil_off(d, q));
+        const float p = S::kRef && PAR == 1 ? phi[i] : phi[static_cast<int>(i)];
         if constexpr (cx(q) != 0) Cx = fma(g * cx(q), p, Cx);
         if constexpr (cy(q) != 0) Cy = fma(g * cy(q), p, Cy);
         if constexpr (cz(q) != 0) Cz = fma(g * cz(q), p, Cz);

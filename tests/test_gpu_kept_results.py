@@ -111,3 +111,24 @@ def test_results_are_kept(case):
     with open(GOLDEN) as f:
         golden = json.load(f)
     assert checksums(*case[1:]) == golden[case[0]]
+
+
+@pytest.mark.parametrize("first", ["fp32", "fp16"])
+def test_storage_changed_on_the_way(first):
+    """A domain whose storage is changed keeps its wetting map: the recorded results of the other storage."""
+    import paper_2007_12266_gb300 as lbm
+    second = "fp16" if first == "fp32" else "fp32"
+    lab = _image()
+    aff = ((1.8 * _uniform(lab.size, 3) - 0.9).reshape(SHAPE) * (lab != 0)).astype(np.float32)
+    phi0 = np.where(_uniform(lab.size, 4).reshape(SHAPE) < 0.5, 1.0, -1.0).astype(np.float32)
+    kw = dict(tau_a=0.8, tau_b=0.8, alpha=0.01, beta=0.95, **FLOWS["walls"])
+    d = lbm.Domain(lab, aff, precision=first, **kw)
+    d.init_fluids(phi0)
+    d.advance(3)
+    d.set_params(precision=second, **kw)
+    d.init_fluids(phi0)
+    d.advance(1)
+    with open(GOLDEN) as f:
+        golden = json.load(f)[f"{second} walls auto"][0]
+    assert [zlib.crc32(np.ascontiguousarray(d.distributions(k)).tobytes()) for k in ("f", "a", "b")] == golden
+    d.close()
