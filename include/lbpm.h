@@ -330,9 +330,11 @@ lbpm_status lbpm_kernel_timing(lbpm_ctx* ctx, double* ms_collide, long long* n_c
 /*
  * Batched form: several jobs (independent contexts on one GPU, same storage
  * precision) advanced together. With the default launch shape, jobs of 81920
- * sites or more on average and every job in the sum form, each job's steps are
- * a chain of launches of its own, three of them in flight at a time (on streams
- * that start after the earlier work of the batch's stream, which waits for them).
+ * sites or more on average, few that are much smaller among them (counting each
+ * job as at least 81920 sites adds no more than a quarter) and every job in the
+ * sum form, each job's steps are a chain of launches of its own, three of them in
+ * flight at a time (on streams that start after the earlier work of the batch's
+ * stream, which waits for them).
  * Otherwise every timestep of the whole batch is ONE launch of the phase pass and ONE of the fused collide-stream kernel, both
  * over a list of tiles that covers all jobs' sites (or, with the fused launch
  * shape of lbpm_batch_set_launch, one kernel runs every pass of a bundle);

@@ -395,11 +395,22 @@ lbpm_status batch_advance_sum(lbpm_batch* b, long long nsteps) {
 // which 32 of 83 k do not (calls of 2, 8, 16 steps: 133 and 128, 122 and 118, 120 and
 // 116), so the line lies between. One, two and four streams: 217, 192, 193 against
 // 190 us on the second set.
+// Small jobs among large ones: their launches wait for the large jobs' blocks, some
+// 7 us a step where one of 8 k sites alone takes 3, so the form is taken only while
+// counting each job as at least kByJobMean sites adds no more than a quarter. One
+// launch per pass and job by job, fp32: 12 of 100 k and one of 8 k sites (adds 6 %)
+// 56 and 42, six of 200 k and 12 of 50 k (23 %) 81 and 64, four of 500 k and four of
+// 8 k (15 %) 90 and 77, two of 2 M and ten of 8 k (19 %) 176 and 183; but two of 2 M
+// and twenty of 8 k (37 %) 179 and 218, and forty (74 %) 187 and 283. Weighing the
+// streams by that count instead of by sites leaves 219 of the 283.
 bool by_job(const lbpm_batch* b) {
     if (b->bt != 192 || b->bps[0] != -1 || b->bps[1] != -1) return false;
-    long long n = 0;
-    for (const lbpm_ctx* c : b->jobs) n += c->N;
-    return n >= kByJobMean * static_cast<long long>(b->jobs.size()) && batch_sum_form(b);
+    long long n = 0, counted = 0;
+    for (const lbpm_ctx* c : b->jobs) {
+        n += c->N;
+        counted += std::max(c->N, kByJobMean);
+    }
+    return n >= kByJobMean * static_cast<long long>(b->jobs.size()) && 4 * counted <= 5 * n && batch_sum_form(b);
 }
 
 // lbpm_batch_advance job by job: each job's whole run is a chain of its own (the
