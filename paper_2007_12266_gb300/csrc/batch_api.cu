@@ -381,9 +381,9 @@ lbpm_status batch_advance_sum(lbpm_batch* b, long long nsteps) {
     return LBPM_OK;
 }
 
-// Whether the batch runs job by job (batch_advance_jobs) instead of one launch per
-// pass over all jobs: with the default launch shape, in the sum form, and with jobs
-// large enough that two or three fill the GPU. A pass over all jobs leaves nothing of
+// Whether the batch, with the default launch shape, runs job by job
+// (batch_advance_jobs) instead of one launch per pass over all jobs: in the sum form,
+// and with jobs large enough that two or three fill the GPU. A pass over all jobs leaves nothing of
 // a job in L2 for the next pass, where a job of some 100 k sites keeps its whole state
 // there from step to step; and the chains cover each other's tails, where a pass ends
 // for all jobs at once. Us per step of one launch per pass (256 threads) and job by
@@ -403,8 +403,7 @@ lbpm_status batch_advance_sum(lbpm_batch* b, long long nsteps) {
 // 8 k (15 %) 90 and 77, two of 2 M and ten of 8 k (19 %) 176 and 183; but two of 2 M
 // and twenty of 8 k (37 %) 179 and 218, and forty (74 %) 187 and 283. Weighing the
 // streams by that count instead of by sites leaves 219 of the 283.
-bool by_job(const lbpm_batch* b) {
-    if (b->bt != 192 || b->bps[0] != -1 || b->bps[1] != -1) return false;
+bool jobs_alone(const lbpm_batch* b) {
     long long n = 0, counted = 0;
     for (const lbpm_ctx* c : b->jobs) {
         n += c->N;
@@ -412,6 +411,9 @@ bool by_job(const lbpm_batch* b) {
     }
     return n >= kByJobMean * static_cast<long long>(b->jobs.size()) && 4 * counted <= 5 * n && batch_sum_form(b);
 }
+
+// whether it does so with the launch shape it has
+bool by_job(const lbpm_batch* b) { return b->bt == 192 && b->bps[0] == -1 && b->bps[1] == -1 && jobs_alone(b); }
 
 // lbpm_batch_advance job by job: each job's whole run is a chain of its own (the
 // single-domain launches and graphs) on one of kJobStreams streams, the largest
@@ -448,7 +450,8 @@ lbpm_status batch_advance_jobs(lbpm_batch* b, long long nsteps) {
     return st;
 }
 
-// launch-shape cache: (gpu, precision, log2 of the site count) -> (bt, bps0, bps1)
+// launch-shape cache: (gpu, precision, log2 of the site count, whether the default shape
+// means job by job) -> (bt, bps0, bps1)
 std::mutex g_tune_mu;
 std::map<std::string, std::vector<int>> g_tune_cache;
 
@@ -459,7 +462,8 @@ std::string tune_key(const lbpm_batch* b) {
     for (const lbpm_ctx* c : b->jobs) n += c->N;
     int lg = 0;
     while ((1LL << (lg + 1)) <= n) ++lg;
-    return std::string(p.name) + "/" + std::to_string(b->precision) + "/" + std::to_string(lg);
+    return std::string(p.name) + "/" + std::to_string(b->precision) + "/" + std::to_string(lg) +
+           (jobs_alone(b) ? "/jobs" : "");
 }
 
 }  // namespace
