@@ -346,7 +346,10 @@ lbpm_status lbpm_kernel_timing(lbpm_ctx* ctx, double* ms_collide, long long* n_c
  * (lbpm_measure, lbpm_read_field, ...) stays valid; a job joins at an even
  * step and must be removed before it is destroyed. After changing a job's
  * parameters, call lbpm_batch_refresh. Work runs on the batch's stream: use
- * the same stream for the jobs, or synchronise them.
+ * the same stream for the jobs, or synchronise them. A call that runs job by job
+ * and fails for want of memory has advanced no job; where a launch fails, the job it
+ * belongs to is flagged unstable (re-initialise or restore it), and
+ * lbpm_step_count tells which of the others were advanced.
  */
 typedef struct lbpm_batch lbpm_batch;
 

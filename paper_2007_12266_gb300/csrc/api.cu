@@ -700,10 +700,9 @@ lbpm_status advance_job(lbpm_ctx* c, long long nsteps, cudaStream_t s, long long
 }
 
 lbpm_status capture_job(lbpm_ctx* c, long long nsteps) {
-    const int sizes[2] = {2, 16};
-    for (int gi = 0; gi < 2; ++gi)   // first, second and last step are plain launches
-        if (nsteps - 3 >= sizes[gi] && !c->sum_graphs[gi])
-            LBPM_CK(c, capture_sum_bundle(c, sizes[gi], &c->sum_graphs[gi]));
+    const long long mid = nsteps - 3;   // first, second and last step are plain launches
+    if (mid >= 16 && !c->sum_graphs[1]) LBPM_CK(c, capture_sum_bundle(c, 16, &c->sum_graphs[1]));
+    if (mid > 0 && mid % 16 >= 2 && !c->sum_graphs[0]) LBPM_CK(c, capture_sum_bundle(c, 2, &c->sum_graphs[0]));
     return LBPM_OK;
 }
 

@@ -419,13 +419,19 @@ bool by_job(const lbpm_batch* b) { return b->bt == 192 && b->bps[0] == -1 && b->
 // single-domain launches and graphs) on one of kJobStreams streams, the largest
 // jobs first and each to the stream with the fewest sites so far. The batch's
 // stream is one of them; the others start after its earlier work, and it waits
-// for them at the end.
+// for them at the end. What can fail for want of memory, the graphs, is made for all
+// jobs before the first launch, so that such a failure leaves every job where it was.
+// A launch that fails all the same leaves its job inside a run, its populations stale:
+// that job is flagged unstable; those before it are advanced, those after it are not.
 lbpm_status batch_advance_jobs(lbpm_batch* b, long long nsteps) {
     for (int k = 0; k < kJobStreams - 1; ++k) {
         if (!b->job_stream[k]) LBPM_BCK(b, cudaStreamCreateWithFlags(&b->job_stream[k], cudaStreamNonBlocking));
         if (!b->job_done[k]) LBPM_BCK(b, cudaEventCreateWithFlags(&b->job_done[k], cudaEventDisableTiming));
     }
     if (!b->job_start) LBPM_BCK(b, cudaEventCreateWithFlags(&b->job_start, cudaEventDisableTiming));
+    lbpm_status st = LBPM_OK;
+    for (lbpm_ctx* c : b->jobs)
+        if ((st = capture_job(c, nsteps))) return bfail(b, st, c->err);
     std::vector<lbpm_ctx*> order(b->jobs.begin(), b->jobs.end());
     std::stable_sort(order.begin(), order.end(), [](const lbpm_ctx* x, const lbpm_ctx* y) { return x->N > y->N; });
     cudaStream_t stream[kJobStreams];
@@ -433,11 +439,11 @@ lbpm_status batch_advance_jobs(lbpm_batch* b, long long nsteps) {
     for (int k = 0; k < kJobStreams; ++k) stream[k] = k == 0 ? b->stream : b->job_stream[k - 1];
     LBPM_BCK(b, cudaEventRecord(b->job_start, b->stream));
     for (int k = 1; k < kJobStreams; ++k) LBPM_BCK(b, cudaStreamWaitEvent(stream[k], b->job_start, 0));
-    lbpm_status st = LBPM_OK;
     for (lbpm_ctx* c : order) {
         const long long k = std::min_element(sites, sites + kJobStreams) - sites;
         sites[k] += c->N;
         if ((st = advance_job(c, nsteps, stream[k], &b->launches))) {
+            c->unstable = true;
             bfail(b, st, c->err);
             break;
         }
