@@ -91,24 +91,26 @@ lbpm_status sfail(lbpm_server* s, lbpm_status st, const std::string& m) {
     return st;
 }
 
-// Device bytes of a job: state, index grids and the transient scans of the
-// indexer (the peak while the image is loaded).
+// Device bytes of a job at its largest, counted as api.cu allocates them: while the
+// image is indexed (scans beside the grids), while the reservoir sites are found, and
+// with its state while a voxel map is uploaded (affinities, initial phase). The scans'
+// sums, the analysis' partial sums and the batch's tables go into the 1 MiB and the
+// last terms.
 size_t estimate_footprint(const lbpm_job_spec& sp, long long n_pore) {
     const double V = static_cast<double>(sp.nx) * sp.ny * sp.nz;
-    const double Vp = (sp.nx + 2.0) * (sp.ny + 2.0) * (sp.nz + 2.0);
-    const double N = static_cast<double>(n_pore);
-    const double es = sp.params.precision == LBPM_FP16 ? 2.0 : 4.0;
+    const double Vp = static_cast<double>(lbm::pitch_of((sp.nx + 2LL) * (sp.ny + 2LL) * (sp.nz + 2LL)));
+    const double P = static_cast<double>(lbm::pitch_of(n_pore));
     const bool h = sp.params.precision == LBPM_FP16;
-    // populations, nsum (+ drho, rsum and the second phase grid with fp16 storage)
-    const double state = 33.0 * es * N + (h ? 12.0 : 4.0) * N + (h ? 4.0 * Vp : 0.0);
-    // labels, vsite, the solids' phase, site_vox. With the indexer's transient grids
-    // (freed before the state is allocated) this also covers, at porosities of rocks,
-    // the per-site records, phase and sums: at porosity 0.22 224 bytes per site in
-    // fp32 (estimated 213) and 170 in fp16 (173), at 0.35 211 (187) and 157 (140).
-    // A job for which it falls short waits, see lbpm_server_run.
-    const double grids = 2.0 * V + 8.0 * Vp + 5.0 * N;
-    const double transient = 8.0 * Vp;
-    return static_cast<size_t>(state + grids + transient + (1 << 20));
+    // labels, ids by voxel, voxels by site, phi_s with the phases (two with fp16 storage)
+    const double grids = 2.0 * V + 4.0 * Vp + 4.0 * P + 4.0 * Vp + (h ? 8.0 : 4.0) * P;
+    const double records = 24.0 * P;
+    // populations, N, component sums (fp16: rho - 1 and the references' sum)
+    const double state = 33.0 * (h ? 2.0 : 4.0) * P + 12.0 * P + (h ? 8.0 : 0.0) * P;
+    const double slabs = sp.params.reservoir_z ? 5.0 * std::min(P, 8.0 * sp.nx * sp.ny) : 0.0;
+    const double indexing = grids + 8.0 * V;
+    const double boundaries = grids + records + slabs + (sp.params.reservoir_z ? 8.0 * P : 0.0);
+    const double running = grids + records + slabs + state + 4.0 * V;
+    return static_cast<size_t>(std::max({indexing, boundaries, running}) + 0.05 * P + 0.01 * V) + (1 << 20);
 }
 
 lbpm_status build_job(lbpm_server* s, Job* j) {
