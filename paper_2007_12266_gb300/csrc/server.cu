@@ -51,6 +51,7 @@ struct Job {
     std::vector<float> affinity, phi0;
     long long n_pore = 0;
     size_t footprint = 0;
+    long long refused_at = -1;   // server's releases when the device last had no memory for the job
     int state = LBPM_JOB_QUEUED;
     lbpm_ctx* ctx = nullptr;
     double t_submit = 0, t_admit = 0, t_done = 0;
@@ -82,6 +83,7 @@ struct lbpm_server {
     std::map<long long, std::unique_ptr<Job>> jobs;
     long long site_updates = 0;
     std::deque<Job*> finished;   // retired jobs still holding device state, oldest first
+    long long releases = 0;      // jobs whose device state was given back so far
 };
 
 namespace {
@@ -133,6 +135,7 @@ void release_job_device(lbpm_server* s, Job* j) {
         lbpm_destroy(j->ctx);
         j->ctx = nullptr;
         s->used -= std::min(s->used, j->footprint);
+        ++s->releases;
     }
 }
 
@@ -263,19 +266,24 @@ lbpm_status lbpm_server_run(lbpm_server* s, int* n_running, int* n_queued, int* 
         }
         if (s->used + s->queue.front()->footprint > s->budget) break;
         Job* j = s->queue.front();
+        // not built again (image uploaded, indexed, given up) before memory was given
+        // back since the device refused it
+        if (j->refused_at == s->releases && !s->running.empty() && s->finished.empty()) break;
+        if (j->refused_at == s->releases && !s->finished.empty()) {
+            release_job_device(s, s->finished.front());
+            s->finished.pop_front();
+        }
         s->queue.pop_front();
         s->used += j->footprint;
         st = build_job(s, j);
         if (st == LBPM_E_OOM && !(s->running.empty() && s->finished.empty())) {
-            // the estimate fell short of what the device can give: the job waits
-            // for the others' memory (a finished job's at once)
+            // the device has less than the budget (other users): the job waits for the
+            // others' memory (a finished job's at once)
             if (j->ctx) release_job_device(s, j);
             else s->used -= j->footprint;
             s->err.clear();
             s->queue.push_front(j);
-            if (s->finished.empty()) break;
-            release_job_device(s, s->finished.front());
-            s->finished.pop_front();
+            j->refused_at = s->releases;
             continue;
         }
         if (st || (st = lbpm_batch_add(s->batch, j->ctx))) {

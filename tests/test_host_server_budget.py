@@ -1,7 +1,8 @@
 """The served jobs' memory estimate and budget, with the library's host code on a CUDA
 runtime that counts what is allocated (no GPU): a job never holds more than its
 footprint, at any porosity and in both storages, and the jobs together never more than
-the budget."""
+the budget; one that the device refuses waits, and is not built again before
+another has given its memory back."""
 import ctypes as ct
 
 import numpy as np
@@ -96,4 +97,45 @@ def test_budget_holds(lib, porosity, precision):
             break
     assert [_poll(lib, s, t).state for t in tickets] == [DONE] * 5
     assert most == 2 and lib.fake_peak() - base <= budget
+    assert lib.lbpm_server_destroy(s) == 0
+
+
+@pytest.mark.parametrize("release", [False, True])     # the first job's result: left to the server, or released
+def test_a_refused_job_is_not_built_again_and_again(lib, release):
+    lab = _image(64, 0.3)
+    s = _server(lib)
+    t1 = _submit(lib, s, lab, max_steps=200)[1]
+    t2 = _submit(lib, s, lab, max_steps=20)[1]
+    lib.fake_memory_limit(lib.fake_live() + int(1.5 * _poll(lib, s, t1).footprint))
+    try:
+        refused, uploads = [lib.fake_refused()], []
+        for _ in range(19):                            # 190 of the first job's 200 steps
+            assert _run(lib, s) == (1, 1)
+            refused.append(lib.fake_refused())
+            uploads.append(lib.fake_uploads())
+        assert refused[1] > refused[0] and set(refused[1:]) == {refused[1]}   # tried once
+        assert len(set(np.diff(uploads[1:]))) == 1     # every round's own few
+        assert _run(lib, s) == (0, 1)
+        assert _poll(lib, s, t1).state == DONE
+        if release:
+            assert lib.lbpm_server_release(s, t1) == 0
+        assert _run(lib, s) == (1, 0)
+        assert _run(lib, s) == (0, 0)
+        assert _poll(lib, s, t2).state == DONE
+        assert lib.fake_refused() == refused[1]
+    finally:
+        lib.fake_memory_limit(2 ** 63)
+    assert lib.lbpm_server_destroy(s) == 0
+
+
+def test_a_job_the_device_cannot_hold_alone_fails(lib):
+    lab = _image(64, 0.3)
+    s = _server(lib)
+    t = _submit(lib, s, lab)[1]
+    lib.fake_memory_limit(lib.fake_live() + _poll(lib, s, t).footprint // 2)
+    try:
+        assert _run(lib, s) == (0, 0)
+    finally:
+        lib.fake_memory_limit(2 ** 63)
+    assert _poll(lib, s, t).state == 3                 # failed
     assert lib.lbpm_server_destroy(s) == 0
