@@ -38,6 +38,22 @@ __host__ __device__ __forceinline__ int link_id(int n, const SiteLinks& l) {
     }
 }
 
+// Where direction Q is written to (and opp(Q) read from) by site n at an odd step: row
+// Q at x + xi_Q, with its id, or where there is none row opp(Q) at n itself, as an
+// offset from row Q. Opposite rows are neighbours, so the offset fits 32 bits for any
+// number of sites below 2^31, without a sign where opp(Q) follows Q, with one where it
+// precedes it.
+template <int Q>
+__host__ __device__ __forceinline__ unsigned slot_word(bool has, int id, int n, int pitch) {
+    const unsigned p = static_cast<unsigned>(pitch);
+    return has ? static_cast<unsigned>(id) : static_cast<unsigned>(n) + (opp(Q) > Q ? p : 0u - p);
+}
+template <int Q, class T>
+__host__ __device__ __forceinline__ T* slot_at(T* row, unsigned word) {   // row: row Q
+    if constexpr (opp(Q) > Q) return row + word;
+    else return row + static_cast<int>(word);
+}
+
 #ifdef __CUDACC__
 // Ids of the six face neighbours of site n into nb[1..6], -1 where there is none.
 template <int K>

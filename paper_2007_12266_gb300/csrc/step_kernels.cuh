@@ -397,7 +397,7 @@ __device__ __forceinline__ void phase_sum_thread(const DomainView& d, int t0, in
 // the slot cache.
 struct SlotCache {
     int* slot;      // DENSE: entry of direction 1 of this thread, direction q at slot[(q - 1) * stride]:
-                    // the slot relative to row q (odd steps), the face neighbour's site id (even steps
+                    // slot_word of q (odd steps), the face neighbour's site id (even steps
                     // of the sum form)
     float* ref;     // the density reference of direction q's slot at ref[(q - 1) * stride] (fp16, odd steps)
     int stride;     // threads per block
@@ -455,11 +455,12 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
         else if constexpr (PAR == 1 || (CF != 0 && q < Q7)) return sc.slot[(q - 1) * sc.stride];
         else return __ldg(d.vsite + v + stencil_off(d, q));
     };
-    // slot that direction q is written to (and opp(q) read from) at odd steps, relative to row q
-    auto slot = [&](auto qc) {
+    // slot that direction q is written to (and opp(q) read from) at odd steps
+    auto slot = [&](auto qc, T* base) {
         constexpr int q = decltype(qc)::value;
-        if constexpr (DENSE) return sc.slot[(q - 1) * sc.stride];
-        else return has(qc) ? id(qc) : n + (opp(q) - q) * pitch;
+        T* const row = base + q * static_cast<size_t>(pitch);
+        if constexpr (DENSE) return slot_at<q>(row, static_cast<unsigned>(sc.slot[(q - 1) * sc.stride]));
+        else return slot_at<q>(row, slot_word<q>(has(qc), id(qc), n, pitch));
     };
     // the record and the pitch from here on are values the compiler knows nothing
     // about: ids, slots and row addresses formed before are formed again instead
@@ -486,9 +487,9 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
             constexpr int o = opp(q);                // direction read from it
             if constexpr (DENSE) {
                 const int m = __ldg(d.vsite + v + stencil_off(d, q));
-                sc.slot[(q - 1) * sc.stride] = m >= 0 ? m : n + (o - q) * pitch;
+                sc.slot[(q - 1) * sc.stride] = static_cast<int>(slot_word<q>(m >= 0, m, n, pitch));
             }
-            const float x = S::ld_s(F + q * static_cast<size_t>(pitch) + slot(qc));
+            const float x = S::ld_s(slot(qc, F));
             float r = 0.0f;
             if constexpr (S::kRef) {
                 r = d.drho[has(qc) ? id(qc) : n];
@@ -612,7 +613,7 @@ __device__ __forceinline__ void collide_site(const DomainView& d, int n, const S
     auto store = [&](auto qc, T* base, float x) {
         constexpr int q = decltype(qc)::value;
         if constexpr (PAR == 0) S::st_s(base + opp(q) * static_cast<size_t>(pitch) + n, x);
-        else S::st_s(base + q * static_cast<size_t>(pitch) + slot(qc), x);
+        else S::st_s(slot(qc, base), x);
     };
 
     // The increments of the moving populations sum to minus the rest
