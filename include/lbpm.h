@@ -335,14 +335,16 @@ lbpm_status lbpm_kernel_timing(lbpm_ctx* ctx, double* ms_collide, long long* n_c
  * sum form, each job's steps are a chain of launches of its own, three of them in
  * flight at a time (on streams that start after the earlier work of the batch's
  * stream, which waits for them).
- * Otherwise every timestep of the whole batch is ONE launch of the phase pass and ONE of the fused collide-stream kernel, both
- * over a list of tiles that covers all jobs' sites (or, with the fused launch
- * shape of lbpm_batch_set_launch, one kernel runs every pass of a bundle);
- * bundles of two steps are replayed from a CUDA graph. Inside a call of two or more steps the
- * components travel as per-site sums when every job allows it (see
- * lbpm_set_step_form). Each job's results agree with
+ * Otherwise every timestep of the whole batch is ONE launch of the phase pass and
+ * ONE of the fused collide-stream kernel, both over a list of tiles that covers all
+ * jobs' sites (or, with the fused launch shape of lbpm_batch_set_launch, one kernel
+ * runs every pass of a bundle); bundles of two steps are replayed from a CUDA graph.
+ * Inside a call of two or more steps the components travel as per-site sums when
+ * every job allows it (see lbpm_set_step_form). Each job's results agree with
  * advancing it alone to fp32 rounding (1e-5 relative per distribution after
- * 24 steps in the tests); two batched runs of the same jobs are bit-identical. Jobs keep their own state and every per-job call
+ * 24 steps in the tests; the operations are the same, so they are equal bit for bit
+ * when the calls split the steps alike); two batched runs of the same jobs are
+ * bit-identical. Jobs keep their own state and every per-job call
  * (lbpm_measure, lbpm_read_field, ...) stays valid; a job joins at an even
  * step and must be removed before it is destroyed. After changing a job's
  * parameters, call lbpm_batch_refresh. Work runs on the batch's stream: use
@@ -391,9 +393,9 @@ lbpm_status lbpm_batch_set_launch(lbpm_batch* batch, int threads, int blocks_per
                                   int blocks_per_sm_collide);
 /* Autotuner: times each candidate launch shape over one advance call of
  * steps_per_candidate (even) real steps - all candidates compute identical
- * results - keeps the fastest, and caches it per GPU, precision and size
- * class (log2 of the batch's site count) for the process. Returns the chosen
- * shape. A call's first and last steps carry the populations and the others
+ * results - keeps the fastest, and caches it per GPU, precision, size
+ * class (log2 of the batch's site count) and whether the default shape runs job by
+ * job, for the process. Returns the chosen shape. A call's first and last steps carry the populations and the others
  * the component sums (lbpm_set_step_form), so a count of 16 or more times
  * mostly the middle steps that dominate long runs. */
 lbpm_status lbpm_batch_tune(lbpm_batch* batch, int steps_per_candidate, int* threads, int* blocks_per_sm_phase,

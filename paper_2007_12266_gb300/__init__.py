@@ -414,12 +414,12 @@ class Domain:
 
 
 class Batch:
-    """Several Domains (same GPU, same storage precision) advanced together by
-    one launch per pass over all their sites, or one fused cooperative launch
-    per bundle of steps (lbpm_batch_* ABI).
-    Results agree with advancing each domain alone to fp32 rounding (the
-    batched kernels are compiled separately, so multiply-add contraction may
-    differ); two batched runs of the same jobs are bit-identical."""
+    """Several Domains (same GPU, same storage precision) advanced together: large
+    ones job by job on a few streams, otherwise by one launch per pass over all their
+    sites, or one fused cooperative launch per bundle of steps (lbpm_batch_* ABI).
+    Results are those of advancing each domain alone in the same calls (the collision
+    is written in explicitly rounded operations); two batched runs of the same jobs
+    are bit-identical."""
 
     def __init__(self, device: int = 0, stream=None, use_torch_allocator: bool = True):
         torch = _torch()

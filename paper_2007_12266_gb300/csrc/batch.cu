@@ -78,7 +78,8 @@ __global__ void __launch_bounds__(BT) k_batch_phase_sum(const __grid_constant__ 
 
 // CF: component form of the collision (see collide_site).
 // 32 resident warps per SM where the block size allows (64 registers), as for
-// the single-domain collision.
+// the single-domain collision; the sum form's odd steps spill 4 bytes in FP32, 8 to 24 in
+// FP16, where the single-domain ones, whose views are uniform operands, spill none.
 template <int PAR, class S, int CF, int BT>
 __global__ void __launch_bounds__(BT, 1024 / BT) k_batch_collide(const __grid_constant__ BatchLaunch p) {
     constexpr int kSlots = PAR == 1 ? (Q19 - 1) * BT : (CF != 0 ? (Q7 - 1) * BT : 1);

@@ -383,18 +383,18 @@ lbpm_status batch_advance_sum(lbpm_batch* b, long long nsteps) {
 
 // Whether the batch, with the default launch shape, runs job by job
 // (batch_advance_jobs) instead of one launch per pass over all jobs: in the sum form,
-// and with jobs large enough that two or three fill the GPU. A pass over all jobs leaves nothing of
-// a job in L2 for the next pass, where a job of some 100 k sites keeps its whole state
-// there from step to step; and the chains cover each other's tails, where a pass ends
-// for all jobs at once. Us per step of one launch per pass (256 threads) and job by
-// job: 12 jobs of 221 k sites on average 116 and 92 (fp32), 114 and 89 (fp16); 12 of
-// 446 k 225 and 190, 227 and 182; 32 of 83 k 119 and 97, 116 and 99; but 12 of 49 k
-// 23 and 27, 26 and 28, and 12 of 28 k 15 and 21, where a job's launches are too small
-// to fill the GPU three at a time; and 48 of 71 k, 40 steps a call 147 and 136, lose in
-// calls of 6 to 16 steps (152 and 161, where launching them takes the host as long),
-// which 32 of 83 k do not (calls of 2, 8, 16 steps: 133 and 128, 122 and 118, 120 and
-// 116), so the line lies between. One, two and four streams: 217, 192, 193 against
-// 190 us on the second set.
+// and with jobs large enough that two or three fill the GPU. A pass over all jobs
+// leaves nothing of a job in L2 for the next pass, where a job of some 100 k sites
+// keeps its whole state there from step to step; and the chains cover each other's
+// tails, where a pass ends for all jobs at once. Us per step of one launch per pass
+// (256 threads) and job by job: 12 jobs of 221 k sites on average 122 and 100 (fp32),
+// 122 and 94 (fp16); 12 of 446 k 242 and 209, 242 and 187; 32 of 83 k 123 and 101, 125
+// and 103; but 12 of 49 k 25.7 and 28.2, 26.8 and 28.3, and 12 of 28 k 16.5 and 21.5,
+// where a job's launches are too small to fill the GPU three at a time; and 48 of 71 k,
+// 159 and 142 with 40 steps a call, lose in calls of 8 and 16 steps (164 and 168, 161
+// and 165, where launching them takes the host as long), which 32 of 83 k do not (129
+// and 122, 126 and 119), so the line lies between. One, two and four streams: 237, 211,
+// 215 against 211 us on the second set (fp16 218, 193, 192 against 192).
 // Small jobs among large ones: their launches wait for the large jobs' blocks, some
 // 7 us a step where one of 8 k sites alone takes 3, so the form is taken only while
 // counting each job as at least kByJobMean sites adds no more than a quarter. One

@@ -42,12 +42,12 @@ __global__ void __launch_bounds__(kBlock) k_phase_sum(DomainView d) {
 }
 
 // Launch shape of the collision: 64 registers and 32 resident warps per SM; 56
-// registers and 36 warps spill and are slower. Blocks of 128 threads in FP16, and in
-// FP32 below kSmallSites: there a launch is a few waves out of L2, which smaller
-// blocks end more evenly (256 / 128 threads, us per step: 3.65 / 3.24 at 7 k sites,
-// 10.1 / 9.7 at 247 k, 21.9 / 21.6 at 657 k, 34.2 / 34.1 at 901 k). Above it the step
-// runs from DRAM and 256 threads are as fast or faster (59.8 / 59.8 at 1.6 M, 91.9 /
-// 92.0 at 2.5 M, 135.6 / 136.5 at 3.7 M).
+// registers and 36 warps spill at odd steps, and gain nothing at even ones, where they
+// do not. Blocks of 128 threads in FP16, and in FP32 below kSmallSites: there a launch
+// is a few waves out of L2, which smaller blocks end more evenly (256 / 128 threads, us
+// per step: 3.78 / 3.36 at 7 k sites, 10.8 / 10.3 at 247 k, 24.7 / 24.5 at 657 k, 38.7 /
+// 38.9 at 901 k). Above it the step runs from DRAM and 256 threads are as fast or
+// faster (53.1 / 53.3 at 1.2 M, 66.8 / 67.8 at 1.6 M, 102 / 104 at 2.5 M).
 constexpr long long kSmallSites = 1LL << 20;
 
 // CF: component form of the collision (see collide_site)
